@@ -204,14 +204,16 @@ LBM_API lbm_status lbm_profile_interior(lbm_ctx* ctx, int64_t nlaunches, double 
  * take one memory round trip each: below the size thresholds of plan 0 the
  * edge tiles alone are faster (2 to 5 times up to 256 x 256). */
 typedef struct {
-    int32_t ring_slots; /* rows of the bulk-copy ring, 4..8 (all of them in flight); 0: default (4) */
+    int32_t ring_slots; /* rows of the interior kernel's pipeline in flight or in work, 4..8; 0:
+                           default (4) */
     int32_t chunk_rows; /* rows per CTA, >= 8; 0: one wave of CTAs over the SMs, at least 8 rows
-                           each (default) */
+                           each, of a large body with shorter chunks after it (default) */
     int32_t aligned;    /* 1: the fewest strips of equal width on 32-byte sector boundaries (at
                            most 120 columns; 112 for 16-bit storage); 2: the same on 16-byte
                            boundaries (at most 124 columns; 120 for 16-bit storage);
-                           0: 124-column strips; -1: default (0; in a batch: 0 for 16-bit
-                           storage, 1 otherwise) */
+                           0: 124-column strips; -1: default (0 for 16-bit storage; otherwise
+                           1 in a batch, and for single bodies in 4-byte storage with 16
+                           rows or more per CTA of a wave) */
     int32_t plan;       /* 0: by size (default): a body of fewer than 2^17 nodes (3 x 2^17 in FP64)
                            runs as small tiles of the edge kernel only, a larger one as the
                            interior kernel plus the edge bands (a 3-node band each side of a

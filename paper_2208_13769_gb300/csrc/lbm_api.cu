@@ -234,6 +234,42 @@ void lbm::plan_rects(const lbm_ctx* c, bool edge_only, bool seams_inside, int ir
     }
 }
 
+// Rows per CTA of one wave (`wave` CTAs per strip), at least 8 (shorter tiles
+// of mid-size bodies cut the row pipeline's latency: 512 x 512 FP32 in 13 us
+// a step with 8-row tiles against 15 us with 16).
+static int one_wave_rows(int h, int64_t wave) { return int(std::max<int64_t>((h + wave - 1) / wave, 8)); }
+
+// The chunks of h rows.  One wave of equal chunks leaves SMs idle at the end:
+// they do not run equally fast (at 4096 x 2048 in FP32 they were busy for 72
+// to 100 % of the launch, 85 % on average), so a long wave gets most of the
+// rows, and shorter chunks, taken as SMs become free, the rest.  4-byte
+// storage at 4096 x 2048: 188 us a step in one wave, 163 with 65 % of the rows
+// in it, then chunks of a quarter and an eighth of its rows; 3000 x 1500: 106
+// and 93; at 1536 x 1536 (22 rows per CTA) 55.8 and 56.7, so below 24 rows one
+// wave stays.  16-bit storage waits less for memory and its SMs keep together:
+// 136 us in one wave, 131 with 90 % in it; at 2500 x 1300 60.9 either way.
+// FP64 is bound by its arithmetic (1500 x 1000: 506 us, 507 in levels).
+static ChunkLevels chunk_levels(int fmt, int h, int64_t wave, int tune_chunk, int max_rows) {
+    ChunkLevels L;
+    memset(&L, 0, sizeof(L));
+    const int one = one_wave_rows(h, wave);
+    const bool four = fmt != kFmtF64 && fmt != kFmtF16 && fmt != kFmtBF16;
+    if (tune_chunk > 0 || fmt == kFmtF64 || one < (four ? 24 : 48) || one > max_rows) {
+        L.rows[0] = std::min(tune_chunk > 0 ? tune_chunk : one, std::min(h, max_rows));
+        L.count[0] = (h + L.rows[0] - 1) / L.rows[0];
+        return L;
+    }
+    const int n = (h + one - 1) / one;
+    L.rows[0] = std::max(8, int(int64_t(h) * (four ? 65 : 90) / (100 * int64_t(n))));
+    L.count[0] = n;
+    L.rows[1] = std::max(8, one / 4);
+    L.count[1] = four ? int(int64_t(h) * 22 / (100 * int64_t(L.rows[1]))) : 0;
+    L.rows[2] = std::max(8, one / 8);
+    const int left = h - n * L.rows[0] - L.count[1] * L.rows[1];
+    L.count[2] = std::max(0, (left + L.rows[2] - 1) / L.rows[2]);
+    return L;
+}
+
 // The interior (nodes >= 2 from bounded edges and from a hole's faces, >= 3
 // from periodic seams, or across them) as up to 4 rectangles for the lean
 // kernel; the bands around the body and around the hole as tiles of the
@@ -257,31 +293,54 @@ static cudaError_t build_plan(lbm_ctx* c) {
         const int per_sm = std::max(1, interior_occupancy(c->fmt, c->i_ring));
         const int64_t slots = int64_t(c->num_sms) * per_sm;
         const int64_t all_area = interior_nodes(c);
+        int strips[4];
+        ChunkLevels lev[4];
+        int64_t nitems = 0;
         for (int q = 0; q < c->n_irect; ++q) {
             const int* r = c->irect[q];
+            // the rectangles of a hole share a wave of CTAs by area
             const int h = r[3] - r[2];
-            interior_strips(c->fmt, r[0], r[1], c->tune_aligned > 0 ? c->tune_aligned : 0, &c->i_strip_x0[q], &c->i_strip_w[q],
-                            &c->i_tiles_x[q]);
-            int64_t rows;
-            if (c->tune_chunk > 0) {
-                rows = c->tune_chunk;
-            } else {
-                // one wave of CTAs per launch (strips x chunks <= SMs x
-                // per_sm), the rectangles of a hole sharing it by area, at
-                // least 8 rows each (shorter tiles of mid-size bodies cut the
-                // row pipeline's latency: 512 x 512 FP32 in 17 us with 8-row
-                // tiles against 25 us with 16)
-                const int64_t area = int64_t(r[1] - r[0]) * h;
-                const int64_t share = std::max<int64_t>(1, slots * area / std::max<int64_t>(1, all_area));
-                const int64_t chunks = std::max<int64_t>(1, share / c->i_tiles_x[q]);
-                rows = std::max<int64_t>((h + chunks - 1) / chunks, 8);
-            }
-            rows = std::min<int64_t>(rows, h);
-            c->i_chunk[q] = int(rows);
-            c->i_tiles_y[q] = int((h + rows - 1) / rows);
+            const int64_t share = std::max<int64_t>(1, slots * (int64_t(r[1] - r[0]) * h) / std::max<int64_t>(1, all_area));
+            // strips on sector boundaries for 4-byte storage where a CTA has
+            // rows enough that its neighbours run apart in time (1536 x 1536:
+            // 55.8 us a step, 57.4 without; 2000 x 1500: 72.1 and 75.1)
+            interior_strips(c->fmt, r[0], r[1], 0, &c->i_strip_x0[q], &c->i_strip_w[q], &strips[q]);
+            const bool four = elem_size_storage(c->fmt) == 4;
+            const int aligned = c->tune_aligned >= 0 ? c->tune_aligned
+                                : four && one_wave_rows(h, std::max<int64_t>(1, share / strips[q])) >= 16 ? 1
+                                                                                                         : 0;
+            if (aligned > 0)
+                interior_strips(c->fmt, r[0], r[1], aligned, &c->i_strip_x0[q], &c->i_strip_w[q], &strips[q]);
+            if (q == 0) c->i_aligned = aligned;
+            lev[q] = chunk_levels(c->fmt, h, std::max<int64_t>(1, share / strips[q]), c->tune_chunk,
+                                  interior_max_rows(c->fmt, c->pitch));
+            c->i_chunk[q] = lev[q].rows[0];
+            nitems += interior_items(r, q, strips[q], lev[q], nullptr, 0);
         }
+        if (nitems > INT32_MAX - 1) return cudaErrorInvalidConfiguration;
+        InteriorItem* items = new (std::nothrow) InteriorItem[size_t(nitems)];
+        if (!items) return cudaErrorMemoryAllocation;
+        int64_t at = 0;
+        for (int q = 0; q < c->n_irect; ++q)
+            at += interior_items(c->irect[q], q, strips[q], lev[q], items + at, nitems - at);
+        // the longest first, so that the short ones even out the launch's end
+        std::stable_sort(items, items + nitems, [](const InteriorItem& a, const InteriorItem& b) {
+            return std::abs(a.rows) > std::abs(b.rows);
+        });
+        cudaError_t e = cudaMalloc(&c->ditems, sizeof(InteriorItem) * size_t(nitems));
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(c->ditems, items, sizeof(InteriorItem) * size_t(nitems), cudaMemcpyHostToDevice, c->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);  // items is freed below
+        delete[] items;
+        if (e != cudaSuccess) return e;
+        c->n_items = int(nitems);
     }
     c->has_interior = c->n_irect > 0;  // a hole may leave the bands only
+    for (int q = 0; q < 2 && c->has_interior; ++q) {
+        cudaError_t e = interior_maps(c->fmt, c->scheme == LBM_SCHEME_EXTRAPOLATED, c->f[q], c->a[q], c->s[q], c->pitch,
+                                      c->plane, c->ny, &c->maps[q]);
+        if (e != cudaSuccess) return e;
+    }
     int n = 0;
     for (int b = 0; b < c->nband; ++b)
         n += edge_tiles_of_rect(c->brect[b], 0, nullptr, 0, false, kEdgeThreads, bounded_sides(c, c->brect[b]));
@@ -333,31 +392,21 @@ static cudaError_t build_plan(lbm_ctx* c) {
 
 // The interior launches of one time step, one per interior rectangle
 // (nothing if the body has no interior).
-static cudaError_t launch_interior_part(lbm_ctx* c, const StepParams& p, bool fields) {
+static cudaError_t launch_interior_part(lbm_ctx* c, int parity, bool fields) {
     if (c->n_irect < 1) return cudaSuccess;
     // one launch over every interior rectangle
     InteriorRects R;
     memset(&R, 0, sizeof(R));
-    int64_t total = 0;
-    for (int q = 0; q < 4; ++q) {
-        if (q < c->n_irect) {
-            for (int k = 0; k < 4; ++k) R.g[q].rect[k] = c->irect[q][k];
-            R.g[q].strip_x0 = c->i_strip_x0[q];
-            R.g[q].strip_w = c->i_strip_w[q];
-            R.g[q].chunk_rows = c->i_chunk[q];
-            R.tiles_x[q] = c->i_tiles_x[q];
-            R.first[q] = int32_t(total);
-            total += int64_t(c->i_tiles_x[q]) * c->i_tiles_y[q];
-        } else {
-            R.tiles_x[q] = 1;
-            R.first[q] = INT32_MAX;
-        }
+    for (int q = 0; q < c->n_irect; ++q) {
+        for (int k = 0; k < 4; ++k) R.g[q].rect[k] = c->irect[q][k];
+        R.g[q].strip_x0 = c->i_strip_x0[q];
+        R.g[q].strip_w = c->i_strip_w[q];
     }
-    if (total > INT32_MAX - 1) return cudaErrorInvalidConfiguration;
-    R.total = int32_t(total);
-    StepParams pi = p;
+    R.items = c->ditems;
+    R.total = c->n_items;
+    StepParams pi = make_params(c, parity);
     pi.ring_slots = c->i_ring;
-    return launch_interior(c->fmt, pi, R, c->stream, fields);
+    return launch_interior(c->fmt, pi, R, c->maps[parity], c->stream, fields);
 }
 
 // The edge-band launch of one time step (the whole body without an interior).
@@ -411,7 +460,7 @@ static cudaError_t launch_step_kernels(lbm_ctx* c, int mode, bool fields, int pa
     if (c->n_img > 0) {
         // the interior across a periodic seam: then the band tiles and the
         // seam images in one launch after it (the images copy what it wrote)
-        cudaError_t e = launch_interior_part(c, make_params(c, parity), fields);
+        cudaError_t e = launch_interior_part(c, parity, fields);
         if (e == cudaSuccess) e = launch_band_images_part(c, parity, fields);
         return e;
     }
@@ -419,7 +468,7 @@ static cudaError_t launch_step_kernels(lbm_ctx* c, int mode, bool fields, int pa
     // stream: the small edge CTAs fill the room the interior CTAs leave
     cudaError_t e = cudaEventRecord(c->ev_fork, c->stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(c->side, c->ev_fork, 0);
-    if (e == cudaSuccess) e = launch_interior_part(c, make_params(c, parity), fields);
+    if (e == cudaSuccess) e = launch_interior_part(c, parity, fields);
     if (e == cudaSuccess) e = launch_band_part(c, parity, fields, c->side);
     if (e == cudaSuccess) e = cudaEventRecord(c->ev_join, c->side);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(c->stream, c->ev_join, 0);
@@ -505,6 +554,7 @@ static void free_all(lbm_ctx* c) {
     cudaFree(c->readout);
     cudaFree(c->dparams);
     cudaFree(c->dtiles);
+    cudaFree(c->ditems);
     cudaFree(c->dimg);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
@@ -782,8 +832,7 @@ lbm_status lbm_profile_steps(lbm_ctx* c, int64_t nsteps, double out[4]) {
     if (err == cudaSuccess) err = cudaEventRecord(ev[0], c->stream);
     for (int64_t k = 0; k < nsteps && err == cudaSuccess; ++k) {
         const bool fields = k + 1 == nsteps;  // the last step refreshes the read-out fields
-        const StepParams p = make_params(c, c->parity);
-        err = launch_interior_part(c, p, fields);
+        err = launch_interior_part(c, c->parity, fields);
         if (err == cudaSuccess) err = cudaEventRecord(ev[2 * k + 1], c->stream);
         if (err == cudaSuccess)
             err = c->n_img > 0 ? launch_band_images_part(c, c->parity, fields)
@@ -843,10 +892,10 @@ lbm_status lbm_profile_interior(lbm_ctx* c, int64_t nlaunches, double out[2]) {
         err = cudaMemcpyAsync(save + fb + ab + sb, c->flag, sizeof(int32_t), cudaMemcpyDeviceToDevice, c->stream);
     if (err == cudaSuccess) err = cudaEventCreate(&e0);
     if (err == cudaSuccess) err = cudaEventCreate(&e1);
-    if (err == cudaSuccess) err = launch_interior_part(c, make_params(c, q), false);  // warm
+    if (err == cudaSuccess) err = launch_interior_part(c, q, false);  // warm
     if (err == cudaSuccess) err = cudaEventRecord(e0, c->stream);
     for (int64_t k = 0; k < nlaunches && err == cudaSuccess; ++k)
-        err = launch_interior_part(c, make_params(c, q ^ int((k + 1) & 1)), false);
+        err = launch_interior_part(c, q ^ int((k + 1) & 1), false);
     if (err == cudaSuccess) err = cudaEventRecord(e1, c->stream);
     // restore: the context continues from the saved state
     if (err == cudaSuccess) err = cudaMemcpyAsync(c->f[q], save, fb, cudaMemcpyDeviceToDevice, c->stream);
@@ -886,7 +935,7 @@ lbm_status lbm_get_tuning(const lbm_ctx* c, lbm_tuning* t) {
     if (c->planned && c->has_interior) {
         t->ring_slots = c->i_ring;
         t->chunk_rows = c->i_chunk[0];
-        t->aligned = c->tune_aligned > 0 ? c->tune_aligned : 0;
+        t->aligned = c->i_aligned;
         t->plan = 2;
     } else {
         t->ring_slots = c->tune_ring;

@@ -30,11 +30,6 @@ namespace {
 
 constexpr int kBatchGraphChunk = 64;  // steps per captured graph (even)
 
-// An interior tile of a member while the work list is built.
-struct InteriorWork {
-    int32_t inst, bx, by;
-};
-
 }  // namespace
 
 struct lbm_batch {
@@ -49,7 +44,8 @@ struct lbm_batch {
     int fmt = 0;
     int n_entries = 0;           // parameter-table entries per parity
     StepParams* dtab = nullptr;  // [2][n_entries]: entry q * n_entries + e at parity base_parity ^ q
-    BatchItem* ditems = nullptr;  // interior tiles, longest first
+    InteriorMaps* dmaps = nullptr;     // [2][n_entries]: the entries' tensor maps
+    InteriorItem* ditems = nullptr;  // interior tiles, longest first
     EdgeTile* dtiles = nullptr;   // edge tiles of every member
     ImageTile* dimg = nullptr;    // seam images of the members with a periodic axis
     int32_t** dflagptr = nullptr;  // device: each member's status flag
@@ -87,6 +83,7 @@ void batch_free(lbm_batch* b) {
     for (int k = 0; k < 2; ++k)
         if (b->graph[k]) cudaGraphExecDestroy(b->graph[k]);
     cudaFree(b->dtab);
+    cudaFree(b->dmaps);
     cudaFree(b->ditems);
     cudaFree(b->dtiles);
     cudaFree(b->dimg);
@@ -109,6 +106,7 @@ cudaError_t batch_launch(lbm_batch* b, int q, bool fields) {
     BatchInteriorLaunch I;
     memset(&I, 0, sizeof(I));
     I.params = tab;
+    I.maps = b->dmaps + size_t(q) * size_t(b->n_entries);
     I.items = b->ditems;
     I.fields = fields ? 1 : 0;
     I.nitems = b->n_work;
@@ -296,11 +294,12 @@ lbm_status lbm_batch_create_tuned(lbm_ctx* const* members, int32_t n, void* cuda
     b->chunk_rows = tuning && tuning->chunk_rows
                         ? tuning->chunk_rows
                         : int(std::min<int64_t>(256, std::max<int64_t>(32, all_interior / (int64_t(120) * wave * 8))));
+    cudaError_t e_maps = cudaSuccess;
     std::vector<StepParams> tab;
-    std::vector<InteriorWork> work;
+    std::vector<InteriorMaps> maps;
     std::vector<EdgeTile> tiles;
     std::vector<ImageTile> imgs;
-    std::vector<BatchItem> items;
+    std::vector<InteriorItem> items;
     try {
         // parameter table: one entry per interior rectangle of each member
         // (at least one per member; its edge tiles use the first), for both
@@ -319,7 +318,6 @@ lbm_status lbm_batch_create_tuned(lbm_ctx* const* members, int32_t n, void* cuda
                     for (int k = 0; k < 4; ++k) p.rect[k] = mri.irect[q][k];
                     interior_strips(b->fmt, p.rect[0], p.rect[1], b->aligned, &p.strip_x0, &p.strip_w, &ns);
                 }
-                p.chunk_rows = b->chunk_rows;
                 p.ring_slots = b->ring;
                 ent.push_back(p);
                 strips.push_back(ns);
@@ -327,14 +325,26 @@ lbm_status lbm_batch_create_tuned(lbm_ctx* const* members, int32_t n, void* cuda
                 if (q < mri.n_irect) {
                     const int e = int(ent.size()) - 1;
                     const int h = p.rect[3] - p.rect[2];
-                    const int sy = (h + b->chunk_rows - 1) / b->chunk_rows;
-                    for (int by = 0; by < sy; ++by)
-                        for (int bx = 0; bx < ns; ++bx) work.push_back(InteriorWork{e, bx, by});
+                    ChunkLevels lev;
+                    memset(&lev, 0, sizeof(lev));
+                    lev.rows[0] = std::min(b->chunk_rows, interior_max_rows(b->fmt, c->pitch));
+                    lev.count[0] = (h + lev.rows[0] - 1) / lev.rows[0];
+                    const int64_t cnt = interior_items(mri.irect[q], e, ns, lev, nullptr, 0);
+                    const size_t at = items.size();
+                    items.resize(at + size_t(cnt));
+                    interior_items(mri.irect[q], e, ns, lev, items.data() + at, cnt);
                 }
             }
         }
         b->n_entries = int(ent.size());
         tab.resize(size_t(2) * ent.size());
+        maps.resize(tab.size());
+        for (size_t e = 0; e < maps.size(); ++e) {
+            const size_t k = e % ent.size();
+            const lbm_ctx* c = b->m[size_t(owner[k])];
+            const int par = b->base_parity[size_t(owner[k])] ^ int(e / ent.size());
+            if (e_maps == cudaSuccess) e_maps = interior_maps(b->fmt, false, c->f[par], c->a[par], c->s[par], c->pitch, c->plane, c->ny, &maps[e]);
+        }
         for (size_t e = 0; e < ent.size(); ++e) {
             tab[e] = ent[e];
             // the other parity: the member's parameters of that parity with
@@ -344,7 +354,6 @@ lbm_status lbm_batch_create_tuned(lbm_ctx* const* members, int32_t n, void* cuda
             for (int k = 0; k < 4; ++k) p.rect[k] = ent[e].rect[k];
             p.strip_x0 = ent[e].strip_x0;
             p.strip_w = ent[e].strip_w;
-            p.chunk_rows = ent[e].chunk_rows;
             p.ring_slots = ent[e].ring_slots;
             tab[ent.size() + e] = p;
         }
@@ -374,14 +383,9 @@ lbm_status lbm_batch_create_tuned(lbm_ctx* const* members, int32_t n, void* cuda
         }
         // longest tiles first: the short tiles of small bodies fill the tail
         // of the last wave
-        auto rows_of = [&](const InteriorWork& w) {
-            const StepParams& p = tab[size_t(w.inst)];
-            return std::min(b->chunk_rows, p.rect[3] - p.rect[2]);
-        };
-        std::stable_sort(work.begin(), work.end(),
-                         [&](const InteriorWork& x, const InteriorWork& y) { return rows_of(x) > rows_of(y); });
-        items.reserve(work.size());
-        for (const InteriorWork& w : work) items.push_back(BatchItem{w.inst, w.bx, w.by, 0});
+        std::stable_sort(items.begin(), items.end(), [](const InteriorItem& x, const InteriorItem& y) {
+            return std::abs(x.rows) > std::abs(y.rows);
+        });
     } catch (...) {
         batch_free(b);
         delete b;
@@ -389,10 +393,14 @@ lbm_status lbm_batch_create_tuned(lbm_ctx* const* members, int32_t n, void* cuda
     }
     if (items.size() > 0x7fffffff || tiles.size() > 0x7fffffff || imgs.size() > 0x7fffffff)
         e = cudaErrorInvalidValue;
-    b->n_work = int(work.size());
+    b->n_work = int(items.size());
     b->n_edge = int(tiles.size());
     b->n_img = int(imgs.size());
+    if (e == cudaSuccess) e = e_maps;
     if (e == cudaSuccess) e = cudaMalloc(&b->dtab, sizeof(StepParams) * tab.size());
+    if (e == cudaSuccess) e = cudaMalloc(&b->dmaps, sizeof(InteriorMaps) * maps.size());
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(b->dmaps, maps.data(), sizeof(InteriorMaps) * maps.size(), cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess) e = cudaMalloc(&b->dflagptr, sizeof(int32_t*) * size_t(n));
     if (e == cudaSuccess) e = cudaMalloc(&b->dflagval, sizeof(int32_t) * size_t(n));
     std::vector<int32_t*> flagptr;
@@ -404,12 +412,12 @@ lbm_status lbm_batch_create_tuned(lbm_ctx* const* members, int32_t n, void* cuda
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(b->dflagptr, flagptr.data(), sizeof(int32_t*) * size_t(n), cudaMemcpyHostToDevice,
                             b->stream);
-    if (e == cudaSuccess && !items.empty()) e = cudaMalloc(&b->ditems, sizeof(BatchItem) * items.size());
+    if (e == cudaSuccess && !items.empty()) e = cudaMalloc(&b->ditems, sizeof(InteriorItem) * items.size());
     if (e == cudaSuccess && !tiles.empty()) e = cudaMalloc(&b->dtiles, sizeof(EdgeTile) * tiles.size());
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(b->dtab, tab.data(), sizeof(StepParams) * tab.size(), cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess && !items.empty())
-        e = cudaMemcpyAsync(b->ditems, items.data(), sizeof(BatchItem) * items.size(), cudaMemcpyHostToDevice,
+        e = cudaMemcpyAsync(b->ditems, items.data(), sizeof(InteriorItem) * items.size(), cudaMemcpyHostToDevice,
                             b->stream);
     if (e == cudaSuccess && !tiles.empty())
         e = cudaMemcpyAsync(b->dtiles, tiles.data(), sizeof(EdgeTile) * tiles.size(), cudaMemcpyHostToDevice,

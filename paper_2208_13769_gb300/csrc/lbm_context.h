@@ -95,14 +95,17 @@ struct lbm_ctx {
     bool has_interior = false;  // n_irect > 0
     int n_irect = 0;
     int irect[4][4];
-    int i_tiles_x[4], i_tiles_y[4], i_chunk[4], i_strip_x0[4], i_strip_w[4];
-    int i_ring = 0;
+    int i_chunk[4], i_strip_x0[4], i_strip_w[4];
+    lbm::InteriorItem* ditems = nullptr;  // device: the interior tiles
+    int n_items = 0;
+    int i_ring = 0, i_aligned = 0;
     // requested decomposition of the interior launch (lbm_set_tuning); 0 / -1:
     // the library's defaults
     int tune_ring = 0, tune_chunk = 0, tune_aligned = -1, tune_plan = 0;
     int nband = 0;
     int brect[12][4];
     lbm::StepParams* dparams = nullptr;  // device: make_params(parity 0), make_params(parity 1)
+    lbm::InteriorMaps maps[2];                // the interior's copies, source state of parity 0 and 1
     lbm::EdgeTile* dtiles = nullptr;     // device: tiles of the edge bands
     int n_etiles = 0;
     // with a hole, the initialisation runs over the bands' tiles and tiles of

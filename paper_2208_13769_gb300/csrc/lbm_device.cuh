@@ -199,6 +199,18 @@ enum CarryLayout : int {
     kCarryPair16 = 2  // FP32 high word, 16-bit low word: x.hi, x.lo16, y.hi, y.lo16 (1.5 planes each)
 };
 
+// The element `o` elements after base, by a 32-bit byte offset (the caller
+// keeps o * sizeof(T) below 2^32).
+template <class T>
+__device__ __forceinline__ T* elem(T* base, uint32_t o) {
+    using B = typename std::conditional<std::is_const<T>::value, const char, char>::type;
+    return reinterpret_cast<T*>(reinterpret_cast<B*>(base) + o * uint32_t(sizeof(T)));
+}
+template <class T>
+__device__ __forceinline__ T* elem(T* base, int64_t o) {
+    return base + o;
+}
+
 template <class T>
 struct UPlain {  // u kept in T itself (FP64 or FP32)
     static constexpr int layout = kCarryOne;
@@ -207,6 +219,7 @@ struct UPlain {  // u kept in T itself (FP64 or FP32)
     template <class P>
     struct ViewT {
         P* w;
+        __device__ __forceinline__ ViewT shifted(int64_t o) const { return ViewT{w + o}; }
     };
     using View = ViewT<T>;
     using CView = ViewT<const T>;
@@ -219,14 +232,17 @@ struct UPlain {  // u kept in T itself (FP64 or FP32)
     // the stored words as loaded (decode() turns them into the value; a
     // prefetch keeps them raw so that nothing waits for the load early)
     using Raw = UPlain;
-    __device__ __forceinline__ static Raw load_raw(const CView& c, int64_t o, int64_t) { return UPlain{c.w[o]}; }
+    template <class O>
+    __device__ __forceinline__ static Raw load_raw(const CView& c, O o) {
+        return UPlain{*elem(c.w, o)};
+    }
     __device__ __forceinline__ static UPlain decode(const Raw& r, const StepParams&) { return r; }
-    __device__ __forceinline__ static UPlain load(const CView& c, int64_t o, int64_t plane, const StepParams& p) {
-        return decode(load_raw(c, o, plane), p);
+    __device__ __forceinline__ static UPlain load(const CView& c, int64_t o, const StepParams& p) {
+        return decode(load_raw(c, o), p);
     }
     template <class Put>
     __device__ __forceinline__ static void store(const UPlain& x, const UPlain& y, const View& cx, const View& cy,
-                                                 int64_t, const StepParams&, Put&& put) {
+                                                 const StepParams&, Put&& put) {
         put(cx.w, x.v);
         put(cy.w, y.v);
     }
@@ -257,9 +273,12 @@ struct UPair {
     struct View {
         float* hi;
         Lo* lo;
+        __device__ __forceinline__ View shifted(int64_t o) const { return View{hi + o, lo + o}; }
     };
     struct CView {
         const float* hi;
+        const Lo* lo;
+        __device__ __forceinline__ CView shifted(int64_t o) const { return CView{hi + o, lo + o}; }
     };
     // first float of component comp: after 2 planes of floats per component,
     // or after 1.5 (a multiple of 32 floats: plane is a multiple of 64)
@@ -271,14 +290,16 @@ struct UPair {
         return View{h, reinterpret_cast<Lo*>(h + plane)};
     }
     __device__ __forceinline__ static CView cview(const void* a, int comp, int64_t plane) {
-        return CView{static_cast<const float*>(a) + comp_offset(comp, plane)};
+        const float* h = static_cast<const float*>(a) + comp_offset(comp, plane);
+        return CView{h, reinterpret_cast<const Lo*>(h + plane)};
     }
     struct Raw {
         float hi;
         Lo lo;
     };
-    __device__ __forceinline__ static Raw load_raw(const CView& c, int64_t o, int64_t plane) {
-        return Raw{c.hi[o], reinterpret_cast<const Lo*>(c.hi + plane)[o]};
+    template <class O>
+    __device__ __forceinline__ static Raw load_raw(const CView& c, O o) {
+        return Raw{*elem(c.hi, o), *elem(c.lo, o)};
     }
     __device__ __forceinline__ static UPair decode(const Raw& r, const StepParams& p) {
         if constexpr (LO16)
@@ -286,8 +307,8 @@ struct UPair {
         else
             return UPair{r.hi, r.lo};
     }
-    __device__ __forceinline__ static UPair load(const CView& c, int64_t o, int64_t plane, const StepParams& p) {
-        return decode(load_raw(c, o, plane), p);
+    __device__ __forceinline__ static UPair load(const CView& c, int64_t o, const StepParams& p) {
+        return decode(load_raw(c, o), p);
     }
     __device__ __forceinline__ Lo lo_word(const StepParams& p) const {
         if constexpr (LO16) {
@@ -304,7 +325,7 @@ struct UPair {
     // interior kernel than component by component)
     template <class Put>
     __device__ __forceinline__ static void store(const UPair& x, const UPair& y, const View& cx, const View& cy,
-                                                 int64_t, const StepParams& p, Put&& put) {
+                                                 const StepParams& p, Put&& put) {
         put(cx.hi, x.hi);
         put(cy.hi, y.hi);
         put(cx.lo, x.lo_word(p));

@@ -228,8 +228,8 @@ __device__ __forceinline__ void edge_tile_body(const EdgeTile& tile, const StepP
 #pragma unroll
         for (int i = 0; i < 9; ++i)
             f[i] = Codec<TS, TC>::ld(fsrc[int64_t(i) * plane + o - ex(i) - int64_t(ey(i)) * pitch], i, p);
-        const UT A0 = UT::load(as0, o, plane, p);
-        const UT A1 = UT::load(as1, o, plane, p);
+        const UT A0 = UT::load(as0, o, p);
+        const UT A1 = UT::load(as1, o, p);
         if (inC) {
             so0 = s_src[o];
             so1 = s_src[o + plane];
@@ -426,7 +426,7 @@ __device__ __forceinline__ void edge_tile_body(const EdgeTile& tile, const StepP
         const TC f0 = MODE == 1 ? TC(2) * ka0 : fo0, f1 = MODE == 1 ? TC(2) * ka1 : fo1;
         const UT A0 = xj ? ux.add(TC(4) * ka0 - f0).renorm() : ux.add(du0 + ka0).renorm();
         const UT A1 = xj ? uy.add(TC(4) * ka1 - f1).renorm() : uy.add(du1 + ka1).renorm();
-        UT::store(A0, A1, ad0, ad1, plane, p, put);
+        UT::store(A0, A1, ad0, ad1, p, put);
         if (xj) {
             const TC d0 = MODE == 1 ? ka0 : so0, d1 = MODE == 1 ? ka1 : so1;
             put(s_dst, ka0);

@@ -23,9 +23,8 @@
 //   stage C, row a - 2 : 1S = rho0 b + Div Q, corrected j and u, equilibrium,
 //                        BGK collision with He forcing, store       (W cols)
 // The 9 population segments of each row arrive in a ring of shared-memory
-// slots by bulk asynchronous copies (cp.async.bulk, one mbarrier per slot)
-// issued D rows ahead of stage A; the two carries are prefetched one row
-// ahead into registers.  u* and Q live in 3-row rolling buffers.
+// slots by tiled asynchronous copies (cp.async.bulk.tensor, one mbarrier per
+// slot), the two carries with them.  u* and Q live in rolling buffers.
 //
 // Lattice units inside the kernels: m = sum_i e_i f_i, Pf = sum_i e_i e_i f_i,
 // s = (dt / c) 1S, jh = j / c, so that the equilibrium (Sec. 5) reads
@@ -39,7 +38,9 @@
 // so that u*_n+1 = A + dX/(2 rho0) m  and  jh_n+1 = m + s_(n+1 or n) / 2.
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "lbm_device.cuh"
@@ -51,100 +52,134 @@ namespace lbm {
 namespace {
 
 // Shared memory of the interior tile: a 128-byte header (the ring's
-// mbarriers, at most 8), the u* rows [3][2][NT] and the Q rows [3][4][NT],
-// then the ring.
+// mbarriers, at most 8, and the abort word), the u* rows [3][2][NT] and the
+// rows of (Q11, Q21) [2][2][NT], then the ring.
 constexpr int kSmemHeader = 128;
+constexpr int kSmemAbort = 64;
 template <class UT, class TC, int NT>
 __host__ __device__ constexpr size_t interior_smem_fixed() {
-    return (kSmemHeader + sizeof(UT) * 6 * NT + sizeof(TC) * 12 * NT + 127) / 128 * 128;
+    return (kSmemHeader + sizeof(UT) * 6 * NT + sizeof(TC) * 4 * NT + 127) / 128 * 128;
 }
 
-// Elements of one bulk-copied row segment: a strip of W <= NT - 4 output
-// columns reads columns x0 - 3 .. x0 + W + 2 from a 16-byte aligned start
-// (up to 16 / sizeof(TS) - 1 columns before x0 - 3), in a whole number of
-// 16-byte units.
-template <class TS, int NT>
-__host__ __device__ constexpr int seg_elems() {
-    return sizeof(TS) == 2 ? NT + 16 : NT + 8;
-}
+// One slot of the ring: everything an iteration of the row loop reads from
+// global memory, as boxes of tensor maps (InteriorMaps) that each start on a
+// 128-byte boundary.
+//  - The populations of stage A's row a.  A pulled row takes plane i from
+//    row a - ey(i): planes {0, 1}, {5, 6} and {7, 8} come in pairs from one
+//    row each, and {2, 3, 4} from rows a - 1, a, a + 1 as one box, by a map
+//    whose plane stride is one plane plus one row.  The issuing thread runs
+//    7 copies with constant coordinates instead of 9 and 6 loads whose 64-bit
+//    addresses it and the others compute each row (483 warp instructions per
+//    32 nodes against 545 at 4096 x 2048 in FP32).
+//  - The u-carry of row a, and the source carry of the row that stage C of
+//    the iteration before works on (three rows behind a).  Loaded into
+//    registers one row ahead they arrived late (issuing the source's half a
+//    row later still cost 10 us of 173); here every slot is in flight.
+// A segment of the populations spans columns x0 - 3 .. x0 + W + 2 of a strip
+// of W <= NT - 4 output columns from a 16-byte aligned start (up to 16 /
+// sizeof(TS) - 1 columns before x0 - 3), one of a carry columns x0 - 2 ..
+// x0 + W + 1.
+template <class TS, class TC, class UT, int NT, bool XJ>
+struct RingSlot {
+    static constexpr int up(int bytes) { return (bytes + 127) / 128 * 128; }
+    static constexpr int ES = int(sizeof(TS)), CS = int(sizeof(TC));
+    static constexpr int SEG = sizeof(TS) == 2 ? NT + 16 : NT + 8;  // elements of a population segment
+    static constexpr int SEGC = NT + 16 / CS;                       // words of a carry segment
+    static constexpr int SEGL = NT + 8;                             // 16-bit low words of the u-carry
+    static constexpr int NA = UT::layout == kCarryPair ? 4 : 2;     // u-carry planes in words of TC
+    static constexpr int NL = UT::layout == kCarryPair16 ? 2 : 0;   // and in 16-bit words
+    static constexpr int NS = XJ ? 4 : 2;                           // source-carry planes
+    static constexpr int F2 = up(2 * SEG * ES), F3 = up(3 * SEG * ES);
+    static constexpr int A = 3 * F2 + F3, L = A + up(NA * SEGC * CS), S = L + up(NL * SEGL * 2);
+    static constexpr int BYTES = S + up(NS * SEGC * CS);
+    static constexpr int TX_S = NS * SEGC * CS;  // bytes copied: the source carry, and all
+    static constexpr int TX = 9 * SEG * ES + NA * SEGC * CS + NL * SEGL * 2 + TX_S;
+    // byte offset of plane i's segment
+    __host__ __device__ static constexpr int plane(int i) {
+        return i < 2 ? i * SEG * ES
+                     : (i < 5 ? 3 * F2 + (i - 2) * SEG * ES
+                              : (i < 7 ? F2 + (i - 5) * SEG * ES : 2 * F2 + (i - 7) * SEG * ES));
+    }
+    // the population of direction i pulled by the column whose element of
+    // plane 0 is at f
+    __device__ __forceinline__ static TS pop(const unsigned char* f, int i) {
+        return *reinterpret_cast<const TS*>(f + plane(i) - ex(i) * ES);
+    }
+    // the stored u-carry of component c: ec, el the column's words in a carry
+    // segment and in a segment of low words
+    __device__ __forceinline__ static typename UT::Raw carry(const unsigned char* slot, int c, int ec, int el) {
+        const TC* a = reinterpret_cast<const TC*>(slot + A) + ec;
+        if constexpr (UT::layout == kCarryOne)
+            return typename UT::Raw{a[c * SEGC]};
+        else if constexpr (UT::layout == kCarryPair)
+            return typename UT::Raw{a[2 * c * SEGC], a[(2 * c + 1) * SEGC]};
+        else
+            return typename UT::Raw{a[c * SEGC], reinterpret_cast<const __half*>(slot + L)[c * SEGL + el]};
+    }
+    // plane c of the source carry
+    __device__ __forceinline__ static TC source(const unsigned char* slot, int c, int ec) {
+        return reinterpret_cast<const TC*>(slot + S)[c * SEGC + ec];
+    }
+};
 
-template <class TS, int NT>
-__host__ __device__ constexpr size_t interior_row_bytes() {
-    return size_t(9) * seg_elems<TS, NT>() * sizeof(TS);
-}
+// Slots of the ring for lbm_tuning.ring_slots rows in flight or in work (the
+// row in work sits in registers).
+__host__ __device__ constexpr int ring_depth(int ring_slots) { return ring_slots - 1; }
 
 }  // namespace
 
 // One tile (column strip bx, row chunk by of the rectangle tg) of one body,
 // the only tile of its CTA.  Returns false if a wait gave up or a copy was
-// refused (reported in p.flag).  UNROLL3: the row loop unrolled by 3 (the
-// row buffers' indices fixed at compile time, the kept populations changing
-// roles instead of moving: fewer instructions, more registers; faster for
-// the formats whose registers allow it).  KEEP: stage C takes the populations of
-// its row from registers that stage A filled two rows earlier (18 more
-// registers, 9 fewer shared-memory loads per node) instead of the ring, and
-// the ring keeps every slot in flight.  XJ: the extrapolated scheme, whose
-// carries are E = u(t) + F (the u* of stage A, in the u-carry planes),
-// D = ku jh(t) and F = ku (3 jh(t) - jh(t - dt)) (in the source planes);
-// else u* is A + ku m and the source planes hold the last source.
-template <class TS, class TC, class UT, int NT, bool KEEP, bool XJ, bool UNROLL3, bool REV>
-__device__ __forceinline__ bool interior_tile(const StepParams& p, const TileGeom& tg, int bx, int by,
-                                              double* fields) {
+// refused (reported in p.flag).  Stage C takes the populations of its row
+// from registers that stage A filled two rows earlier, and Q12, Q22 of the
+// rows above and below from registers of stage B.  UNROLL3: the row loop
+// unrolled by 3 (the row buffers' indices fixed at compile time, the kept
+// values changing roles instead of moving: fewer instructions, more
+// registers; faster for the formats whose registers allow it).  XJ: the
+// extrapolated scheme, whose carries are E = u(t) + F (the u* of stage A, in
+// the u-carry planes), D = ku jh(t) and F = ku (3 jh(t) - jh(t - dt)) (in
+// the source planes); else u* is A + ku m and the source planes hold the
+// last source.
+template <class TS, class TC, class UT, int NT, bool XJ, bool UNROLL3, bool REV>
+__device__ __forceinline__ bool interior_tile(const StepParams& p, const InteriorMaps* maps, const TileGeom& tg,
+                                              int bx, int y_begin, int y_end, double* fields) {
+    using Slot = RingSlot<TS, TC, UT, NT, XJ>;
     const int W = tg.strip_w;
-    constexpr int SEG = seg_elems<TS, NT>();
-    constexpr int ROW_BYTES = int(interior_row_bytes<TS, NT>());
-    static_assert(ROW_BYTES % 16 == 0, "row size");
     constexpr int ALIGN_COLS = 16 / int(sizeof(TS));
 
     extern __shared__ __align__(128) unsigned char smem[];
-    const int R = p.ring_slots;  // row slots: lookahead + 3
+    const int R = ring_depth(p.ring_slots);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem);
-    UT* su = reinterpret_cast<UT*>(smem + kSmemHeader);                          // [3][2][NT]
-    TC* sq = reinterpret_cast<TC*>(smem + kSmemHeader + sizeof(UT) * 6 * NT);   // [3][4][NT]
+    // a wait gave up: read after the row's first barrier, so every thread
+    // takes the same decision
+    volatile int* s_abort = reinterpret_cast<volatile int*>(smem + kSmemAbort);
+    UT* su = reinterpret_cast<UT*>(smem + kSmemHeader);                        // u*: [3][2][NT]
+    TC* sq = reinterpret_cast<TC*>(smem + kSmemHeader + sizeof(UT) * 6 * NT);  // Q11, Q21: [2][2][NT]
     unsigned char* ring = smem + interior_smem_fixed<UT, TC, NT>();
-    // a wait gave up: set in stage A, read after the row's first barrier, so
-    // every thread takes the same decision
-    __shared__ int s_abort;
 
     LatConsts<TC> k;
     k.load(p);
     const int64_t pitch = p.pitch, plane = p.plane;
     const int t = threadIdx.x;
-    const int rx0 = tg.rect[0], rx1 = tg.rect[1], ry0 = tg.rect[2], ry1 = tg.rect[3];
+    const int rx0 = tg.rect[0], rx1 = tg.rect[1];
     // strip bx of the strip grid, clipped to the rectangle
     const int x0 = tg.strip_x0 + bx * W;
     const int x_lo = max(rx0, x0), x_hi = min(rx1, x0 + W);
-    const int chunk_rows = tg.chunk_rows;
-    if (x_lo >= x_hi || by * chunk_rows >= ry1 - ry0) return true;
-    int y_begin = ry0 + by * chunk_rows;
-    if (y_begin > ry1 - chunk_rows) y_begin = ry1 - chunk_rows > ry0 ? ry1 - chunk_rows : ry0;
-    const int y_end = min(ry1, y_begin + chunk_rows);
+    if (x_lo >= x_hi || y_begin >= y_end) return true;
     // first column of the row segments: 16-byte aligned, inside the plane
     int seg0 = x0 - 3;
     seg0 = (seg0 >= 0 ? seg0 : seg0 - (ALIGN_COLS - 1)) / ALIGN_COLS * ALIGN_COLS;
     if (seg0 < -kPadCols) seg0 = -kPadCols;
-    // elements of each segment this tile copies: through column x_hi + 2 (the
-    // last one stage A pulls from), in whole 16-byte units (a strip narrower
-    // than the widest copies less)
-    const int seg_n = min(SEG, (x_hi + 3 - seg0 + ALIGN_COLS - 1) / ALIGN_COLS * ALIGN_COLS);
-
-    const TS* __restrict__ fsrc = static_cast<const TS*>(p.f_src);
-    TS* __restrict__ fdst = static_cast<TS*>(p.f_dst);
-    // the u-carry's planes, per component
-    const void* __restrict__ a_src = p.a_src;
-    void* __restrict__ a_dst = p.a_dst;
-    const typename UT::CView as0 = UT::cview(a_src, 0, plane), as1 = UT::cview(a_src, 1, plane);
-    const typename UT::View ad0 = UT::view(a_dst, 0, plane), ad1 = UT::view(a_dst, 1, plane);
-    const TC* __restrict__ s_src = static_cast<const TC*>(p.s_src);
-    TC* __restrict__ s_dst = static_cast<TC*>(p.s_dst);
 
     const int gx = x0 - 2 + t;  // this thread's column
     const bool colA = gx >= x_lo - 2 && gx < x_hi + 2;
     const bool colB = gx >= x_lo - 1 && gx < x_hi + 1;
     const bool colC = gx >= x_lo && gx < x_hi;
     const int tm = t > 0 ? t - 1 : t, tp = t < NT - 1 ? t + 1 : t;
-    const int e_own = gx - seg0;
-    const int64_t col_off = int64_t(gx) + kPadCols;
+    // where the segments start in a plane's row, and this column in them
+    const int xf = seg0 + kPadCols, xc = (x0 - 2 + kPadCols) & ~(16 / int(sizeof(TC)) - 1),
+              xl = (x0 - 2 + kPadCols) & ~7;
+    const int e_own = (gx - seg0) * int(sizeof(TS)), ec = gx + kPadCols - xc, el = gx + kPadCols - xl;
 
     // the row walk: down the chunk, or up it (REV), so that two chunks
     // sharing a boundary read its halo rows at the same time (both at their
@@ -154,139 +189,114 @@ __device__ __forceinline__ bool interior_tile(const StepParams& p, const TileGeo
     constexpr int sg = REV ? -1 : 1;
     const int a0 = rev ? y_end + 1 : y_begin - 2;
     const int niter = (y_end - y_begin) + 4;
-    const TS* src_seg = fsrc + int64_t(kPadRows) * pitch + seg0 + kPadCols;  // row 0 of plane 0
 
-    // bulk copies of row a into ring slot s (thread 0); the 16-byte alignment
-    // of every address is checked before anything is issued.  A refused row
-    // is reported in p.flag (bit 8) and never arrives, so the wait for it
-    // gives up and the tile stops at the next barrier
-    auto issue_row = [&](int a, int s) -> bool {
-        unsigned char* base = ring + size_t(s) * ROW_BYTES;
-        const uintptr_t acc = reinterpret_cast<uintptr_t>(base) | reinterpret_cast<uintptr_t>(src_seg) |
-                              uintptr_t(pitch * int64_t(sizeof(TS))) | uintptr_t(plane * int64_t(sizeof(TS))) |
-                              uintptr_t(seg_n * int(sizeof(TS)));
-        if (acc & 15) {
-            atomicOr(p.flag, 8);
-            return false;
-        }
-        mbar_expect_tx(&bars[s], uint32_t(9 * seg_n * int(sizeof(TS))));
-        TS* dst = reinterpret_cast<TS*>(base);
-#pragma unroll
-        for (int i = 0; i < 9; ++i)
-            bulk_load(dst + i * SEG, src_seg + i * plane + int64_t(a - ey(i)) * pitch, uint32_t(seg_n * sizeof(TS)),
-                      &bars[s]);
-        return true;
+    // the copies of iteration j into ring slot s (thread 0): iteration niter
+    // holds only the source carry of the last one's stage C.  A copy's first
+    // column must start on a 16-byte boundary: a tile whose does not (none
+    // does, by seg0) is refused before anything is issued, in p.flag (bit 8)
+    const uint32_t ring_at = smem_addr(ring), bars_at = smem_addr(bars);
+    auto issue_row = [&](int j, int s) {
+        const uint32_t dst = ring_at + uint32_t(s * Slot::BYTES), bar = bars_at + uint32_t(s * 8);
+        const int r = a0 + sg * j + kPadRows;
+        const bool all = j < niter;
+        mbar_expect_tx(&bars[s], uint32_t(all ? Slot::TX : Slot::TX_S));
+        tensor_load(dst + Slot::S, &maps->s, xc, r - 3 * sg, 0, bar);
+        if (!all) return;
+        tensor_load(dst, &maps->f, xf, r, 0, bar);                      // planes 0, 1 of row a
+        tensor_load(dst + Slot::F2, &maps->f, xf, r - 1, 5, bar);       // 5, 6 of row a - 1
+        tensor_load(dst + 2 * Slot::F2, &maps->f, xf, r + 1, 7, bar);   // 7, 8 of row a + 1
+        tensor_load(dst + 3 * Slot::F2, &maps->f3, xf, r - 1, 0, bar);  // 2, 3, 4 of rows a - 1, a, a + 1
+        tensor_load(dst + Slot::A, &maps->a, xc, r, 0, bar);
+        if (Slot::NL > 0) tensor_load(dst + Slot::L, &maps->lo, xl, r, 0, bar);
     };
+    if (xf < 0 || xf % ALIGN_COLS != 0) {  // uniform over the CTA
+        if (t == 0) atomicOr(p.flag, 8);
+        return false;
+    }
 
+    uint32_t phase = 0, issued = 0;
     if (t == 0) {
-        s_abort = 0;
+        *s_abort = 0;
         for (int s = 0; s < R; ++s) mbar_init(&bars[s], 1);
         fence_mbar_init();
     }
     __syncthreads();
-    // rows of lookahead: with KEEP a row's ring slot is free once stage A has
-    // read it (stage C takes the row's populations from registers), so every
-    // slot holds a row in flight; otherwise it also serves stage C two rows
-    // later
-    const int D = KEEP ? R : R - 3;
-    uint32_t phase = 0, issued = 0;
     if (t == 0) {
         fence_proxy_async();  // the CTA's earlier shared-memory accesses precede the copies into the ring
-    }
-    if (t == 0)
-        for (int j = 0; j < D && j < niter; ++j) {
-            if (issue_row(a0 + sg * j, j)) issued |= 1u << j;
+        for (int j = 0; j < R && j <= niter; ++j) {
+            issue_row(j, j);
+            issued |= 1u << j;
         }
+    }
 
-    // 32-bit element offsets inside a plane (a plane holds fewer than 2^31
-    // elements, checked at context creation) and per-plane base pointers,
-    // which are the same for every thread of the CTA
-    const int32_t pitch32 = int32_t(pitch);
-    int32_t off_a = (a0 + kPadRows) * pitch32 + int32_t(col_off);  // row a of stage A, this column
-    const int32_t dpitch = rev ? -pitch32 : pitch32;                   // to the walk's next row
+    // Addresses: a base per plane, the same for every thread of the CTA
+    // (column gx of thread 0 in the tile's lowest row), and a 32-bit offset
+    // from it, which advances by a row (the host keeps a tile's rows few
+    // enough for its byte offsets to fit, interior_max_rows).
+    const uint32_t pitch32 = uint32_t(pitch);
+    uint32_t off_a = uint32_t(t) + (rev ? uint32_t(niter - 1) * pitch32 : 0u);  // row a of stage A, this column
+    const uint32_t dpitch = rev ? 0u - pitch32 : pitch32;                       // to the walk's next row
+    const int64_t base = int64_t(y_begin - 2 + kPadRows) * pitch + (x0 - 2) + kPadCols;
     TS* fd[9];
 #pragma unroll
-    for (int i = 0; i < 9; ++i) fd[i] = fdst + int64_t(i) * plane;
-    const TC* ss1 = s_src + plane;
-    TC* sd1 = s_dst + plane;
-    // the extrapolated scheme's F (planes 2, 3)
-    const TC* sf0 = s_src + 2 * plane;
-    const TC* sf1 = s_src + 3 * plane;
-
-    // carries prefetched one row ahead
-    typename UT::Raw an0, an1;  // as stored: decoded where stage A uses them
-    TC sn_old0 = TC(0), sn_old1 = TC(0), f_old0 = TC(0), f_old1 = TC(0);
-    if (colA) {
-        an0 = UT::load_raw(as0, off_a, plane);
-        an1 = UT::load_raw(as1, off_a, plane);
-    }
-
+    for (int i = 0; i < 9; ++i) fd[i] = static_cast<TS*>(p.f_dst) + int64_t(i) * plane + base;
+    const typename UT::View ad0 = UT::view(p.a_dst, 0, plane).shifted(base);
+    const typename UT::View ad1 = UT::view(p.a_dst, 1, plane).shifted(base);
+    TC* sd[Slot::NS];
+#pragma unroll
+    for (int i = 0; i < Slot::NS; ++i) sd[i] = static_cast<TC*>(p.s_dst) + int64_t(i) * plane + base;
     bool bad = false;
+    // waits for slot s's copies
+    auto wait_slot = [&](int s) {
+        if (!mbar_wait(&bars[s], (phase >> s) & 1u)) *s_abort = 1;
+        phase ^= 1u << s;
+        issued &= ~(1u << s);
+    };
+    wait_slot(0);
     int ra = 0;
-    // the populations of this column as stage A pulled them (KEEP): stage C
-    // of row a - 2 takes them from here, not the ring
-    TC F0[9], F1[9], F2[9];
+    // rows kept in registers for stage C two iterations later: the
+    // populations of this column as stage A pulled them, Q12 and Q22 of stage B
+    TC F0[9], F1[9], F2[9], V0[2], V1[2], V2[2];
 #pragma unroll
     for (int i = 0; i < 9; ++i) F0[i] = F1[i] = F2[i] = TC(0);
-    // One row of the pipeline.  sa = q mod 3 selects the u* and Q row buffers
-    // (a compile-time constant when the loop is unrolled by 3); gcur receives
-    // stage A's populations of row a, fp2 holds those of row a - 2.  Returns
-    // false when the tile gives up.
-    auto row = [&](int q, auto sa, TC* gcur, const TC* fp2) -> bool {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) V0[i] = V1[i] = V2[i] = TC(0);
+    // One row of the pipeline.  sa = q mod 3 selects the u* row buffer (a
+    // compile-time constant when the loop is unrolled by 3); gcur receives
+    // stage A's populations of row a and vcur stage B's Q12, Q22 of row
+    // a - sg, fp2 and vp2 hold those of two iterations ago.  Returns false
+    // when the tile gives up.
+    auto row = [&](int q, auto sa, TC* gcur, const TC* fp2, TC* vcur, const TC* vp2) -> bool {
         const int sA = sa;                    // slot of row a
         const int sB = sA == 0 ? 2 : sA - 1;  // slot of row a - 1
-        const int sC = sA == 2 ? 0 : sA + 1;  // slot of row a - 2 (and Q of row a - 3 in sq[sA])
-        const int rc = ra >= 2 ? ra - 2 : ra - 2 + R;
-        const TC so0 = sn_old0, so1 = sn_old1;  // source carry (XJ: D) of stage C's row
-        const TC fo0 = f_old0, fo1 = f_old1;    // XJ: F of stage C's row
+        const int sC = sA == 2 ? 0 : sA + 1;  // slot of row a - 2
+        const int rn = ra + 1 == R ? 0 : ra + 1;  // ring slot of the next iteration
 
         // ---------------- stage A: row a
-        if (!s_abort && !mbar_wait(&bars[ra], (phase >> ra) & 1u)) s_abort = 1;
-        phase ^= 1u << ra;
-        issued &= ~(1u << ra);
         if (colA) {
-            const TS* pf = reinterpret_cast<const TS*>(ring + size_t(ra) * ROW_BYTES) + e_own;
-            TC g[9];
+            const unsigned char* slot = ring + ra * Slot::BYTES;
+            const unsigned char* pf = slot + e_own;
 #pragma unroll
-            for (int i = 1; i < 9; ++i) g[i] = Codec<TS, TC>::ld(pf[i * SEG - ex(i)], i, p);
-            if (KEEP) {
-                gcur[0] = Codec<TS, TC>::ld(pf[0], 0, p);
-#pragma unroll
-                for (int i = 1; i < 9; ++i) gcur[i] = g[i];
-            }
+            for (int i = 0; i < 9; ++i) gcur[i] = Codec<TS, TC>::ld(Slot::pop(pf, i), i, p);
+            const UT A0 = UT::decode(Slot::carry(slot, 0, ec, el), p), A1 = UT::decode(Slot::carry(slot, 1, ec, el), p);
             if (XJ) {  // u* = u(t) + ku (3 jh(t) - jh(t - dt)) = E
-                su[(sA * 2) * NT + t] = UT::decode(an0, p);
-                su[(sA * 2 + 1) * NT + t] = UT::decode(an1, p);
+                su[(sA * 2) * NT + t] = A0;
+                su[(sA * 2 + 1) * NT + t] = A1;
             } else {
+                const TC* g = gcur;
                 const TC m0 = (g[1] - g[3]) + (g[5] - g[6]) + (g[8] - g[7]);
                 const TC m1 = (g[2] - g[4]) + (g[5] - g[8]) + (g[6] - g[7]);
-                su[(sA * 2) * NT + t] = UT::decode(an0, p).add(k.ku * m0);
-                su[(sA * 2 + 1) * NT + t] = UT::decode(an1, p).add(k.ku * m1);
-            }
-            if (q + 1 < niter) {
-                an0 = UT::load_raw(as0, off_a + dpitch, plane);
-                an1 = UT::load_raw(as1, off_a + dpitch, plane);
+                su[(sA * 2) * NT + t] = A0.add(k.ku * m0);
+                su[(sA * 2 + 1) * NT + t] = A1.add(k.ku * m1);
             }
         }
         __syncthreads();
-        if (s_abort) return false;
-        if (t == 0 && q + D < niter) {
-            // KEEP: the slot row a just left; else the slot of row a - 3, done
-            const int rn = KEEP ? ra : (ra + D < R ? ra + D : ra + D - R);
+        if (*s_abort) return false;
+        if (t == 0 && q + R <= niter) {  // into the slot that stage A has just read
             fence_proxy_async();
-            if (issue_row(a0 + sg * (q + D), rn)) issued |= 1u << rn;
+            issue_row(q + R, ra);
+            issued |= 1u << ra;
         }
-        // source carry of the next iteration's stage C row (a - 1)
-        if (colC && q >= 3 && q + 1 < niter) {
-            const int32_t o = off_a - dpitch;  // row a - sg
-            sn_old0 = s_src[o];
-            sn_old1 = ss1[o];
-            if (XJ) {
-                f_old0 = sf0[o];
-                f_old1 = sf1[o];
-            }
-        }
-
         // ---------------- stage B: row a - sg
         if (colB && q >= 2) {
             const UT* r0 = su + (sB * 2) * NT;
@@ -300,33 +310,33 @@ __device__ __forceinline__ bool interior_tile(const StepParams& p, const TileGeo
             TC q11, q12, q21, q22;
             const TC J = stress_remainder<TC>(h11, h12, h21, h22, k.lam, k.mu, q11, q12, q21, q22);
             bad |= !(J > TC(0));  // also catches a non-finite displacement gradient
-            TC* qr = sq + (sB * 4) * NT;
+            TC* qr = sq + (q & 1) * 2 * NT;
             qr[t] = q11;
-            qr[NT + t] = q12;
-            qr[2 * NT + t] = q21;
-            qr[3 * NT + t] = q22;
+            qr[NT + t] = q21;
+            vcur[0] = q12;
+            vcur[1] = q22;
         }
+        wait_slot(rn);
         __syncthreads();
 
         // ---------------- stage C: row a - 2 sg
         if (colC && q >= 4) {
             const int gy = a0 + sg * (q - 2);
-            const TC* qc = sq + (sC * 4) * NT;                 // Q of row a - 2 sg
-            const TC* qm = sq + ((rev ? sB : sA) * 4) * NT;    // Q of the row below it
-            const TC* qp = sq + ((rev ? sA : sB) * 4) * NT;    // Q of the row above it
-            // s = (dt / c) 1S, 1S = rho0 b + Div(P + Pbar)   (Eq. source1)
-            const TC sn0 = k.sb0 + k.sq_scale * ((qc[tp] - qc[tm]) + (qp[NT + t] - qm[NT + t]));
-            const TC sn1 = k.sb1 + k.sq_scale * ((qc[2 * NT + tp] - qc[2 * NT + tm]) + (qp[3 * NT + t] - qm[3 * NT + t]));
-
-            const TS* pf = reinterpret_cast<const TS*>(ring + size_t(rc) * ROW_BYTES) + e_own;
-            TC f[9];
-            if (KEEP) {
-#pragma unroll
-                for (int i = 0; i < 9; ++i) f[i] = fp2[i];
-            } else {
-#pragma unroll
-                for (int i = 0; i < 9; ++i) f[i] = Codec<TS, TC>::ld(pf[i * SEG - ex(i)], i, p);
+            const unsigned char* next = ring + rn * Slot::BYTES;
+            const TC so0 = Slot::source(next, 0, ec), so1 = Slot::source(next, 1, ec);  // source carry (XJ: D)
+            TC fo0 = TC(0), fo1 = TC(0);                                                // XJ: F
+            if (XJ) {
+                fo0 = Slot::source(next, Slot::NS - 2, ec);
+                fo1 = Slot::source(next, Slot::NS - 1, ec);
             }
+            const TC* qc = sq + ((q & 1) ^ 1) * 2 * NT;                      // Q11, Q21 of row a - 2 sg
+            const TC* qm = rev ? vcur : vp2;                                 // Q12, Q22 of the row below it
+            const TC* qp = rev ? vp2 : vcur;                                 // and of the row above it
+            // s = (dt / c) 1S, 1S = rho0 b + Div(P + Pbar)   (Eq. source1)
+            const TC sn0 = k.sb0 + k.sq_scale * ((qc[tp] - qc[tm]) + (qp[0] - qm[0]));
+            const TC sn1 = k.sb1 + k.sq_scale * ((qc[NT + tp] - qc[NT + tm]) + (qp[1] - qm[1]));
+
+            const TC* f = fp2;
             const TC r = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8];
             const TC m0 = (f[1] - f[3]) + (f[5] - f[6]) + (f[8] - f[7]);
             const TC m1 = (f[2] - f[4]) + (f[5] - f[8]) + (f[6] - f[7]);
@@ -374,9 +384,9 @@ __device__ __forceinline__ bool interior_tile(const StepParams& p, const TileGeo
             fc[7] = k.one_m_omega * f[7] + (ap - bp);
             fc[6] = k.one_m_omega * f[6] + (am + bm);
             fc[8] = k.one_m_omega * f[8] + (am - bm);
-            const int32_t o = off_a - 2 * dpitch;  // row a - 2 sg = gy
+            const uint32_t o = off_a - 2 * dpitch;  // row a - 2 sg = gy
 #pragma unroll
-            for (int i = 0; i < 9; ++i) fd[i][o] = Codec<TS, TC>::st(fc[i], i, p);
+            for (int i = 0; i < 9; ++i) *elem(fd[i], o) = Codec<TS, TC>::st(fc[i], i, p);
 
             // carries: A' = u + ku (jh + s/2), u = u* + du;  s' = s
             // (XJ: E' = u + ku (3 jh - jh(t)) = E - F + 4 D', D' = ku jh,
@@ -386,16 +396,13 @@ __device__ __forceinline__ bool interior_tile(const StepParams& p, const TileGeo
             const TC ka1 = XJ ? k.ku * j1 : k.ku * (j1 + TC(0.5) * sn1);
             const UT A0 = XJ ? ux.add(TC(4) * ka0 - fo0).renorm() : ux.add(du0 + ka0).renorm();
             const UT A1 = XJ ? uy.add(TC(4) * ka1 - fo1).renorm() : uy.add(du1 + ka1).renorm();
-            auto put = [o](auto* base, auto v) { base[o] = v; };
-            UT::store(A0, A1, ad0, ad1, plane, p, put);
+            auto put = [o](auto* at, auto v) { *elem(at, o) = v; };
+            UT::store(A0, A1, ad0, ad1, p, put);
+            *elem(sd[0], o) = XJ ? ka0 : sn0;
+            *elem(sd[1], o) = XJ ? ka1 : sn1;
             if (XJ) {
-                s_dst[o] = ka0;
-                sd1[o] = ka1;
-                s_dst[o + 2 * plane] = TC(3) * ka0 - so0;
-                s_dst[o + 3 * plane] = TC(3) * ka1 - so1;
-            } else {
-                s_dst[o] = sn0;
-                sd1[o] = sn1;
+                *elem(sd[Slot::NS - 2], o) = TC(3) * ka0 - so0;
+                *elem(sd[Slot::NS - 1], o) = TC(3) * ka1 - so1;
             }
             if (fields != nullptr) {
                 const int64_t fo = int64_t(gy) * p.nx + gx;
@@ -408,36 +415,39 @@ __device__ __forceinline__ bool interior_tile(const StepParams& p, const TileGeo
                 if (!(isfinite(j0) && isfinite(j1))) bad = true;  // in the arithmetic type: no FP64 work
             }
         }
-        ra = ra + 1 == R ? 0 : ra + 1;
+        ra = rn;
         off_a += dpitch;
         return true;
     };
     if (UNROLL3) {
-        // the kept populations change roles instead of moving: row q in
-        // F[q mod 3], row q - 2 in F[(q + 1) mod 3]
+        // the kept values change roles instead of moving: iteration q's in
+        // F[q mod 3], those of q - 2 in F[(q + 1) mod 3]
         for (int q = 0; q < niter;) {
-            if (!row(q, std::integral_constant<int, 0>(), F0, F1) || ++q >= niter) break;
-            if (!row(q, std::integral_constant<int, 1>(), F1, F2) || ++q >= niter) break;
-            if (!row(q, std::integral_constant<int, 2>(), F2, F0) || ++q >= niter) break;
+            if (!row(q, std::integral_constant<int, 0>(), F0, F1, V0, V1) || ++q >= niter) break;
+            if (!row(q, std::integral_constant<int, 1>(), F1, F2, V1, V2) || ++q >= niter) break;
+            if (!row(q, std::integral_constant<int, 2>(), F2, F0, V2, V0) || ++q >= niter) break;
         }
     } else {
-        // F1 and F2 keep rows a - 1 and a - 2, rotated after each row
+        // F1 and F2 keep the values of the last two iterations, moved after each
         int sa = 0;
         for (int q = 0; q < niter; ++q) {
-            TC gcur[9];
-            if (!row(q, sa, gcur, F2)) break;
-            if (KEEP) {
+            TC gcur[9], vcur[2];
+            if (!row(q, sa, gcur, F2, vcur, V2)) break;
 #pragma unroll
-                for (int i = 0; i < 9; ++i) {
-                    F2[i] = F1[i];
-                    F1[i] = gcur[i];
-                }
+            for (int i = 0; i < 9; ++i) {
+                F2[i] = F1[i];
+                F1[i] = gcur[i];
+            }
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                V2[i] = V1[i];
+                V1[i] = vcur[i];
             }
             sa = sa == 2 ? 0 : sa + 1;
         }
     }
     if (bad) atomicOr(p.flag, 1);
-    if (s_abort) {
+    if (*s_abort) {
         if (t == 0) {
             atomicOr(p.flag, 4);
             for (int s = 0; s < R; ++s)
@@ -463,37 +473,17 @@ __host__ __device__ constexpr bool alternate_walk() {
 
 template <class TS, class TC, class UT, int NT, int MINB, bool XJ, bool UNROLL3>
 __global__ void __launch_bounds__(NT, MINB)
-    interior_step_kernel(const __grid_constant__ StepParams p, const __grid_constant__ InteriorRects R) {
-    constexpr bool ALT = alternate_walk<UNROLL3>();
-    const int b = int(blockIdx.x);
-    const int q = (b >= R.first[1]) + (b >= R.first[2]) + (b >= R.first[3]);
-    TileGeom tg;
-    int tx, f;
+    interior_step_kernel(const __grid_constant__ StepParams p, const __grid_constant__ InteriorRects R,
+                         const __grid_constant__ InteriorMaps maps) {
+    const InteriorItem it = R.items[blockIdx.x];
     // the rectangle by constant indices (no indexed reads of the parameters)
-    if (q == 0) {
-        tg = R.g[0];
-        tx = R.tiles_x[0];
-        f = R.first[0];
-    } else if (q == 1) {
-        tg = R.g[1];
-        tx = R.tiles_x[1];
-        f = R.first[1];
-    } else if (q == 2) {
-        tg = R.g[2];
-        tx = R.tiles_x[2];
-        f = R.first[2];
-    } else {
-        tg = R.g[3];
-        tx = R.tiles_x[3];
-        f = R.first[3];
-    }
-    const int local = b - f;
-    // chunks of odd index walk up (see interior_tile)
-    const int bx = local % tx, by = local / tx;
-    if (ALT && (by & 1))
-        interior_tile<TS, TC, UT, NT, true, XJ, UNROLL3, true>(p, tg, bx, by, p.fields);
+    const TileGeom tg = it.inst == 0 ? R.g[0] : (it.inst == 1 ? R.g[1] : (it.inst == 2 ? R.g[2] : R.g[3]));
+    const bool up = it.rows < 0;
+    const int y1 = it.y0 + (up ? -it.rows : it.rows);
+    if (alternate_walk<UNROLL3>() && up)
+        interior_tile<TS, TC, UT, NT, XJ, UNROLL3, true>(p, &maps, tg, it.strip, it.y0, y1, p.fields);
     else
-        interior_tile<TS, TC, UT, NT, true, XJ, UNROLL3, false>(p, tg, bx, by, p.fields);
+        interior_tile<TS, TC, UT, NT, XJ, UNROLL3, false>(p, &maps, tg, it.strip, it.y0, y1, p.fields);
 }
 
 // The interiors of a batch of bodies for one time step: one CTA per interior
@@ -505,34 +495,41 @@ __global__ void __launch_bounds__(NT, MINB)
 template <class TS, class TC, class UT, int NT, int MINB, bool UNROLL3>
 __global__ void __launch_bounds__(NT, MINB) batch_interior_kernel(const __grid_constant__ BatchInteriorLaunch L) {
     __shared__ __align__(16) StepParams sp;
-    const BatchItem it = L.items[blockIdx.x];
+    const InteriorItem it = L.items[blockIdx.x];
     {
         const int4* src = reinterpret_cast<const int4*>(L.params + it.inst);
         int4* dst = reinterpret_cast<int4*>(&sp);
         for (int q = int(threadIdx.x); q < int(sizeof(StepParams) / 16); q += NT) dst[q] = src[q];
     }
+    const InteriorMaps* maps = L.maps + it.inst;
+    if (threadIdx.x == 0) {  // the thread that issues the copies
+        acquire_tensor_map(&maps->f);
+        acquire_tensor_map(&maps->f3);
+        acquire_tensor_map(&maps->a);
+        if (UT::layout == kCarryPair16) acquire_tensor_map(&maps->lo);
+        acquire_tensor_map(&maps->s);
+    }
     __syncthreads();
-    const TileGeom tg = {{sp.rect[0], sp.rect[1], sp.rect[2], sp.rect[3]}, sp.strip_x0, sp.strip_w, sp.chunk_rows};
-    // chunks of odd index walk up their rows, as in the single-body kernel:
-    // the list holds a member's chunks row by row, so the chunks on either
-    // side of a boundary run at about the same time and read its halo rows
-    // together (not the unrolled row loop, whose second copy would cost more
-    // than the L2 hits give)
-    if (!UNROLL3 && (it.b & 1))
-        interior_tile<TS, TC, UT, NT, true, false, UNROLL3, true>(sp, tg, it.a, it.b, L.fields ? sp.fields : nullptr);
+    const TileGeom tg = {{sp.rect[0], sp.rect[1], sp.rect[2], sp.rect[3]}, sp.strip_x0, sp.strip_w};
+    const bool up = it.rows < 0;
+    const int y1 = it.y0 + (up ? -it.rows : it.rows);
+    double* fields = L.fields ? sp.fields : nullptr;
+    if (alternate_walk<UNROLL3>() && up)
+        interior_tile<TS, TC, UT, NT, false, UNROLL3, true>(sp, maps, tg, it.strip, it.y0, y1, fields);
     else
-        interior_tile<TS, TC, UT, NT, true, false, UNROLL3, false>(sp, tg, it.a, it.b, L.fields ? sp.fields : nullptr);
+        interior_tile<TS, TC, UT, NT, false, UNROLL3, false>(sp, maps, tg, it.strip, it.y0, y1, fields);
 }
 
-template <class TS, class TC, class UT, int NT>
+template <class TS, class TC, class UT, int NT, bool XJ>
 size_t interior_smem_bytes(int ring_slots) {
-    return interior_smem_fixed<UT, TC, NT>() + interior_row_bytes<TS, NT>() * size_t(ring_slots);
+    return interior_smem_fixed<UT, TC, NT>() +
+           size_t(RingSlot<TS, TC, UT, NT, XJ>::BYTES) * size_t(ring_depth(ring_slots));
 }
 
 template <class TS, class TC, class UT, int NT, int MINB, bool UNROLL3, bool XJ>
-cudaError_t launch_interior_x(const StepParams& p, const InteriorRects& R, cudaStream_t s) {
+cudaError_t launch_interior_x(const StepParams& p, const InteriorRects& R, const InteriorMaps& maps, cudaStream_t s) {
     auto kern = interior_step_kernel<TS, TC, UT, NT, MINB, XJ, UNROLL3>;
-    const size_t sm = interior_smem_bytes<TS, TC, UT, NT>(p.ring_slots);
+    const size_t sm = interior_smem_bytes<TS, TC, UT, NT, XJ>(p.ring_slots);
     static size_t configured = 0;
     if (sm > configured) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
@@ -540,22 +537,22 @@ cudaError_t launch_interior_x(const StepParams& p, const InteriorRects& R, cudaS
         configured = sm;
     }
     if (R.total <= 0) return cudaSuccess;
-    kern<<<R.total, NT, sm, s>>>(p, R);
+    kern<<<R.total, NT, sm, s>>>(p, R, maps);
     return cudaGetLastError();
 }
 
 // (the extrapolated scheme's variant keeps the rotating loop: its extra
 // carries leave no registers for the unrolled one)
 template <class TS, class TC, class UT, int NT, int MINB, bool UNROLL3>
-cudaError_t launch_interior_t(const StepParams& p, const InteriorRects& R, cudaStream_t s) {
-    return p.scheme == 2 ? launch_interior_x<TS, TC, UT, NT, MINB, false, true>(p, R, s)
-                         : launch_interior_x<TS, TC, UT, NT, MINB, UNROLL3, false>(p, R, s);
+cudaError_t launch_interior_t(const StepParams& p, const InteriorRects& R, const InteriorMaps& maps, cudaStream_t s) {
+    return p.scheme == 2 ? launch_interior_x<TS, TC, UT, NT, MINB, false, true>(p, R, maps, s)
+                         : launch_interior_x<TS, TC, UT, NT, MINB, UNROLL3, false>(p, R, maps, s);
 }
 
 template <class TS, class TC, class UT, int NT, int MINB, bool UNROLL3>
 cudaError_t launch_batch_interior_t(const BatchInteriorLaunch& L, int ring_slots, cudaStream_t s, int* resident) {
     auto kern = batch_interior_kernel<TS, TC, UT, NT, MINB, UNROLL3>;
-    const size_t sm = interior_smem_bytes<TS, TC, UT, NT>(ring_slots);
+    const size_t sm = interior_smem_bytes<TS, TC, UT, NT, false>(ring_slots);
     static size_t configured = 0;
     if (sm > configured) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
@@ -581,7 +578,7 @@ cudaError_t launch_batch_interior(int fmt, const BatchInteriorLaunch& L, int rin
     constexpr int NT = kInteriorThreads;
     switch (fmt) {
         case kFmtF64:
-            return launch_batch_interior_t<double, double, UPlain<double>, NT, 2, false>(L, ring_slots, s, resident);
+            return launch_batch_interior_t<double, double, UPlain<double>, NT, 3, false>(L, ring_slots, s, resident);
         case kFmtF32:
             return launch_batch_interior_t<float, float, UPlain<float>, NT, 6, true>(L, ring_slots, s, resident);
         case kFmtF32C:
@@ -624,7 +621,7 @@ void interior_strips(int fmt, int rx0, int rx1, int aligned, int* strip_x0, int*
 template <class TS, class TC, class UT, int NT, int MINB, bool UNROLL3>
 int interior_occupancy_t(int ring_slots) {
     auto kern = interior_step_kernel<TS, TC, UT, NT, MINB, false, UNROLL3>;
-    const size_t sm = interior_smem_bytes<TS, TC, UT, NT>(ring_slots);
+    const size_t sm = interior_smem_bytes<TS, TC, UT, NT, false>(ring_slots);
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm)) != cudaSuccess) return 0;
     int n = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, NT, sm) != cudaSuccess) return 0;
@@ -638,36 +635,119 @@ int interior_occupancy_t(int ring_slots) {
 // rotating loop (the unrolled one was 3 % slower at 80 registers).
 int interior_occupancy(int fmt, int ring_slots) {
     switch (fmt) {
-        case kFmtF64: return interior_occupancy_t<double, double, UPlain<double>, 128, 2, false>(ring_slots);
+        case kFmtF64: return interior_occupancy_t<double, double, UPlain<double>, 128, 3, false>(ring_slots);
         case kFmtF32: return interior_occupancy_t<float, float, UPlain<float>, 128, 7, true>(ring_slots);
-        case kFmtF32C: return interior_occupancy_t<float, float, UComp, 128, 4, false>(ring_slots);
-        case kFmtF32H: return interior_occupancy_t<float, float, UCompH, 128, 4, false>(ring_slots);
-        case kFmtF16: return interior_occupancy_t<__half, float, UComp, 128, 4, true>(ring_slots);
-        default: return interior_occupancy_t<__nv_bfloat16, float, UComp, 128, 4, true>(ring_slots);
+        case kFmtF32C: return interior_occupancy_t<float, float, UComp, 128, 6, false>(ring_slots);
+        case kFmtF32H: return interior_occupancy_t<float, float, UCompH, 128, 6, false>(ring_slots);
+        case kFmtF16: return interior_occupancy_t<__half, float, UComp, 128, 6, true>(ring_slots);
+        default: return interior_occupancy_t<__nv_bfloat16, float, UComp, 128, 6, true>(ring_slots);
     }
 }
 
-size_t interior_smem(int fmt, int ring_slots) {
+int64_t interior_items(const int rect[4], int inst, int strips, const ChunkLevels& L, InteriorItem* out, int64_t cap) {
+    int64_t n = 0;
+    int y = rect[2], by = 0;
+    for (int k = 0; k < 4; ++k)
+        for (int c = 0; c < L.count[k] && y < rect[3]; ++c, ++by) {
+            const int rows = std::min(L.rows[k], rect[3] - y);
+            for (int bx = 0; bx < strips; ++bx, ++n)
+                if (out && n < cap) out[n] = InteriorItem{inst, bx, y, (by & 1) ? -rows : rows};
+            y += rows;
+        }
+    return n;
+}
+
+namespace {
+
+using EncodeTiled = decltype(&cuTensorMapEncodeTiled);
+
+// The driver's encoder (the library does not link against libcuda).
+EncodeTiled encode_tiled() {
+    static const EncodeTiled fn = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess)
+            f = nullptr;
+        return reinterpret_cast<EncodeTiled>(f);
+    }();
+    return fn;
+}
+
+// The maps of one state with the boxes of RingSlot.
+template <class TS, class TC, class UT, bool XJ>
+bool encode_maps(const void* f, const void* a, const void* src, int64_t pitch, int64_t plane, int ny,
+                 InteriorMaps* out) {
+    using Slot = RingSlot<TS, TC, UT, kInteriorThreads, XJ>;
+    const EncodeTiled enc = encode_tiled();
+    if (!enc) return false;
+    const int64_t rows = int64_t(ny) + 2 * kPadRows;
+    // words of `es` bytes from `at` on; planes `step` bytes apart, of `nrows` rows; boxes of w columns of np planes
+    auto make = [&](CUtensorMap* m, const void* at, int es, int64_t nrows, int nplanes, int64_t step, int w, int np) {
+        const CUtensorMapDataType type = es == 8   ? CU_TENSOR_MAP_DATA_TYPE_UINT64
+                                         : es == 4 ? CU_TENSOR_MAP_DATA_TYPE_UINT32
+                                                   : CU_TENSOR_MAP_DATA_TYPE_UINT16;
+        const cuuint64_t dim[3] = {cuuint64_t(pitch), cuuint64_t(nrows), cuuint64_t(nplanes)};
+        const cuuint64_t stride[2] = {cuuint64_t(pitch * es), cuuint64_t(step)};
+        const cuuint32_t box[3] = {cuuint32_t(w), 1, cuuint32_t(np)}, unit[3] = {1, 1, 1};
+        return enc(m, type, 3, const_cast<void*>(at), dim, stride, box, unit, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                   CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    };
+    const char* f0 = static_cast<const char*>(f);
+    const char* a0 = static_cast<const char*>(a);
+    constexpr int ES = Slot::ES, CS = Slot::CS;
+    constexpr bool half_lo = UT::layout == kCarryPair16;  // components 1.5 planes apart, low words after the high ones
+    return make(&out->f, f0, ES, rows, 9, plane * ES, Slot::SEG, 2) &&
+           make(&out->f3, f0 + 2 * plane * ES, ES, rows - 2, 3, (plane + pitch) * ES, Slot::SEG, 3) &&
+           make(&out->a, a0, CS, rows, Slot::NA, half_lo ? plane * 6 : plane * CS, Slot::SEGC, Slot::NA) &&
+           (!half_lo || make(&out->lo, a0 + plane * 4, 2, rows, 2, plane * 6, Slot::SEGL, 2)) &&
+           make(&out->s, src, CS, rows, Slot::NS, plane * CS, Slot::SEGC, Slot::NS);
+}
+
+}  // namespace
+
+cudaError_t interior_maps(int fmt, bool xj, const void* f, const void* a, const void* s, int64_t pitch, int64_t plane,
+                          int ny, InteriorMaps* out) {
+    memset(out, 0, sizeof(*out));
+    auto enc = [&](auto ts, auto tc, auto ut) {
+        using TS = decltype(ts);
+        using TC = decltype(tc);
+        using UT = decltype(ut);
+        return xj ? encode_maps<TS, TC, UT, true>(f, a, s, pitch, plane, ny, out)
+                  : encode_maps<TS, TC, UT, false>(f, a, s, pitch, plane, ny, out);
+    };
+    bool ok = false;
     switch (fmt) {
-        case kFmtF64: return interior_smem_bytes<double, double, UPlain<double>, 128>(ring_slots);
-        case kFmtF32: return interior_smem_bytes<float, float, UPlain<float>, 128>(ring_slots);
-        case kFmtF32C: return interior_smem_bytes<float, float, UComp, 128>(ring_slots);
-        case kFmtF32H: return interior_smem_bytes<float, float, UCompH, 128>(ring_slots);
-        case kFmtF16: return interior_smem_bytes<__half, float, UComp, 128>(ring_slots);
-        default: return interior_smem_bytes<__nv_bfloat16, float, UComp, 128>(ring_slots);
+        case kFmtF64: ok = enc(double(), double(), UPlain<double>()); break;
+        case kFmtF32: ok = enc(float(), float(), UPlain<float>()); break;
+        case kFmtF32C: ok = enc(float(), float(), UComp()); break;
+        case kFmtF32H: ok = enc(float(), float(), UCompH()); break;
+        case kFmtF16: ok = enc(__half(), float(), UComp()); break;
+        case kFmtBF16: ok = enc(__nv_bfloat16(), float(), UComp()); break;
     }
+    return ok ? cudaSuccess : cudaErrorNotSupported;
 }
 
-cudaError_t launch_interior(int fmt, const StepParams& p0, const InteriorRects& R, cudaStream_t s, bool fields) {
+// The widest element of a plane that interior_tile addresses by a 32-bit
+// byte offset is 8 bytes in FP64 and 4 otherwise; a tile spans its rows and
+// 4 more.
+int interior_max_rows(int fmt, int64_t pitch) {
+    const int64_t row = pitch * (fmt == kFmtF64 ? 8 : 4);
+    return int(std::max<int64_t>(8, (int64_t(1) << 32) / row - 8));
+}
+
+cudaError_t launch_interior(int fmt, const StepParams& p0, const InteriorRects& R, const InteriorMaps& maps, cudaStream_t s,
+                            bool fields) {
     StepParams p = p0;
     if (!fields) p.fields = nullptr;
     switch (fmt) {
-        case kFmtF64: return launch_interior_t<double, double, UPlain<double>, 128, 2, false>(p, R, s);
-        case kFmtF32: return launch_interior_t<float, float, UPlain<float>, 128, 7, true>(p, R, s);
-        case kFmtF32C: return launch_interior_t<float, float, UComp, 128, 4, false>(p, R, s);
-        case kFmtF32H: return launch_interior_t<float, float, UCompH, 128, 4, false>(p, R, s);
-        case kFmtF16: return launch_interior_t<__half, float, UComp, 128, 4, true>(p, R, s);
-        case kFmtBF16: return launch_interior_t<__nv_bfloat16, float, UComp, 128, 4, true>(p, R, s);
+        case kFmtF64: return launch_interior_t<double, double, UPlain<double>, 128, 3, false>(p, R, maps, s);
+        case kFmtF32: return launch_interior_t<float, float, UPlain<float>, 128, 7, true>(p, R, maps, s);
+        case kFmtF32C: return launch_interior_t<float, float, UComp, 128, 6, false>(p, R, maps, s);
+        case kFmtF32H: return launch_interior_t<float, float, UCompH, 128, 6, false>(p, R, maps, s);
+        case kFmtF16: return launch_interior_t<__half, float, UComp, 128, 6, true>(p, R, maps, s);
+        case kFmtBF16: return launch_interior_t<__nv_bfloat16, float, UComp, 128, 6, true>(p, R, maps, s);
     }
     return cudaErrorInvalidValue;
 }

@@ -1,6 +1,7 @@
 // lbm_kernels.h -- host-visible launchers of the solver's kernels.
 #pragma once
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include "lbm_params.h"
@@ -22,13 +23,12 @@ enum Format : int {
 // lie at least 2 nodes from bounded edges and 3 from periodic seams.  A CTA
 // has kInteriorThreads threads, one per column of its strip and halo.
 constexpr int kInteriorThreads = 128;
-size_t interior_smem(int fmt, int ring_slots);
 // CTAs of the interior kernel resident per SM with this ring (0 on error);
 // also sets the kernel's dynamic shared-memory limit, so call it before any
 // stream capture.
 int interior_occupancy(int fmt, int ring_slots);
-// Rows of the interior kernel's bulk-copy ring by default, all of them in
-// flight (4 measured fastest for single bodies and for batches).
+// Rows of the interior kernel's ring by default, those in flight and the one
+// in work (4 measured fastest for single bodies and for batches).
 constexpr int kInteriorRing = 4;
 constexpr int kBatchRing = 4;
 // The strip grid of the interior kernel over columns [rx0, rx1): origin of
@@ -40,34 +40,61 @@ constexpr int kBatchRing = 4;
 void interior_strips(int fmt, int rx0, int rx1, int aligned, int* strip_x0, int* strip_w, int* nstrips);
 
 // One interior rectangle of a launch: its nodes [rect[0], rect[1]) x
-// [rect[2], rect[3]), the strip grid over its columns and the rows per tile.
+// [rect[2], rect[3]) and the strip grid over its columns.
 struct TileGeom {
     int32_t rect[4];
-    int32_t strip_x0, strip_w, chunk_rows;
+    int32_t strip_x0, strip_w;
+};
+// An interior tile, the work of one CTA: strip `strip` and rows [y0, y0 +
+// rows) of rectangle `inst` (of the launch's rectangles, or in a batch entry
+// `inst` of the parameter table); rows negative: those -rows rows, walked
+// upwards.
+struct InteriorItem {
+    int32_t inst, strip, y0, rows;
 };
 // The rectangles of one interior launch (a hole splits the interior into up
-// to 4): tiles_x x tiles_y tiles each, numbered from first[q] in one 1-D grid
-// of total tiles.
+// to 4), and its tiles.
 struct InteriorRects {
     TileGeom g[4];
-    int32_t tiles_x[4];
-    int32_t first[4];  // unused entries: INT32_MAX
+    const InteriorItem* items;  // device list, one per CTA
     int32_t total;
 };
+// The rows of a rectangle as chunks: count[k] chunks of rows[k] rows for each
+// level k in turn (the last of them clipped to the rectangle).
+struct ChunkLevels {
+    int32_t rows[4], count[4];
+};
+// The tiles of a rectangle: its chunks in order, every strip of each; chunks
+// of odd index walk up, so that the chunks on either side of a boundary read
+// its halo rows together.  Returns their number (written to out, at most cap,
+// when out is not NULL).
+int64_t interior_items(const int rect[4], int inst, int strips, const ChunkLevels& L, InteriorItem* out, int64_t cap);
+
+// The tensor maps, over (x, row, plane), by which the interior kernel copies
+// its rows from one parity's state (boxes: RingSlot in lbm_interior.cu): f
+// the populations, f3 from plane 2 on with a plane stride of one plane plus
+// one row, a the u-carry's words, lo its 16-bit low words (kFmtF32H only),
+// s the source carry.
+struct alignas(128) InteriorMaps {
+    CUtensorMap f, f3, a, lo, s;
+};
+// The maps of the state (f, a, s); xj: of the extrapolated scheme.
+cudaError_t interior_maps(int fmt, bool xj, const void* f, const void* a, const void* s, int64_t pitch, int64_t plane,
+                          int ny, InteriorMaps* out);
+// The most rows an interior tile may have at this pitch (its byte offsets
+// are 32-bit).
+int interior_max_rows(int fmt, int64_t pitch);
 // One step of the interior: a launch of R.total CTAs over the rectangles.
-cudaError_t launch_interior(int fmt, const StepParams& p, const InteriorRects& R, cudaStream_t s, bool fields);
+cudaError_t launch_interior(int fmt, const StepParams& p, const InteriorRects& R, const InteriorMaps& maps, cudaStream_t s,
+                            bool fields);
 
 // The interiors of a batch of bodies for one time step: one CTA of
-// kInteriorThreads threads per item, the interior tile (strip a, chunk b) of
-// the parameter-table entry inst (a member's rectangle, with its strip grid
-// and rows per chunk).
-struct BatchItem {
-    int32_t inst, a, b;
-    int32_t pad;
-};
+// kInteriorThreads threads per item, a tile of the parameter-table entry inst
+// (a member's rectangle, with its strip grid).
 struct BatchInteriorLaunch {
-    const StepParams* params;  // device table, indexed by BatchItem::inst
-    const BatchItem* items;    // device list of interior tiles, one per CTA
+    const StepParams* params;  // device table, indexed by InteriorItem::inst
+    const InteriorMaps* maps;       // device table of the entries' tensor maps, indexed as params
+    const InteriorItem* items; // device list of interior tiles, one per CTA
     int32_t fields;            // also write u, v, r to params.fields
     int32_t nitems;            // tiles in the list
 };

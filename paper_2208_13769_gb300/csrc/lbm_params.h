@@ -37,9 +37,8 @@ struct StepParams {
     int32_t scheme;  // 0 explicit (Algorithm 1), 1 predictor-corrector
     // interior kernel: output rectangle, its grid and its row ring
     int32_t rect[4];     // x_lo, x_hi, y_lo, y_hi
-    int32_t tiles_x, tiles_y;  // column strips x row chunks
-    int32_t chunk_rows;        // rows per chunk
-    int32_t ring_slots;        // row slots of the bulk-copy ring (lookahead + 3)
+    int32_t pad0[3];
+    int32_t ring_slots;        // rows of the ring, in flight or in work
     int32_t strip_x0;          // first column of strip 0
     int32_t strip_w;           // output columns per strip
     int32_t pad1[2];

@@ -53,13 +53,23 @@ __device__ __forceinline__ bool mbar_wait_n(uint64_t* bar, uint32_t parity, uint
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
     return mbar_wait_n(bar, parity, kSpinLimit);
 }
-// Bulk global -> shared copy; both addresses 16-byte aligned, bytes % 16 == 0.
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+
+// Tiled global -> shared copy of a 3-D box (x, row, plane) by a tensor map;
+// dst is 128-byte aligned, x times the element size a multiple of 16.
+__device__ __forceinline__ void tensor_load(uint32_t dst, const void* map, int x, int row, int plane, uint32_t bar) {
     asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            smem_addr(dst)),
-        "l"(src), "r"(bytes), "r"(smem_addr(bar))
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
+        "[%5];" ::"r"(dst),
+        "l"(map), "r"(x), "r"(row), "r"(plane), "r"(bar)
         : "memory");
+}
+__device__ __forceinline__ void prefetch_tensor_map(const void* map) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
+}
+// A tensor map that the host wrote to global memory, before this thread's
+// first copy by it.
+__device__ __forceinline__ void acquire_tensor_map(const void* map) {
+    asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(map) : "memory");
 }
 
 // T*(t) of a Neumann edge: T0 outside [t_on, t_off), ramping to T1 over t_ramp.
