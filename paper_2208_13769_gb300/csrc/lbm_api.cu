@@ -121,6 +121,15 @@ StepParams lbm::make_params(const lbm_ctx* c, int parity) {
     L[kLatCOverRho0] = p.c / p.rho0;
     L[kLatRho0OverC] = p.rho0 / p.c;
     L[kLatRho0] = p.rho0;
+    L[kLatOmega18] = p.omega / 18.0;
+    L[kLatOmega12] = p.omega / 12.0;
+    L[kLatOmega4] = p.omega / 4.0;
+    L[kLatOmega3] = p.omega / 3.0;
+    L[kLatForce3] = L[kLatForcePref] / 3.0;
+    L[kLatHalfOneMOmega] = 0.5 * L[kLatOneMOmega];
+    L[kLatOmega18Lo] = fma(-18.0, L[kLatOmega18], p.omega) / 18.0;
+    L[kLatOmega3Lo] = fma(-3.0, L[kLatOmega3], p.omega) / 3.0;
+    L[kLatForce3Lo] = fma(-3.0, L[kLatForce3], L[kLatForcePref]) / 3.0;
     for (int k = 0; k < kLatCount; ++k) p.lat_f[k] = float(L[k]);
     for (int k = 0; k < 4; ++k) p.hole[k] = c->hole[k];
     for (int k = 0; k < 8; ++k) p.hole_T[k] = c->hole_T[k];

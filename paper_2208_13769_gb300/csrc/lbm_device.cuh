@@ -113,14 +113,29 @@ __device__ __forceinline__ T feq_odd_over_w(int i, T j0, T j1, T inv_c) {
 // 1 / J, J = det F near 1 for any admissible deformation.  FP32: the
 // hardware's approximate reciprocal, one instruction on the critical path of
 // stage B (its error, about an ulp, is far inside the FP32 path's
-// tolerance); FP64: the correctly rounded reciprocal, for the FP64 path's
-// parity with the oracle.
+// tolerance); FP64: the hardware's seed (20 bits or more) and one step of
+// Householder's third-order iteration, x (1 + e + e^2) with e = 1 - J x,
+// which leaves e^3 < 2^-60 and the roundings of three operations (the
+// correctly rounded reciprocal takes more than twice as many).
 __device__ __forceinline__ float rcp_j(float x) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-__device__ __forceinline__ double rcp_j(double x) { return __drcp_rn(x); }
+__device__ __forceinline__ double rcp_j(double x) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+
+// !(J > 0), NaN included.  FP64: on the bits, since a comparison would take
+// a slot of the FP64 pipe.
+__device__ __forceinline__ bool not_positive(float J) { return !(J > 0.0f); }
+__device__ __forceinline__ bool not_positive(double J) {
+    const long long b = __double_as_longlong(J);
+    return b <= 0 || b > 0x7ff0000000000000LL;
+}
 
 template <class T>
 __device__ __forceinline__ T stress_remainder(T h11, T h12, T h21, T h22, T lam, T mu, T& q11, T& q12,
@@ -133,6 +148,28 @@ __device__ __forceinline__ T stress_remainder(T h11, T h12, T h21, T h22, T lam,
     q11 = (mu * (T(2) * D - d * (T(1) + T(2) * h11 + h22)) + vol * (T(1) + h22)) * invJ;
     q22 = (mu * (T(2) * D - d * (T(1) + T(2) * h22 + h11)) + vol * (T(1) + h11)) * invJ;
     const T g = -d * (mu + T(0.5) * lam * (T(2) + d)) * invJ;
+    q12 = g * h21;
+    q21 = g * h12;
+    return J;
+}
+
+// The same in FP64.  This part's SMs issue two FP64 lanes a cycle against
+// 128 of FP32, so the FP64 step is bound by the number of its FP64
+// operations (82 % of the pipe busy at 171 a node): here 34 against about 50,
+// with the terms that J Q11 and J Q22 share formed once and mu and the
+// volumetric factor scaled by 1 / J before they are used.
+template <>
+__device__ __forceinline__ double stress_remainder<double>(double h11, double h12, double h21, double h22, double lam,
+                                                           double mu, double& q11, double& q12, double& q21,
+                                                           double& q22) {
+    const double D = fma(h11, h22, -(h12 * h21));
+    const double tr = h11 + h22, d = tr + D, J = 1.0 + d;
+    const double invJ = rcp_j(J);
+    const double vJ = d * fma(0.5 * lam, d, lam) * invJ, mJ = mu * invJ;  // (lambda / 2 d (2 + d), mu) / J
+    const double g1 = 1.0 + h22, g2 = 1.0 + h11, D2 = D + D;
+    q11 = fma(vJ, g1, mJ * fma(-d, tr + g2, D2));
+    q22 = fma(vJ, g2, mJ * fma(-d, tr + g1, D2));
+    const double g = -fma(d, mJ, vJ);
     q12 = g * h21;
     q21 = g * h12;
     return J;

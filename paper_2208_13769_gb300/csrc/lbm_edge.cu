@@ -26,7 +26,7 @@ namespace lbm {
 static_assert(sizeof(StepParams) % 16 == 0, "StepParams is copied to shared memory in 16-byte words");
 
 template <class TS, class TC, class UT, int MODE, bool HOLE, bool XJ>
-__global__ void __launch_bounds__(kEdgeThreads, 3)
+__global__ void __launch_bounds__(kEdgeThreads, sizeof(TC) == 8 ? 2 : 3)
     edge_tile_kernel(const __grid_constant__ EdgeLaunch L, const __grid_constant__ ImageLaunch I) {
     constexpr int N = kEdgeThreads;
     static_assert(kImageThreads <= N, "an image tile fits an edge CTA");

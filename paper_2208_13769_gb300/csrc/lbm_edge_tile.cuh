@@ -140,6 +140,17 @@ __device__ __noinline__ void boundary_links(TS* fdst, Geo g, const StepParams& p
     }
 }
 
+// |a| + |b| + |c| + |d| < 1e30.  FP64: on the exponents (each below 2^97 is
+// enough), the sum itself only where those do not settle it.
+__device__ __forceinline__ bool moderate(float a, float b, float c, float d) {
+    return fabsf(a) + fabsf(b) + fabsf(c) + fabsf(d) < 1e30f;
+}
+__device__ __forceinline__ bool moderate(double a, double b, double c, double d) {
+    auto mag = [](double x) { return __double2hiint(x) & 0x7fffffff; };
+    if (max(max(mag(a), mag(b)), max(mag(c), mag(d))) < 0x46000000) return true;
+    return fabs(a) + fabs(b) + fabs(c) + fabs(d) < 1e30;
+}
+
 // The tile `tile` of the body whose parameters are p (mode 0: one time step;
 // mode 1: the initialisation).  Every thread of the CTA calls it (threads
 // beyond tw x th idle through the barriers).  Shared memory: su holds 2 x
@@ -230,6 +241,12 @@ __device__ __forceinline__ void edge_tile_body(const EdgeTile& tile, const StepP
             f[i] = Codec<TS, TC>::ld(fsrc[int64_t(i) * plane + o - ex(i) - int64_t(ey(i)) * pitch], i, p);
         const UT A0 = UT::load(as0, o, p);
         const UT A1 = UT::load(as1, o, p);
+        if constexpr (sizeof(TC) == 8) {  // FP64 goes on with sums and differences of opposite populations
+            double h[9];
+            pairs64(f, h);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) f[i] = h[i];
+        }
         if (inC) {
             so0 = s_src[o];
             so1 = s_src[o + plane];
@@ -242,8 +259,13 @@ __device__ __forceinline__ void edge_tile_body(const EdgeTile& tile, const StepP
             su[(ty * 2) * tw + tx] = A0;
             su[(ty * 2 + 1) * tw + tx] = A1;
         } else {
-            const TC m0 = (f[1] - f[3]) + (f[5] - f[6]) + (f[8] - f[7]);
-            const TC m1 = (f[2] - f[4]) + (f[5] - f[8]) + (f[6] - f[7]);
+            TC m0, m1;
+            if constexpr (sizeof(TC) == 8) {
+                momentum64(f, m0, m1);
+            } else {
+                m0 = (f[1] - f[3]) + (f[5] - f[6]) + (f[8] - f[7]);
+                m1 = (f[2] - f[4]) + (f[5] - f[8]) + (f[6] - f[7]);
+            }
             su[(ty * 2) * tw + tx] = A0.add(k.ku * m0);
             su[(ty * 2 + 1) * tw + tx] = A1.add(k.ku * m1);
         }
@@ -276,7 +298,7 @@ __device__ __forceinline__ void edge_tile_body(const EdgeTile& tile, const StepP
         TC q11, q12, q21, q22;
         const TC J =
             stress_remainder<TC>(hh[0][0], hh[0][1], hh[1][0], hh[1][1], k.lam, k.mu, q11, q12, q21, q22);
-        bad |= !(J > TC(0)) || !(fabs(q11) + fabs(q12) + fabs(q21) + fabs(q22) < TC(1e30));
+        bad |= not_positive(J) || !moderate(q11, q12, q21, q22);
         TC* qr = sq + (ty * 4) * tw + tx;
         qr[0] = q11;
         qr[tw] = q12;
@@ -312,14 +334,20 @@ __device__ __forceinline__ void edge_tile_body(const EdgeTile& tile, const StepP
         const UT ux = su[(ty * 2) * tw + tx], uy = su[(ty * 2 + 1) * tw + tx];
         TC r, j0, j1, pxx, pxy, pyy;
         TC du0 = TC(0), du1 = TC(0);  // predictor correction of u*
+        constexpr bool PAIRS = MODE == 0 && sizeof(TC) == 8;
         if (MODE == 0) {
-            r = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8];
-            const TC m0 = (f[1] - f[3]) + (f[5] - f[6]) + (f[8] - f[7]);
-            const TC m1 = (f[2] - f[4]) + (f[5] - f[8]) + (f[6] - f[7]);
-            const TC dg = (f[5] + f[6]) + (f[7] + f[8]);
-            pxx = (f[1] + f[3]) + dg;
-            pyy = (f[2] + f[4]) + dg;
-            pxy = (f[5] - f[6]) + (f[7] - f[8]);
+            TC m0, m1;
+            if constexpr (PAIRS) {
+                momentum64(f, m0, m1);
+            } else {
+                r = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8];
+                m0 = (f[1] - f[3]) + (f[5] - f[6]) + (f[8] - f[7]);
+                m1 = (f[2] - f[4]) + (f[5] - f[8]) + (f[6] - f[7]);
+                const TC dg = (f[5] + f[6]) + (f[7] + f[8]);
+                pxx = (f[1] + f[3]) + dg;
+                pyy = (f[2] + f[4]) + dg;
+                pxy = (f[5] - f[6]) + (f[7] - f[8]);
+            }
             if (XJ) {  // u(t + dt) = u(t) + ku (jh(t) + jh) = E - (F - D) + ku jh
                 j0 = m0 + TC(0.5) * sn0;
                 j1 = m1 + TC(0.5) * sn1;
@@ -347,45 +375,53 @@ __device__ __forceinline__ void edge_tile_body(const EdgeTile& tile, const StepP
             j1 = k.rho0_over_c * TC(p.v0 ? p.v0[hh + 1] : 0.0);
         }
 
-        // equilibrium (Sec. 5), He forcing (Eq. source), BGK collision
-        // (Eq. col), by opposite pairs: f^col_i = (1 - omega) f_i
-        //   + w_i (omega E_i + 3 e_i.(omega jh + (1 - omega/2) s)),
-        // E_i the even part of f^eq_i / w_i (equal for i and its opposite)
-        const TC tr15 = TC(1.5) * (pxx + pyy);
-        const TC E0 = TC(2) * r - tr15;
-        const TC Ex = TC(0.5) * r + TC(4.5) * pxx - tr15;
-        const TC Ey = TC(0.5) * r + TC(4.5) * pyy - tr15;
-        const TC Ed = -r + TC(4.5) * (pxx + pyy) - tr15;
-        const TC Ep = Ed + TC(9) * pxy, Em = Ed - TC(9) * pxy;
-        const TC w0 = wgt<TC>(0), w1 = wgt<TC>(1), w5 = wgt<TC>(5);
-        if (MODE == 1) {
-            const TC o0 = TC(3) * j0, o1 = TC(3) * j1;
-            f[0] = w0 * E0;
-            f[1] = w1 * (Ex + o0);
-            f[3] = w1 * (Ex - o0);
-            f[2] = w1 * (Ey + o1);
-            f[4] = w1 * (Ey - o1);
-            f[5] = w5 * (Ep + o0 + o1);
-            f[7] = w5 * (Ep - o0 - o1);
-            f[6] = w5 * (Em - o0 + o1);
-            f[8] = w5 * (Em + o0 - o1);
-        }
-        const TC b0 = TC(3) * (k.omega * j0 + k.force_pref * sn0);
-        const TC b1 = TC(3) * (k.omega * j1 + k.force_pref * sn1);
-        const TC ax = wmul<TS>(w1, k.omega * Ex), ay = wmul<TS>(w1, k.omega * Ey);
-        const TC ap = wmul<TS>(w5, k.omega * Ep), am = wmul<TS>(w5, k.omega * Em);
-        const TC bx = wmul<TS>(w1, b0), by = wmul<TS>(w1, b1);
-        const TC bp = wmul<TS>(w5, b0 + b1), bm = wmul<TS>(w5, b1 - b0);
         TC fc[9];
-        fc[0] = k.one_m_omega * f[0] + wmul<TS>(w0, k.omega * E0);
-        fc[1] = k.one_m_omega * f[1] + (ax + bx);
-        fc[3] = k.one_m_omega * f[3] + (ax - bx);
-        fc[2] = k.one_m_omega * f[2] + (ay + by);
-        fc[4] = k.one_m_omega * f[4] + (ay - by);
-        fc[5] = k.one_m_omega * f[5] + (ap + bp);
-        fc[7] = k.one_m_omega * f[7] + (ap - bp);
-        fc[6] = k.one_m_omega * f[6] + (am + bm);
-        fc[8] = k.one_m_omega * f[8] + (am - bm);
+        if constexpr (PAIRS) {
+            TC dg;
+            collide64(f, j0, j1, sn0, sn1, k, fc, dg, r);
+            pxx = f[1] + dg;
+            pyy = f[2] + dg;
+            pxy = f[3] - f[4];
+        } else {
+            // equilibrium (Sec. 5), He forcing (Eq. source), BGK collision
+            // (Eq. col), by opposite pairs: f^col_i = (1 - omega) f_i
+            //   + w_i (omega E_i + 3 e_i.(omega jh + (1 - omega/2) s)),
+            // E_i the even part of f^eq_i / w_i (equal for i and its opposite)
+            const TC tr15 = TC(1.5) * (pxx + pyy);
+            const TC E0 = TC(2) * r - tr15;
+            const TC Ex = TC(0.5) * r + TC(4.5) * pxx - tr15;
+            const TC Ey = TC(0.5) * r + TC(4.5) * pyy - tr15;
+            const TC Ed = -r + TC(4.5) * (pxx + pyy) - tr15;
+            const TC Ep = Ed + TC(9) * pxy, Em = Ed - TC(9) * pxy;
+            const TC w0 = wgt<TC>(0), w1 = wgt<TC>(1), w5 = wgt<TC>(5);
+            if (MODE == 1) {
+                const TC o0 = TC(3) * j0, o1 = TC(3) * j1;
+                f[0] = w0 * E0;
+                f[1] = w1 * (Ex + o0);
+                f[3] = w1 * (Ex - o0);
+                f[2] = w1 * (Ey + o1);
+                f[4] = w1 * (Ey - o1);
+                f[5] = w5 * (Ep + o0 + o1);
+                f[7] = w5 * (Ep - o0 - o1);
+                f[6] = w5 * (Em - o0 + o1);
+                f[8] = w5 * (Em + o0 - o1);
+            }
+            const TC b0 = TC(3) * (k.omega * j0 + k.force_pref * sn0);
+            const TC b1 = TC(3) * (k.omega * j1 + k.force_pref * sn1);
+            const TC ax = wmul<TS>(w1, k.omega * Ex), ay = wmul<TS>(w1, k.omega * Ey);
+            const TC ap = wmul<TS>(w5, k.omega * Ep), am = wmul<TS>(w5, k.omega * Em);
+            const TC bx = wmul<TS>(w1, b0), by = wmul<TS>(w1, b1);
+            const TC bp = wmul<TS>(w5, b0 + b1), bm = wmul<TS>(w5, b1 - b0);
+            fc[0] = k.one_m_omega * f[0] + wmul<TS>(w0, k.omega * E0);
+            fc[1] = k.one_m_omega * f[1] + (ax + bx);
+            fc[3] = k.one_m_omega * f[3] + (ax - bx);
+            fc[2] = k.one_m_omega * f[2] + (ay + by);
+            fc[4] = k.one_m_omega * f[4] + (ay - by);
+            fc[5] = k.one_m_omega * f[5] + (ap + bp);
+            fc[7] = k.one_m_omega * f[7] + (ap - bp);
+            fc[6] = k.one_m_omega * f[6] + (am + bm);
+            fc[8] = k.one_m_omega * f[8] + (am - bm);
+        }
 
         // stores, with the periodic images of nodes near a seam
         const bool short_x = g.perx && nx < 6, short_y = g.pery && ny < 6;

@@ -278,14 +278,25 @@ __device__ __forceinline__ bool interior_tile(const StepParams& p, const Interio
             const unsigned char* pf = slot + e_own;
 #pragma unroll
             for (int i = 0; i < 9; ++i) gcur[i] = Codec<TS, TC>::ld(Slot::pop(pf, i), i, p);
+            if constexpr (sizeof(TC) == 8) {  // FP64 keeps them as sums and differences of opposite ones
+                double f[9];
+#pragma unroll
+                for (int i = 0; i < 9; ++i) f[i] = gcur[i];
+                pairs64(f, gcur);
+            }
             const UT A0 = UT::decode(Slot::carry(slot, 0, ec, el), p), A1 = UT::decode(Slot::carry(slot, 1, ec, el), p);
             if (XJ) {  // u* = u(t) + ku (3 jh(t) - jh(t - dt)) = E
                 su[(sA * 2) * NT + t] = A0;
                 su[(sA * 2 + 1) * NT + t] = A1;
             } else {
                 const TC* g = gcur;
-                const TC m0 = (g[1] - g[3]) + (g[5] - g[6]) + (g[8] - g[7]);
-                const TC m1 = (g[2] - g[4]) + (g[5] - g[8]) + (g[6] - g[7]);
+                TC m0, m1;
+                if constexpr (sizeof(TC) == 8) {
+                    momentum64(g, m0, m1);
+                } else {
+                    m0 = (g[1] - g[3]) + (g[5] - g[6]) + (g[8] - g[7]);
+                    m1 = (g[2] - g[4]) + (g[5] - g[8]) + (g[6] - g[7]);
+                }
                 su[(sA * 2) * NT + t] = A0.add(k.ku * m0);
                 su[(sA * 2 + 1) * NT + t] = A1.add(k.ku * m1);
             }
@@ -309,7 +320,7 @@ __device__ __forceinline__ bool interior_tile(const StepParams& p, const Interio
             const TC h22 = rp[NT + t].minus(rm[NT + t]) * k.inv_2dx;
             TC q11, q12, q21, q22;
             const TC J = stress_remainder<TC>(h11, h12, h21, h22, k.lam, k.mu, q11, q12, q21, q22);
-            bad |= !(J > TC(0));  // also catches a non-finite displacement gradient
+            bad |= not_positive(J);  // also catches a non-finite displacement gradient
             TC* qr = sq + (q & 1) * 2 * NT;
             qr[t] = q11;
             qr[NT + t] = q21;
@@ -337,13 +348,14 @@ __device__ __forceinline__ bool interior_tile(const StepParams& p, const Interio
             const TC sn1 = k.sb1 + k.sq_scale * ((qc[NT + tp] - qc[NT + tm]) + (qp[1] - qm[1]));
 
             const TC* f = fp2;
-            const TC r = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8];
-            const TC m0 = (f[1] - f[3]) + (f[5] - f[6]) + (f[8] - f[7]);
-            const TC m1 = (f[2] - f[4]) + (f[5] - f[8]) + (f[6] - f[7]);
-            const TC dg = (f[5] + f[6]) + (f[7] + f[8]);
-            const TC pxx = (f[1] + f[3]) + dg;
-            const TC pyy = (f[2] + f[4]) + dg;
-            const TC pxy = (f[5] - f[6]) + (f[7] - f[8]);
+            TC r, m0, m1;
+            if constexpr (sizeof(TC) == 8) {
+                momentum64(f, m0, m1);
+            } else {
+                r = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8];
+                m0 = (f[1] - f[3]) + (f[5] - f[6]) + (f[8] - f[7]);
+                m1 = (f[2] - f[4]) + (f[5] - f[8]) + (f[6] - f[7]);
+            }
             TC j0, j1, du0 = TC(0), du1 = TC(0);
             if (XJ) {  // u(t + dt) = u(t) + ku (jh(t) + jh) = E - (F - D) + ku jh
                 j0 = m0 + TC(0.5) * sn0;
@@ -360,30 +372,39 @@ __device__ __forceinline__ bool interior_tile(const StepParams& p, const Interio
                 j1 = m1 + TC(0.5) * so1;
             }
 
-            // equilibrium, He forcing and BGK collision by opposite pairs
-            const TC tr15 = TC(1.5) * (pxx + pyy);
-            const TC E0 = TC(2) * r - tr15;
-            const TC Ex = TC(0.5) * r + TC(4.5) * pxx - tr15;
-            const TC Ey = TC(0.5) * r + TC(4.5) * pyy - tr15;
-            const TC Ed = -r + TC(4.5) * (pxx + pyy) - tr15;
-            const TC Ep = Ed + TC(9) * pxy, Em = Ed - TC(9) * pxy;
-            const TC w0 = wgt<TC>(0), w1 = wgt<TC>(1), w5 = wgt<TC>(5);
-            const TC b0 = TC(3) * (k.omega * j0 + k.force_pref * sn0);
-            const TC b1 = TC(3) * (k.omega * j1 + k.force_pref * sn1);
-            const TC ax = wmul<TS>(w1, k.omega * Ex), ay = wmul<TS>(w1, k.omega * Ey);
-            const TC ap = wmul<TS>(w5, k.omega * Ep), am = wmul<TS>(w5, k.omega * Em);
-            const TC bx = wmul<TS>(w1, b0), by = wmul<TS>(w1, b1);
-            const TC bp = wmul<TS>(w5, b0 + b1), bm = wmul<TS>(w5, b1 - b0);
             TC fc[9];
-            fc[0] = k.one_m_omega * f[0] + wmul<TS>(w0, k.omega * E0);
-            fc[1] = k.one_m_omega * f[1] + (ax + bx);
-            fc[3] = k.one_m_omega * f[3] + (ax - bx);
-            fc[2] = k.one_m_omega * f[2] + (ay + by);
-            fc[4] = k.one_m_omega * f[4] + (ay - by);
-            fc[5] = k.one_m_omega * f[5] + (ap + bp);
-            fc[7] = k.one_m_omega * f[7] + (ap - bp);
-            fc[6] = k.one_m_omega * f[6] + (am + bm);
-            fc[8] = k.one_m_omega * f[8] + (am - bm);
+            if constexpr (sizeof(TC) == 8) {
+                TC dg;
+                collide64(f, j0, j1, sn0, sn1, k, fc, dg, r);
+            } else {
+                const TC dg = (f[5] + f[6]) + (f[7] + f[8]);
+                const TC pxx = (f[1] + f[3]) + dg;
+                const TC pyy = (f[2] + f[4]) + dg;
+                const TC pxy = (f[5] - f[6]) + (f[7] - f[8]);
+                // equilibrium, He forcing and BGK collision by opposite pairs
+                const TC tr15 = TC(1.5) * (pxx + pyy);
+                const TC E0 = TC(2) * r - tr15;
+                const TC Ex = TC(0.5) * r + TC(4.5) * pxx - tr15;
+                const TC Ey = TC(0.5) * r + TC(4.5) * pyy - tr15;
+                const TC Ed = -r + TC(4.5) * (pxx + pyy) - tr15;
+                const TC Ep = Ed + TC(9) * pxy, Em = Ed - TC(9) * pxy;
+                const TC w0 = wgt<TC>(0), w1 = wgt<TC>(1), w5 = wgt<TC>(5);
+                const TC b0 = TC(3) * (k.omega * j0 + k.force_pref * sn0);
+                const TC b1 = TC(3) * (k.omega * j1 + k.force_pref * sn1);
+                const TC ax = wmul<TS>(w1, k.omega * Ex), ay = wmul<TS>(w1, k.omega * Ey);
+                const TC ap = wmul<TS>(w5, k.omega * Ep), am = wmul<TS>(w5, k.omega * Em);
+                const TC bx = wmul<TS>(w1, b0), by = wmul<TS>(w1, b1);
+                const TC bp = wmul<TS>(w5, b0 + b1), bm = wmul<TS>(w5, b1 - b0);
+                fc[0] = k.one_m_omega * f[0] + wmul<TS>(w0, k.omega * E0);
+                fc[1] = k.one_m_omega * f[1] + (ax + bx);
+                fc[3] = k.one_m_omega * f[3] + (ax - bx);
+                fc[2] = k.one_m_omega * f[2] + (ay + by);
+                fc[4] = k.one_m_omega * f[4] + (ay - by);
+                fc[5] = k.one_m_omega * f[5] + (ap + bp);
+                fc[7] = k.one_m_omega * f[7] + (ap - bp);
+                fc[6] = k.one_m_omega * f[6] + (am + bm);
+                fc[8] = k.one_m_omega * f[8] + (am - bm);
+            }
             const uint32_t o = off_a - 2 * dpitch;  // row a - 2 sg = gy
 #pragma unroll
             for (int i = 0; i < 9; ++i) *elem(fd[i], o) = Codec<TS, TC>::st(fc[i], i, p);

@@ -66,8 +66,8 @@ struct StepParams {
     EdgeBC bc[4];
     // lattice constants, computed once on the host in FP64 (kLat* indices);
     // lat_f holds the same values rounded to FP32
-    double lat_d[16];
-    float lat_f[16];
+    double lat_d[24];
+    float lat_f[24];
     // a rectangular hole (Sec. 7's plate with a hole): removed nodes x0 <= x
     // < x1, y0 <= y < y1 (x0 >= x1: none), and the constant traction on its
     // faces at x0, x1, y0, y1 (x and y components)
@@ -96,6 +96,15 @@ enum LatIndex : int {
     kLatCOverRho0,      // c / rho0
     kLatRho0OverC,      // rho0 / c
     kLatRho0,           // rho0
+    kLatOmega18,        // omega / 18 (the FP64 collision's products of omega
+    kLatOmega12,        // omega / 12  and the lattice weights, collide64)
+    kLatOmega4,         // omega / 4
+    kLatOmega3,         // omega / 3
+    kLatForce3,         // (1 - omega / 2) / 3
+    kLatHalfOneMOmega,  // (1 - omega) / 2
+    kLatOmega18Lo,      // what kLatOmega18, kLatOmega3 and kLatForce3 lack of
+    kLatOmega3Lo,       // the exact quotients
+    kLatForce3Lo,
     kLatCount
 };
 

@@ -152,6 +152,7 @@ template <class TC>
 struct LatConsts {
     TC omega, one_m_omega, force_pref, ku, inv_2dx, sq_scale, sb0, sb1, lam, mu, inv_c2, c_over_rho0,
         rho0_over_c, rho0;
+    TC omega18, omega12, omega4, omega3, force3, half_one_m_omega, omega18_lo, omega3_lo, force3_lo;
     __device__ __forceinline__ void load(const StepParams& p) {
         omega = lat_const<TC>(p, kLatOmega);
         one_m_omega = lat_const<TC>(p, kLatOneMOmega);
@@ -167,8 +168,68 @@ struct LatConsts {
         c_over_rho0 = lat_const<TC>(p, kLatCOverRho0);
         rho0_over_c = lat_const<TC>(p, kLatRho0OverC);
         rho0 = lat_const<TC>(p, kLatRho0);
+        omega18 = lat_const<TC>(p, kLatOmega18);
+        omega12 = lat_const<TC>(p, kLatOmega12);
+        omega4 = lat_const<TC>(p, kLatOmega4);
+        omega3 = lat_const<TC>(p, kLatOmega3);
+        force3 = lat_const<TC>(p, kLatForce3);
+        half_one_m_omega = lat_const<TC>(p, kLatHalfOneMOmega);
+        omega18_lo = lat_const<TC>(p, kLatOmega18Lo);
+        omega3_lo = lat_const<TC>(p, kLatOmega3Lo);
+        force3_lo = lat_const<TC>(p, kLatForce3Lo);
     }
 };
+
+// The FP64 collision on sums and differences of opposite populations, g =
+// {f0, f1 + f3, f2 + f4, f5 + f7, f6 + f8, f1 - f3, f2 - f4, f5 - f7, f6 -
+// f8}: the moments, equilibrium and forcing need only these, each pair's
+// even and odd part relax separately, and omega times the lattice weights
+// come from the constants (stage C in 64 FP64 operations against about 95).
+// Mass and momentum are what a step must keep: there the constants' rounding
+// errors (2^-54, of the same sign at every node and step) are made good.
+__device__ __forceinline__ void pairs64(const double* f, double* g) {
+    g[0] = f[0];
+    g[1] = f[1] + f[3];
+    g[2] = f[2] + f[4];
+    g[3] = f[5] + f[7];
+    g[4] = f[6] + f[8];
+    g[5] = f[1] - f[3];
+    g[6] = f[2] - f[4];
+    g[7] = f[5] - f[7];
+    g[8] = f[6] - f[8];
+}
+__device__ __forceinline__ void momentum64(const double* g, double& m0, double& m1) {
+    m0 = g[5] + (g[7] - g[8]);
+    m1 = g[6] + (g[7] + g[8]);
+}
+// fc: the post-collision populations; j, s: jh and s; dg, r: the diagonals'
+// sum and the zeroth moment.
+__device__ __forceinline__ void collide64(const double* g, double j0, double j1, double s0, double s1,
+                                          const LatConsts<double>& k, double* fc, double& dg, double& r) {
+    dg = g[3] + g[4];
+    const double ax = g[1] + g[2];
+    r = (g[0] + ax) + dg;
+    const double q = k.omega12 * fma(2.0, dg, ax);  // omega / 12 tr Pf
+    const double pd = k.omega4 * (g[1] - g[2]), pxy = k.omega4 * (g[3] - g[4]);
+    const double er = fma(k.omega18, r, k.omega18_lo * r);
+    const double e1 = er + q, e5 = fma(-0.5, er, q);
+    fc[0] = fma(k.one_m_omega, g[0], fma(16.0, er, -8.0 * q));
+    const double bx = fma(k.omega3, j0, fma(k.force3, s0, fma(k.omega3_lo, j0, k.force3_lo * s0)));
+    const double by = fma(k.omega3, j1, fma(k.force3, s1, fma(k.omega3_lo, j1, k.force3_lo * s1)));
+    const double h = k.half_one_m_omega;
+    const double p1 = fma(h, g[1], e1 + pd), o1 = fma(h, g[5], bx);
+    const double p2 = fma(h, g[2], e1 - pd), o2 = fma(h, g[6], by);
+    const double p5 = fma(h, g[3], e5 + pxy), o5 = fma(h, g[7], 0.25 * (bx + by));
+    const double p6 = fma(h, g[4], e5 - pxy), o6 = fma(h, g[8], 0.25 * (by - bx));
+    fc[1] = p1 + o1;
+    fc[3] = p1 - o1;
+    fc[2] = p2 + o2;
+    fc[4] = p2 - o2;
+    fc[5] = p5 + o5;
+    fc[7] = p5 - o5;
+    fc[6] = p6 + o6;
+    fc[8] = p6 - o6;
+}
 
 // Lattice-unit equilibrium over w_i, even part (r, Pf): used by the
 // anti-bounce-back rule.
