@@ -348,13 +348,17 @@ __device__ __forceinline__ bool interior_tile(const StepParams& p, const Interio
             const TC sn1 = k.sb1 + k.sq_scale * ((qc[NT + tp] - qc[NT + tm]) + (qp[1] - qm[1]));
 
             const TC* f = fp2;
-            TC r, m0, m1;
+            TC r, m0, m1, pxx, pyy, pxy;
             if constexpr (sizeof(TC) == 8) {
                 momentum64(f, m0, m1);
             } else {
                 r = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8];
                 m0 = (f[1] - f[3]) + (f[5] - f[6]) + (f[8] - f[7]);
                 m1 = (f[2] - f[4]) + (f[5] - f[8]) + (f[6] - f[7]);
+                const TC dg = (f[5] + f[6]) + (f[7] + f[8]);
+                pxx = (f[1] + f[3]) + dg;
+                pyy = (f[2] + f[4]) + dg;
+                pxy = (f[5] - f[6]) + (f[7] - f[8]);
             }
             TC j0, j1, du0 = TC(0), du1 = TC(0);
             if (XJ) {  // u(t + dt) = u(t) + ku (jh(t) + jh) = E - (F - D) + ku jh
@@ -377,10 +381,6 @@ __device__ __forceinline__ bool interior_tile(const StepParams& p, const Interio
                 TC dg;
                 collide64(f, j0, j1, sn0, sn1, k, fc, dg, r);
             } else {
-                const TC dg = (f[5] + f[6]) + (f[7] + f[8]);
-                const TC pxx = (f[1] + f[3]) + dg;
-                const TC pyy = (f[2] + f[4]) + dg;
-                const TC pxy = (f[5] - f[6]) + (f[7] - f[8]);
                 // equilibrium, He forcing and BGK collision by opposite pairs
                 const TC tr15 = TC(1.5) * (pxx + pyy);
                 const TC E0 = TC(2) * r - tr15;
