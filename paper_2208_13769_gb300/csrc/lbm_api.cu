@@ -243,6 +243,35 @@ void lbm::plan_rects(const lbm_ctx* c, bool edge_only, bool seams_inside, int ir
     }
 }
 
+// The tile shape of a body that runs as edge tiles only.
+// FP64 is bound by its operations, of which an SM issues one warp's in 16
+// cycles: a tile costs about 570 of them at 28 x 4 nodes, 770 at 12 x 12 (830
+// with what its narrower rows cost more) and 320 at 12 x 4 with 128 threads,
+// and the fullest SM decides: 64 x 64 takes 9.2 / 11.2 / 8.0 us a step, 128 x
+// 128 19.3 / 17.0 / 17.7, 200 x 200 27.8 / 24.3 / 30.7, 350 x 300 53 / 57 / 62.
+// Otherwise a tile is bound by latency and the waves of 3 CTAs per SM decide:
+// 12 x 12 where they are fewer (301 x 203 in FP32: 442 tiles instead of 561,
+// 7.6 us instead of 9.9; 350 x 350: 12.4 and 14.0), else 28 x 4 (256 x 256,
+// two waves of either: 9.2 and 9.0).
+static EdgeShape edge_shape(const lbm_ctx* c) {
+    const EdgeShape shapes[3] = {kEdgeWide, {kEdgeThreads, 16}, {kEdgeThreads / 2, 8}};
+    const int64_t ops[3] = {570, 830, 320};
+    const bool f64 = c->fmt == kFmtF64;
+    EdgeShape best = kEdgeWide;
+    int64_t least = INT64_MAX;
+    for (int k = 0; k < (f64 ? 3 : 2); ++k) {
+        int64_t n = 0;
+        for (int b = 0; b < c->nband; ++b)
+            n += edge_tiles_of_rect(c->brect[b], 0, nullptr, 0, false, shapes[k], bounded_sides(c, c->brect[b]));
+        const int64_t per = int64_t(c->num_sms) * (f64 ? 1 : 3), cost = (n + per - 1) / per * (f64 ? ops[k] : 1);
+        if (cost < least) {
+            least = cost;
+            best = shapes[k];
+        }
+    }
+    return best;
+}
+
 // Rows per CTA of one wave (`wave` CTAs per strip), at least 8 (shorter tiles
 // of mid-size bodies cut the row pipeline's latency: 512 x 512 FP32 in 13 us
 // a step with 8-row tiles against 15 us with 16).
@@ -350,21 +379,22 @@ static cudaError_t build_plan(lbm_ctx* c) {
                                       c->plane, c->ny, &c->maps[q]);
         if (e != cudaSuccess) return e;
     }
+    c->edge_shape = c->has_interior ? kEdgeWide : edge_shape(c);
     int n = 0;
     for (int b = 0; b < c->nband; ++b)
-        n += edge_tiles_of_rect(c->brect[b], 0, nullptr, 0, false, kEdgeThreads, bounded_sides(c, c->brect[b]));
+        n += edge_tiles_of_rect(c->brect[b], 0, nullptr, 0, false, c->edge_shape, bounded_sides(c, c->brect[b]));
     int ni = n;  // the initialisation's tiles: with a hole, the interior rectangles' too
     if (hole)
         for (int q = 0; q < c->n_irect; ++q)
-            ni += edge_tiles_of_rect(c->irect[q], 0, nullptr, 0, false, kEdgeThreads, 0);
+            ni += edge_tiles_of_rect(c->irect[q], 0, nullptr, 0, false, c->edge_shape, 0);
     EdgeTile* h = new (std::nothrow) EdgeTile[size_t(ni)];
     if (!h) return cudaErrorMemoryAllocation;
     int m = 0;
     for (int b = 0; b < c->nband; ++b)
-        m += edge_tiles_of_rect(c->brect[b], 0, h + m, n - m, m == 0, kEdgeThreads, bounded_sides(c, c->brect[b]));
+        m += edge_tiles_of_rect(c->brect[b], 0, h + m, n - m, m == 0, c->edge_shape, bounded_sides(c, c->brect[b]));
     if (hole)
         for (int q = 0; q < c->n_irect; ++q)
-            m += edge_tiles_of_rect(c->irect[q], 0, h + m, ni - m, false, kEdgeThreads, 0);
+            m += edge_tiles_of_rect(c->irect[q], 0, h + m, ni - m, false, c->edge_shape, 0);
     // the images of the interior's nodes next to a periodic seam
     const bool perx = c->bc[0].kind == kPeriodic, pery = c->bc[2].kind == kPeriodic;
     int nimg = 0;
@@ -425,6 +455,7 @@ static cudaError_t launch_band_part(lbm_ctx* c, int parity, bool fields, cudaStr
     L.params = c->dparams + parity;
     L.tiles = c->dtiles;
     L.fields = fields ? 1 : 0;
+    L.threads = c->edge_shape.threads;
     return launch_edge(c->fmt, L, c->n_etiles, st, 0, c->hole[0] < c->hole[1], c->scheme == LBM_SCHEME_EXTRAPOLATED);
 }
 
@@ -436,6 +467,7 @@ static cudaError_t launch_band_images_part(lbm_ctx* c, int parity, bool fields) 
     L.params = c->dparams + parity;
     L.tiles = c->dtiles;
     L.fields = fields ? 1 : 0;
+    L.threads = c->edge_shape.threads;
     return launch_edge_images(c->fmt, L, c->n_etiles, c->dimg, c->n_img, c->stream, c->hole[0] < c->hole[1],
                               c->scheme == LBM_SCHEME_EXTRAPOLATED);
 }
@@ -448,6 +480,7 @@ static cudaError_t launch_step_kernels(lbm_ctx* c, int mode, bool fields, int pa
         L.params = c->dparams + parity;
         L.tiles = c->dtiles;
         L.fields = fields ? 1 : 0;
+        L.threads = c->edge_shape.threads;
         return launch_edge(c->fmt, L, c->n_itiles, c->stream, 1, true, false);
     }
     if (mode == 1) {

@@ -108,6 +108,7 @@ struct lbm_ctx {
     lbm::InteriorMaps maps[2];                // the interior's copies, source state of parity 0 and 1
     lbm::EdgeTile* dtiles = nullptr;     // device: tiles of the edge bands
     int n_etiles = 0;
+    lbm::EdgeShape edge_shape = lbm::kEdgeWide;
     // with a hole, the initialisation runs over the bands' tiles and tiles of
     // the interior rectangles (then after the band tiles in dtiles), so that
     // every face of the hole sees a tile as thick as its band

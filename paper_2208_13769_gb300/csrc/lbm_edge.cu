@@ -3,10 +3,11 @@
 // itself is edge_tile_body of lbm_edge_tile.cuh).
 //
 // The bands hold few nodes, so what bounds their cost is latency, not
-// bandwidth.  Each CTA of 256 threads runs one tile of (tw - 4) x (th - 4)
-// output nodes (tw x th <= 256: tiles exactly as thick as a band, 28 x 4 over
-// larger areas), one thread per node of the tile and its 2-node halo, and
-// hundreds of tiles run at once.
+// bandwidth.  Each CTA of 256 threads (128 where FP64 tiles would not fill
+// the SMs) runs one tile of (tw - 4) x (th - 4) output nodes (tw x th threads:
+// tiles exactly as thick as a band, 28 x 4, 12 x 12 or 12 x 4 over larger
+// areas), one thread per node of the tile and its 2-node halo, and hundreds
+// of tiles run at once.
 //
 // Tiles come from a list (instance, output rectangle, shape), and each
 // instance's parameters from a table in device memory, so one launch serves
@@ -59,11 +60,12 @@ __global__ void __launch_bounds__(kEdgeThreads, sizeof(TC) == 8 ? 2 : 3)
         tile.hx = 2;
         tile.hy = 2;
         tile.lead = b == 0;
+        tile.inv_tw = (65536 + kInitTileW - 1) / kInitTileW;
     }
     {
         const int4* src = reinterpret_cast<const int4*>(L.params + tile.inst);
         int4* dst = reinterpret_cast<int4*>(&sp);
-        for (int q = int(threadIdx.x); q < int(sizeof(StepParams) / 16); q += N) dst[q] = src[q];
+        for (int q = int(threadIdx.x); q < int(sizeof(StepParams) / 16); q += int(blockDim.x)) dst[q] = src[q];
     }
     __syncthreads();
     edge_tile_body<TS, TC, UT, MODE, HOLE, XJ>(tile, sp, L.fields != 0, su, sq, MODE == 1 ? sinit : nullptr,
@@ -81,17 +83,17 @@ cudaError_t launch_edge_t(const EdgeLaunch& L, int ntiles, const ImageTile* img,
     const int64_t total = int64_t(ntiles) + n_img;
     if (total <= 0) return cudaSuccess;
     if (total > 0x7fffffff) return cudaErrorInvalidConfiguration;
-    const int grid = int(total);
+    const int grid = int(total), threads = L.threads > 0 && mode == 0 ? L.threads : kEdgeThreads;
     // the initialisation runs once: one variant, which handles a hole and
     // reads the scheme
     if (mode == 1)
-        edge_tile_kernel<TS, TC, UT, 1, true, false><<<grid, kEdgeThreads, 0, s>>>(L, I);
+        edge_tile_kernel<TS, TC, UT, 1, true, false><<<grid, threads, 0, s>>>(L, I);
     else if (xj)
-        edge_tile_kernel<TS, TC, UT, 0, true, true><<<grid, kEdgeThreads, 0, s>>>(L, I);
+        edge_tile_kernel<TS, TC, UT, 0, true, true><<<grid, threads, 0, s>>>(L, I);
     else if (holed)
-        edge_tile_kernel<TS, TC, UT, 0, true, false><<<grid, kEdgeThreads, 0, s>>>(L, I);
+        edge_tile_kernel<TS, TC, UT, 0, true, false><<<grid, threads, 0, s>>>(L, I);
     else
-        edge_tile_kernel<TS, TC, UT, 0, false, false><<<grid, kEdgeThreads, 0, s>>>(L, I);
+        edge_tile_kernel<TS, TC, UT, 0, false, false><<<grid, threads, 0, s>>>(L, I);
     return cudaGetLastError();
 }
 
@@ -117,21 +119,21 @@ cudaError_t launch_edge_images(int fmt, const EdgeLaunch& L, int n_edge, const I
     return launch_edge_fmt(fmt, L, n_edge, img, n_img, s, 0, holed, xj);
 }
 
-// Tiles of one rectangle for CTAs of nthreads threads.  A band at most 3
+// Tiles of one rectangle for CTAs of shape.threads threads.  A band at most 3
 // nodes thick gets tiles exactly as thick (th = thickness + 4 rows of
 // threads, 2 fewer for each side on a bounded edge of the body, where the
-// halo would lie outside it; tw = nthreads / th columns), so few threads
-// compute halo only; a larger rectangle gets wide tiles (32 x 8 threads for
-// 256, 16 x 8 for 128).  Every tile has the full extent min(rectangle, tile)
-// along both axes (the last one of a row or column is shifted back,
-// recomputing its neighbour's nodes bit for bit), so each output node on a
-// bounded edge (bodies and bands are at least 2 nodes thick) finds the Q of
-// its two inward neighbours, which stage B computes for the output nodes and
-// their 1-node ring, inside the tile.  Returns the number of tiles (written
-// to out, at most cap, when out is not NULL).
-int edge_tiles_of_rect(const int rect[4], int inst, EdgeTile* out, int cap, bool lead_first, int nthreads,
+// halo would lie outside it; tw = threads / th columns), so few threads
+// compute halo only; a larger rectangle gets tiles of the shape.  Every tile
+// has the full extent min(rectangle, tile) along both axes (the last one of a
+// row or column is shifted back, recomputing its neighbour's nodes bit for
+// bit), so each output node on a bounded edge (bodies and bands are at least
+// 2 nodes thick) finds the Q of its two inward neighbours, which stage B
+// computes for the output nodes and their 1-node ring, inside the tile.
+// Returns the number of tiles (written to out, at most cap, when out is not
+// NULL).
+int edge_tiles_of_rect(const int rect[4], int inst, EdgeTile* out, int cap, bool lead_first, EdgeShape shape,
                        unsigned bounded) {
-    const int w = rect[1] - rect[0], h = rect[3] - rect[2];
+    const int w = rect[1] - rect[0], h = rect[3] - rect[2], nthreads = shape.threads;
     if (w <= 0 || h <= 0 || nthreads < 128) return 0;
     int tw, th, hx = 2, hy = 2, ow, oh;
     if (h <= 3) {
@@ -147,7 +149,7 @@ int edge_tiles_of_rect(const int rect[4], int inst, EdgeTile* out, int cap, bool
         ow = w;
         oh = th - 4;
     } else {
-        th = 8;
+        th = shape.th;
         tw = nthreads / th >= 32 ? 32 : nthreads / th;
         ow = tw - 4;
         oh = th - 4;
@@ -169,6 +171,7 @@ int edge_tiles_of_rect(const int rect[4], int inst, EdgeTile* out, int cap, bool
                 e.hx = uint8_t(hx);
                 e.hy = uint8_t(hy);
                 e.lead = int16_t(lead_first && n == 0);
+                e.inv_tw = uint16_t((65536 + tw - 1) / tw);
             }
             ++n;
         }

@@ -21,6 +21,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "lbm_device.cuh"
 #include "lbm_kernels.h"
 #include "lbm_pipeline.cuh"
@@ -37,10 +39,17 @@ __device__ __noinline__ void store_img_slow(T* base, Geo g, int x, int y, T v) {
     store_img(base, g, x, y, v);
 }
 
-template <class TC>
-struct Pops {
-    TC v[9];
-};
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return fma(a, b, c); }
+// -fci + w x, w twice a lattice weight: wmul's product for FP32 storage, else
+// one FMA.
+template <class TS, class TC>
+__device__ __forceinline__ TC back_value(TC fci, TC w, TC x) {
+    if constexpr (std::is_same<TS, float>::value)
+        return -fci + wmul<TS>(w, x);
+    else
+        return fma_rn(w, x, -fci);
+}
 
 // Eq. (abbcon) for link i with the node's post-collision population fci
 // across a wall of outward normal (sx, sy) inv_len (inv_len = 1/sqrt(2) at a
@@ -60,83 +69,160 @@ __device__ __forceinline__ TC abb_value(int i, TC fci, int sx, int sy, TC inv_le
     const TC sxx = pnn * N0 * N0 + TC(2) * pnt * N0 * t0 + ptt * t0 * t0;
     const TC syy = pnn * N1 * N1 + TC(2) * pnt * N1 * t1 + ptt * t1 * t1;
     const TC sxy = pnn * N0 * N1 + pnt * (N0 * t1 + t0 * N1) + ptt * t0 * t1;
-    return -fci + wmul<TS>(TC(2) * wgt<TC>(i), eq_even<TC>(i, r, sxx, sxy, syy));
+    return back_value<TS>(fci, TC(2) * wgt<TC>(i), eq_even<TC>(i, r, sxx, sxy, syy));
 }
 
-// Links of node (gx, gy) that leave the body through a bounded edge: the
-// boundary rules of Sec. 6, written into the first ghost row/column.  fc:
-// the node's post-collision populations; r, pxx, pxy, pyy: its moments;
-// q: its Q = P + Pbar.  HOLE: links may also enter a hole.
+// Stores a population that the boundary rules send back into the ghost cell
+// (x, y), and into its images on a body with a periodic axis.
+template <class T>
+__device__ __forceinline__ void store_back(T* base, const Geo& g, int x, int y, T v) {
+    if (g.perx || g.pery)
+        store_img_slow(base, g, x, y, v);
+    else
+        base[g.at(x, y)] = v;
+}
+
+// The links of node (gx, gy) through one wall of outward normal (SX, SY), an
+// edge of the body or a face of a hole: Eq. (bbcon) for a Dirichlet wall
+// (dirichlet; wall momentum jh* = rho0 v* / c), else Eq. (abbcon) with the
+// wall's traction.  fc: the node's post-collision populations; r, pxx, pyy:
+// its moments; q: its Q (11, 12, 21, 22).  lo, hi: whether the diagonal link
+// towards lower / higher coordinates along the wall leaves through this wall
+// alone.  Along an axis the wall's frame is the lattice's, so the Poisson
+// stress Pbar* of Sec. 6 is the quasi-traction and the tangential moment
+// themselves, formed once for the wall's three links: about 35 operations,
+// where the general form (abb_value) took 60 for each of them in a loop over
+// all eight directions.  The operations that remain are abb_value's, in its
+// order (what it adds and multiplies besides is exactly 0 and 1).
+template <int SX, int SY, class TS, class TC>
+__device__ __forceinline__ void wall_links(TS* fdst, const Geo& g, const StepParams& p, int gx, int gy, const TC* fc,
+                                           TC r, TC pxx, TC pyy, const TC* q, bool dirichlet, TC jh0, TC jh1, TC T0,
+                                           TC T1, TC inv_c2, bool lo, bool hi) {
+    constexpr int S = SX + SY;  // +-1
+    // the axis link and the diagonals towards lower and higher coordinates along the wall
+    constexpr int ia = SX > 0 ? 1 : (SX < 0 ? 3 : (SY > 0 ? 2 : 4));
+    constexpr int il = SX > 0 ? 8 : (SX < 0 ? 7 : (SY > 0 ? 6 : 7));
+    constexpr int ih = SX > 0 ? 5 : (SX < 0 ? 6 : (SY > 0 ? 5 : 8));
+    TC sxx, sxy, syy;
+    if (SX != 0) {
+        sxx = (TC(S) * (TC(S) * q[0] - T0)) * inv_c2;
+        sxy = (TC(S) * (TC(S) * q[2] - T1)) * inv_c2;
+        syy = pyy;
+    } else {
+        sxx = pxx;
+        sxy = (TC(S) * (TC(S) * q[1] - T0)) * inv_c2;
+        syy = (TC(S) * (TC(S) * q[3] - T1)) * inv_c2;
+    }
+    const TC tr = sxx + syy;
+    auto link = [&](auto I) {
+        constexpr int i = decltype(I)::value, oi = opp(i);
+        constexpr bool diag = i > 4;
+        TC val;
+        if (dirichlet) {
+            const TC e = TC(3) * (diag ? (TC(ex(i)) * jh0 + TC(ey(i)) * jh1) : TC(ex(i) + ey(i)) * (ex(i) != 0 ? jh0 : jh1));
+            val = back_value<TS>(-fc[i], -(TC(2) * wgt<TC>(i)), e);
+        } else {
+            const TC epe = diag ? tr + TC(2 * ex(i) * ey(i)) * sxy : (ex(i) != 0 ? sxx : syy);
+            const TC rterm = diag ? -r : TC(0.5) * r;
+            val = back_value<TS>(fc[i], TC(2) * wgt<TC>(i), fma_rn(TC(1.5), fma_rn(TC(3), epe, -tr), rterm));
+        }
+        store_back(fdst + oi * g.plane, g, gx + ex(i), gy + ey(i), Codec<TS, TC>::st(val, oi, p));
+    };
+    link(std::integral_constant<int, ia>());
+    if (lo) link(std::integral_constant<int, il>());
+    if (hi) link(std::integral_constant<int, ih>());
+}
+
+// The link i of node (gx, gy) through a corner: of two bounded edges of the
+// body, ea and eb (Eq. (bbcon) if either is Dirichlet, with the mean of their
+// wall momenta if both are, else Eq. (abbcon) with N = (N1 + N2)/sqrt(2), T* =
+// (T1 + T2)/sqrt(2)), or of the hole (two Neumann faces).
+template <class TS, class TC, class UT>
+__device__ __noinline__ void corner_link(TS* fdst, Geo g, const StepParams& p, const EdgeNow<TC, UT>* ea,
+                                         const EdgeNow<TC, UT>* eb, int i, int gx, int gy, TC fci, TC r, TC pxx, TC pxy,
+                                         TC pyy, TC q11, TC q12, TC q21, TC q22, TC T0, TC T1, TC inv_c2) {
+    const bool da = ea && ea->kind == kDirichlet, db = eb && eb->kind == kDirichlet;
+    TC val;
+    if (da || db) {
+        TC a0c, a1c;
+        if (da && db) {
+            a0c = TC(0.5) * (ea->jh[0] + eb->jh[0]);
+            a1c = TC(0.5) * (ea->jh[1] + eb->jh[1]);
+        } else {
+            const EdgeNow<TC, UT>* e = da ? ea : eb;
+            a0c = e->jh[0];
+            a1c = e->jh[1];
+        }
+        val = back_value<TS>(-fci, -(TC(2) * wgt<TC>(i)), eq_odd<TC>(i, a0c, a1c));
+    } else {
+        val = abb_value<TS, TC>(i, fci, ex(i), ey(i), TC(0.70710678118654752440), T0, T1, r, pxx, pxy, pyy, q11, q12,
+                                q21, q22, inv_c2);
+    }
+    const int oi = opp(i);
+    store_img(fdst + oi * g.plane, g, gx + ex(i), gy + ey(i), Codec<TS, TC>::st(val, oi, p));
+}
+
+// The boundary rules of Sec. 6 for a node on a bounded edge or next to the
+// hole, written into the ghost cells the links lead to.  edges: bits 0..3,
+// the node lies on x-, x+, y-, y+; faces: bits 0..3, next to the hole's face
+// at x0, x1, y0, y1; near_hole: within one node of the hole.  Out of line:
+// few nodes take it, and the tile's registers are spoken for.
+template <class TC>
+struct BackNode {
+    TC fc[9], r, pxx, pxy, pyy, q[4];
+};
 template <class TS, class TC, class UT, bool HOLE>
 __device__ __noinline__ void boundary_links(TS* fdst, Geo g, const StepParams& p, const EdgeNow<TC, UT>* s_edge,
-                                            int gx, int gy, Pops<TC> fc, TC r, TC pxx, TC pxy, TC pyy, TC q11,
-                                            TC q12, TC q21, TC q22, TC inv_c2) {
-    const int nx = g.nx, ny = g.ny;
+                                            int gx, int gy, unsigned edges, unsigned faces, bool near_hole,
+                                            BackNode<TC> n, TC inv_c2) {
+    const bool exl = edges & 1, exh = edges & 2, eyl = edges & 4, eyh = edges & 8;
+    auto edge = [&](auto SX, auto SY, int e, bool lo, bool hi) {
+        const EdgeNow<TC, UT>& w = s_edge[e];
+        wall_links<decltype(SX)::value, decltype(SY)::value, TS, TC>(fdst, g, p, gx, gy, n.fc, n.r, n.pxx, n.pyy, n.q,
+                                                                     w.kind == kDirichlet, w.jh[0], w.jh[1], w.T[0],
+                                                                     w.T[1], inv_c2, lo, hi);
+    };
+    using M1 = std::integral_constant<int, -1>;
+    using Z0 = std::integral_constant<int, 0>;
+    using P1 = std::integral_constant<int, 1>;
+    if (exl) edge(M1(), Z0(), 0, !eyl, !eyh);
+    if (exh) edge(P1(), Z0(), 1, !eyl, !eyh);
+    if (eyl) edge(Z0(), M1(), 2, !exl, !exh);
+    if (eyh) edge(Z0(), P1(), 3, !exl, !exh);
+    if (HOLE && near_hole) {
+        auto face = [&](auto SX, auto SY, int fa) {
+            constexpr int sx = decltype(SX)::value, sy = decltype(SY)::value;
+            const bool lo = in_hole(p.hole, gx + (sx != 0 ? sx : -1), gy + (sx != 0 ? -1 : sy));
+            const bool hi = in_hole(p.hole, gx + (sx != 0 ? sx : 1), gy + (sx != 0 ? 1 : sy));
+            wall_links<sx, sy, TS, TC>(fdst, g, p, gx, gy, n.fc, n.r, n.pxx, n.pyy, n.q, false, TC(0), TC(0),
+                                       TC(p.hole_T[2 * fa]), TC(p.hole_T[2 * fa + 1]), inv_c2, lo, hi);
+        };
+        if (faces & 1) face(P1(), Z0(), 0);  // entered along +x
+        if (faces & 2) face(M1(), Z0(), 1);
+        if (faces & 4) face(Z0(), P1(), 2);
+        if (faces & 8) face(Z0(), M1(), 3);
+    }
+    if (!((exl || exh) && (eyl || eyh)) && !(HOLE && near_hole)) return;
+    // the diagonal link through a corner of the body, or of the hole
 #pragma unroll 1
-    for (int i = 1; i < 9; ++i) {
-        const int dx = gx + ex(i), dy = gy + ey(i);
-        if (HOLE && in_hole(p.hole, dx, dy)) {
-            // Eq. (abbcon) across the face of the hole the link crosses, or
-            // both faces at the hole's corner
-            const bool cx = ex(i) != 0 && in_hole(p.hole, gx + ex(i), gy);
-            const bool cy = ey(i) != 0 && in_hole(p.hole, gx, gy + ey(i));
-            const int sx = (cx || !cy) ? ex(i) : 0, sy = (cy || !cx) ? ey(i) : 0;
-            TC T0 = TC(0), T1 = TC(0);
-            if (sx != 0) {  // the face at x0 (entered along +x) or at x1
-                const int fa = sx > 0 ? 0 : 1;
-                T0 += TC(p.hole_T[2 * fa]);
-                T1 += TC(p.hole_T[2 * fa + 1]);
-            }
-            if (sy != 0) {  // the face at y0 or at y1
-                const int fa = sy > 0 ? 2 : 3;
-                T0 += TC(p.hole_T[2 * fa]);
-                T1 += TC(p.hole_T[2 * fa + 1]);
-            }
-            const TC inv_len = (sx != 0 && sy != 0) ? TC(0.70710678118654752440) : TC(1);
-            const TC val =
-                abb_value<TS, TC>(i, fc.v[i], sx, sy, inv_len, T0, T1, r, pxx, pxy, pyy, q11, q12, q21, q22, inv_c2);
-            const int oi = opp(i);
-            store_img(fdst + oi * g.plane, g, dx, dy, Codec<TS, TC>::st(val, oi, p));
-            continue;
-        }
-        const bool bx2 = !g.perx && (dx < 0 || dx >= nx);
-        const bool by2 = !g.pery && (dy < 0 || dy >= ny);
-        if (!bx2 && !by2) continue;
-        const int oi = opp(i);
-        const EdgeNow<TC, UT>* ea = bx2 ? &s_edge[dx < 0 ? 0 : 1] : nullptr;
-        const EdgeNow<TC, UT>* eb = by2 ? &s_edge[dy < 0 ? 2 : 3] : nullptr;
-        const bool da = ea && ea->kind == kDirichlet, db = eb && eb->kind == kDirichlet;
-        TC val;
-        if (da || db) {
-            // Eq. (bbcon) with jh* = rho0 v* / c (averaged over the Dirichlet
-            // edges of a corner link)
-            TC a0c, a1c;
-            if (da && db) {
-                a0c = TC(0.5) * (ea->jh[0] + eb->jh[0]);
-                a1c = TC(0.5) * (ea->jh[1] + eb->jh[1]);
-            } else {
-                const EdgeNow<TC, UT>* e = da ? ea : eb;
-                a0c = e->jh[0];
-                a1c = e->jh[1];
-            }
-            val = fc.v[i] - wmul<TS>(TC(2) * wgt<TC>(i), eq_odd<TC>(i, a0c, a1c));
+    for (int i = 5; i < 9; ++i) {
+        const EdgeNow<TC, UT>*ea = nullptr, *eb = nullptr;
+        TC T0, T1;
+        if (HOLE && near_hole) {  // into the hole through neither of its faces alone
+            const int dx = gx + ex(i), dy = gy + ey(i);
+            if (!in_hole(p.hole, dx, dy) || in_hole(p.hole, dx, gy) || in_hole(p.hole, gx, dy)) continue;
+            const int fx = ex(i) > 0 ? 0 : 1, fy = ey(i) > 0 ? 2 : 3;
+            T0 = TC(p.hole_T[2 * fx]) + TC(p.hole_T[2 * fy]);
+            T1 = TC(p.hole_T[2 * fx + 1]) + TC(p.hole_T[2 * fy + 1]);
         } else {
-            // Eq. (abbcon) with Pbar* of Sec. 6 in the wall-normal frame; a
-            // corner link: N = (N1 + N2)/sqrt(2), T* = (T1 + T2)/sqrt(2)
-            const int sx = bx2 ? (dx < 0 ? -1 : 1) : 0, sy = by2 ? (dy < 0 ? -1 : 1) : 0;
-            const TC inv_len = (sx != 0 && sy != 0) ? TC(0.70710678118654752440) : TC(1);
-            TC T0 = TC(0), T1 = TC(0);
-            if (ea) {
-                T0 += ea->T[0];
-                T1 += ea->T[1];
-            }
-            if (eb) {
-                T0 += eb->T[0];
-                T1 += eb->T[1];
-            }
-            val = abb_value<TS, TC>(i, fc.v[i], sx, sy, inv_len, T0, T1, r, pxx, pxy, pyy, q11, q12, q21, q22, inv_c2);
+            if (!((ex(i) < 0 ? exl : exh) && (ey(i) < 0 ? eyl : eyh))) continue;
+            ea = &s_edge[ex(i) < 0 ? 0 : 1];
+            eb = &s_edge[ey(i) < 0 ? 2 : 3];
+            T0 = ea->T[0] + eb->T[0];
+            T1 = ea->T[1] + eb->T[1];
         }
-        store_img(fdst + oi * g.plane, g, dx, dy, Codec<TS, TC>::st(val, oi, p));
+        corner_link<TS, TC, UT>(fdst, g, p, ea, eb, i, gx, gy, n.fc[i], n.r, n.pxx, n.pxy, n.pyy, n.q[0], n.q[1],
+                                n.q[2], n.q[3], T0, T1, inv_c2);
     }
 }
 
@@ -153,7 +239,8 @@ __device__ __forceinline__ bool moderate(double a, double b, double c, double d)
 
 // The tile `tile` of the body whose parameters are p (mode 0: one time step;
 // mode 1: the initialisation).  Every thread of the CTA calls it (threads
-// beyond tw x th idle through the barriers).  Shared memory: su holds 2 x
+// beyond tw x th idle through the barriers; t / tw by tile.inv_tw = ceil(2^16
+// / tw), exact for t tw < 2^16).  Shared memory: su holds 2 x
 // tw x th u-carry values, sq 4 x tw x th arithmetic values, sinit (mode 1)
 // 4 x tw x th, s_edge the boundary data of the 4 edges and of a hole's faces
 // (5 entries).  want_fields: also write u, v, r to p.fields.  HOLE: the
@@ -195,14 +282,15 @@ __device__ __forceinline__ void edge_tile_body(const EdgeTile& tile, const StepP
     // ---- this thread's node: raw coordinates (an image beyond a periodic
     // seam) and node coordinates
     const int tw = tile.tw, th = tile.th;
-    const int tx = t % tw, ty = t / tw;  // ty >= th: an idle thread
+    const int ty = (t * int(tile.inv_tw)) >> 16, tx = t - ty * tw;  // ty >= th: an idle thread
     const int nxo = tile.x1 - tile.x0, nyo = tile.y1 - tile.y0;  // output extent
     const int hx = tile.hx, hy = tile.hy;  // halo before the output nodes
     const int gxr = tile.x0 - hx + tx, gyr = tile.y0 - hy + ty;
     const bool okx = g.perx ? (gxr >= -2 && gxr < nx + 2) : (gxr >= 0 && gxr < nx);
     const bool oky = g.pery ? (gyr >= -2 && gyr < ny + 2) : (gyr >= 0 && gyr < ny);
-    const int gx = g.perx ? wrap_coord(gxr, nx) : gxr;
-    const int gy = g.pery ? wrap_coord(gyr, ny) : gyr;
+    // (an image is at most 2 beyond the seam, and an axis has 3 nodes or more)
+    const int gx = !g.perx ? gxr : (gxr < 0 ? gxr + nx : (gxr >= nx ? gxr - nx : gxr));
+    const int gy = !g.pery ? gyr : (gyr < 0 ? gyr + ny : (gyr >= ny ? gyr - ny : gyr));
     // a node of the hole is not part of the body: it holds nothing, and the
     // cells of the hole next to its faces receive the populations the
     // anti-bounce-back rule sends back
@@ -445,11 +533,20 @@ __device__ __forceinline__ void edge_tile_body(const EdgeTile& tile, const StepP
         // links that leave the body through a bounded edge or enter the hole
         if (gxl || gxh || gyl || gyh || near_hole) {
             const TC* qr = sq + (ty * 4) * tw + tx;
-            Pops<TC> pc;
+            BackNode<TC> n;
 #pragma unroll
-            for (int i = 0; i < 9; ++i) pc.v[i] = fc[i];
-            boundary_links<TS, TC, UT, HOLE>(fdst, g, p, s_edge, gx, gy, pc, r, pxx, pxy, pyy, qr[0], qr[tw], qr[2 * tw],
-                                       qr[3 * tw], k.inv_c2);
+            for (int i = 0; i < 9; ++i) n.fc[i] = fc[i];
+            n.r = r;
+            n.pxx = pxx;
+            n.pxy = pxy;
+            n.pyy = pyy;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) n.q[c] = qr[c * tw];
+            // the body's edges (a node next to the hole is next to none), the hole's faces
+            const unsigned edges = unsigned(gxl && !hxl) | unsigned(gxh && !hxh) << 1 | unsigned(gyl && !hyl) << 2 |
+                                   unsigned(gyh && !hyh) << 3;
+            const unsigned faces = unsigned(hxh) | unsigned(hxl) << 1 | unsigned(hyh) << 2 | unsigned(hyl) << 3;
+            boundary_links<TS, TC, UT, HOLE>(fdst, g, p, s_edge, gx, gy, edges, faces, HOLE && near_hole, n, k.inv_c2);
         }
 
         // carries for the next step: A' = u + ku (jh + s/2), u = u* + du;

@@ -117,7 +117,15 @@ struct EdgeTile {
     uint8_t tw, th;  // threads along x and y
     uint8_t hx, hy;  // halo nodes before the first output node (2, or 0 on a bounded edge)
     int16_t lead;    // this tile advances the instance's step counter
+    uint16_t inv_tw; // ceil(2^16 / tw)
 };
+
+// Tiles over rectangles more than 3 nodes thick: th rows of min(32, threads /
+// th) threads (a band takes tiles exactly as thick, of `threads` threads).
+struct EdgeShape {
+    int threads, th;
+};
+constexpr EdgeShape kEdgeWide = {kEdgeThreads, 8};  // 28 x 4 output nodes
 
 struct EdgeLaunch {
     const StepParams* params;  // device table, indexed by EdgeTile::inst
@@ -125,6 +133,8 @@ struct EdgeLaunch {
     int32_t fields;            // also write u, v, r to params.fields
     int32_t rtiles_x;          // implicit grid: tiles per row of rect
     int32_t rect[4];           // implicit grid: x_lo, x_hi, y_lo, y_hi
+    int32_t threads;           // of a CTA; 0: kEdgeThreads
+    int32_t pad;
 };
 
 // One step (mode 0) or the initialisation (mode 1) over ntiles tiles.
@@ -132,11 +142,11 @@ struct EdgeLaunch {
 // initialisation reads the scheme from the parameters).
 cudaError_t launch_edge(int fmt, const EdgeLaunch& L, int ntiles, cudaStream_t s, int mode, bool holed, bool xj);
 
-// Tiles of one band rectangle for CTAs of `nthreads` threads (kEdgeThreads
-// for the edge kernel); count only when out is NULL.  bounded: the sides of
-// rect that lie on a bounded edge of the body (bit 0: x low, 1: x high,
-// 2: y low, 3: y high), beyond which a band's tiles need no halo.
-int edge_tiles_of_rect(const int rect[4], int inst, EdgeTile* out, int cap, bool lead_first, int nthreads,
+// Tiles of one rectangle in the given shape; count only when out is NULL.
+// bounded: the sides of rect that lie on a bounded edge of the body (bit 0: x
+// low, 1: x high, 2: y low, 3: y high), beyond which a band's tiles need no
+// halo.
+int edge_tiles_of_rect(const int rect[4], int inst, EdgeTile* out, int cap, bool lead_first, EdgeShape shape,
                        unsigned bounded);
 
 // Read-out parameters: stresses from the FP64 displacement field.
