@@ -29,9 +29,16 @@ static_assert(sizeof(StepParams) % 16 == 0, "StepParams is copied to shared memo
 template <class TS, class TC, class UT, int MODE, bool HOLE, bool XJ>
 __global__ void __launch_bounds__(kEdgeThreads, sizeof(TC) == 8 ? 2 : 3)
     edge_tile_kernel(const __grid_constant__ EdgeLaunch L, const __grid_constant__ ImageLaunch I) {
+    // the next launch may start; in FP64 only once this one is done, so that
+    // its tiles find the SMs free (started early, two of them share an SM's
+    // FP64 units while others idle: 64 x 64 in 12.8 us a step, 6.7 so, 8.0
+    // without the overlap)
+    constexpr bool early = sizeof(TC) == 4;
+    if (early) grid_launch_dependents();
     constexpr int N = kEdgeThreads;
     static_assert(kImageThreads <= N, "an image tile fits an edge CTA");
     if (I.tiles != nullptr && int(blockIdx.x) >= I.n_edge) {  // a seam-image CTA (uniform per CTA)
+        grid_wait();
         if (int(threadIdx.x) < kImageThreads)
             image_copy<int(sizeof(TS)), int(sizeof(TC)), UT::layout>(L.params, I.tiles[blockIdx.x - I.n_edge],
                                                                     int(threadIdx.x));
@@ -70,6 +77,7 @@ __global__ void __launch_bounds__(kEdgeThreads, sizeof(TC) == 8 ? 2 : 3)
     __syncthreads();
     edge_tile_body<TS, TC, UT, MODE, HOLE, XJ>(tile, sp, L.fields != 0, su, sq, MODE == 1 ? sinit : nullptr,
                                                 s_edge);
+    if (!early) grid_launch_dependents();
 }
 
 // ---------------------------------------------------------------- launchers
@@ -83,18 +91,25 @@ cudaError_t launch_edge_t(const EdgeLaunch& L, int ntiles, const ImageTile* img,
     const int64_t total = int64_t(ntiles) + n_img;
     if (total <= 0) return cudaSuccess;
     if (total > 0x7fffffff) return cudaErrorInvalidConfiguration;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = mode == 0 && L.chain ? 1 : 0;
     const int grid = int(total), threads = L.threads > 0 && mode == 0 ? L.threads : kEdgeThreads;
+    cfg.gridDim = dim3(unsigned(grid));
+    cfg.blockDim = dim3(unsigned(threads));
     // the initialisation runs once: one variant, which handles a hole and
     // reads the scheme
     if (mode == 1)
-        edge_tile_kernel<TS, TC, UT, 1, true, false><<<grid, threads, 0, s>>>(L, I);
-    else if (xj)
-        edge_tile_kernel<TS, TC, UT, 0, true, true><<<grid, threads, 0, s>>>(L, I);
-    else if (holed)
-        edge_tile_kernel<TS, TC, UT, 0, true, false><<<grid, threads, 0, s>>>(L, I);
-    else
-        edge_tile_kernel<TS, TC, UT, 0, false, false><<<grid, threads, 0, s>>>(L, I);
-    return cudaGetLastError();
+        return cudaLaunchKernelEx(&cfg, edge_tile_kernel<TS, TC, UT, 1, true, false>, L, I);
+    if (xj)
+        return cudaLaunchKernelEx(&cfg, edge_tile_kernel<TS, TC, UT, 0, true, true>, L, I);
+    if (holed)
+        return cudaLaunchKernelEx(&cfg, edge_tile_kernel<TS, TC, UT, 0, true, false>, L, I);
+    return cudaLaunchKernelEx(&cfg, edge_tile_kernel<TS, TC, UT, 0, false, false>, L, I);
 }
 
 static cudaError_t launch_edge_fmt(int fmt, const EdgeLaunch& L, int ntiles, const ImageTile* img, int n_img,

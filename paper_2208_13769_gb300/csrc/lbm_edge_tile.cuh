@@ -253,9 +253,14 @@ __device__ __forceinline__ void edge_tile_body(const EdgeTile& tile, const StepP
                                                TC* sq, TC* sinit, EdgeNow<TC, UT>* s_edge) {
     const int t = threadIdx.x;
 
+    // boundary data that do not depend on the time, while the previous launch
+    // still runs (their FP64 operations take longer than a memory round trip)
+    if (t < 4 && p.bc[t].steady) edge_now<TC, UT>(s_edge[t], p.bc[t], 0.0, p.lat_d[kLatRho0OverC]);
+
     // the collision of this launch is at t_now = n_now dt; the step counter
     // is read here and used once stage A has issued its loads, so that the
     // two memory round trips overlap
+    grid_wait();  // before the first read of what the previous step wrote
     int64_t n_now = 0;
     if (MODE == 0 && t < 4) n_now = p.counter[p.parity] + 1;
 
@@ -363,7 +368,8 @@ __device__ __forceinline__ void edge_tile_body(const EdgeTile& tile, const StepP
         su[(ty * 2 + 1) * tw + tx] = UT::from_double(p.u0 ? p.u0[hh + 1] : 0.0);
     }
     if (tile.lead && t == 0) p.counter[p.parity ^ 1] = n_now;
-    if (t < 4) edge_now<TC, UT>(s_edge[t], p.bc[t], double(n_now) * p.dt, p.lat_d[kLatRho0OverC]);
+    if (t < 4 && !p.bc[t].steady)
+        edge_now<TC, UT>(s_edge[t], p.bc[t], double(n_now) * p.dt, p.lat_d[kLatRho0OverC]);
     if (HOLE && t == 4) s_edge[4].kind = kNeumann;  // the faces of a hole (only the kind is read)
     __syncthreads();
 

@@ -134,7 +134,7 @@ struct EdgeLaunch {
     int32_t rtiles_x;          // implicit grid: tiles per row of rect
     int32_t rect[4];           // implicit grid: x_lo, x_hi, y_lo, y_hi
     int32_t threads;           // of a CTA; 0: kEdgeThreads
-    int32_t pad;
+    int32_t chain;             // mode 0: overlap the launch with the end of the stream's previous kernel
 };
 
 // One step (mode 0) or the initialisation (mode 1) over ntiles tiles.

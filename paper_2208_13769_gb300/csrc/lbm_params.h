@@ -22,7 +22,7 @@ constexpr int kPadCols = 8;
 // One edge (0 = x-, 1 = x+, 2 = y-, 3 = y+) of Sec. 6's boundary value problem.
 struct EdgeBC {
     int32_t kind;
-    int32_t pad;
+    int32_t steady;   // its boundary data do not depend on the time
     double value[2];  // Dirichlet: u* at t = 0;  Neumann: T0
     double rate[2];   // Dirichlet: v*;           Neumann: T1
     double times[3];  // Neumann: t_on, t_ramp, t_off

@@ -72,6 +72,12 @@ __device__ __forceinline__ void acquire_tensor_map(const void* map) {
     asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(map) : "memory");
 }
 
+// A launch chained to its predecessor (programmatic stream serialization):
+// lets the next one's CTAs start, and waits until the previous one is
+// complete and its writes are visible.  Both do nothing in other launches.
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // T*(t) of a Neumann edge: T0 outside [t_on, t_off), ramping to T1 over t_ramp.
 __device__ __forceinline__ void traction(const EdgeBC& e, double t, double& tx, double& ty) {
     double s;
