@@ -206,8 +206,9 @@ LBM_API lbm_status lbm_profile_interior(lbm_ctx* ctx, int64_t nlaunches, double 
 typedef struct {
     int32_t ring_slots; /* rows of the interior kernel's pipeline in flight or in work, 4..8; 0:
                            default (4) */
-    int32_t chunk_rows; /* rows per CTA, >= 8; 0: one wave of CTAs over the SMs, at least 8 rows
-                           each, of a large body with shorter chunks after it (default) */
+    int32_t chunk_rows; /* rows per CTA, >= 8; 0: one wave of CTAs over the SMs, with shorter
+                           chunks after it on a large body; on a body of less than about 10
+                           rows each the 4 to 12 rows that take least time (default) */
     int32_t aligned;    /* 1: the fewest strips of equal width on 32-byte sector boundaries (at
                            most 120 columns; 112 for 16-bit storage); 2: the same on 16-byte
                            boundaries (at most 124 columns; 120 for 16-bit storage);

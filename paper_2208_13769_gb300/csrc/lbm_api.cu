@@ -277,25 +277,54 @@ static EdgeShape edge_shape(const lbm_ctx* c) {
     return best;
 }
 
-// Rows per CTA of one wave (`wave` CTAs per strip), at least 8 (shorter tiles
-// of mid-size bodies cut the row pipeline's latency: 512 x 512 FP32 in 13 us
-// a step with 8-row tiles against 15 us with 16).
-static int one_wave_rows(int h, int64_t wave) { return int(std::max<int64_t>((h + wave - 1) / wave, 8)); }
+// Rows per CTA where one wave would give each few: a tile of r rows takes
+// about r + 4 iterations of its row pipeline (4 fill it), each of which lasts
+// as long as its chain of waits and barriers while an SM holds up to 2 CTAs,
+// then longer (they share its issue slots), and half as long again from about
+// 4.5 on.  `load` is the full-width CTAs per SM that 1-row tiles would make.
+// Measured (FP16 / FP32 us a step, with at least 8 rows and so): 420 x 400 12.6
+// / 13.2 and 9.4 / 10.0 (4 rows), 512 x 512 13.1 / 13.1 and 11.2 / 11.6 (4),
+// 600 x 600 13.2 / 14.2 (8 either way), 800 x 700 16.4 / 17.4 and 15.6 / 16.4
+// (7), 1000 x 777 22.1 / 24.5 and 20.3 / 21.1 (10).
+static int short_rows(double load) {
+    int best = 8;
+    double least = INFINITY;
+    for (int r = 4; r <= 12; ++r) {
+        const double x = load / r;
+        const double g = x <= 2.0   ? 0.72
+                         : x <= 3.0 ? 0.72 + 0.25 * (x - 2.0)
+                         : x <= 4.3 ? 0.97 + 0.14 * (x - 3.0)
+                         : x <= 4.8 ? 1.15 + (x - 4.3)
+                                    : 1.65 * x / 4.8;
+        if ((r + 4) * g < least) {
+            least = (r + 4) * g;
+            best = r;
+        }
+    }
+    return best;
+}
+
+// Rows per CTA of a rectangle of w x h nodes for a wave of `wave` CTAs per
+// strip on `sms` SMs.
+static int one_wave_rows(int fmt, int w, int h, int64_t wave, double sms) {
+    const int one = int((h + wave - 1) / wave);
+    if (fmt == kFmtF64) return std::max(one, 8);
+    return one > 10 ? one : short_rows(double(w) * h / (kInteriorThreads - 4) / std::max(1.0, sms));
+}
 
 // The chunks of h rows.  One wave of equal chunks leaves SMs idle at the end:
 // they do not run equally fast (at 4096 x 2048 in FP32 they were busy for 72
 // to 100 % of the launch, 85 % on average), so a long wave gets most of the
 // rows, and shorter chunks, taken as SMs become free, the rest.  4-byte
-// storage at 4096 x 2048: 188 us a step in one wave, 163 with 65 % of the rows
-// in it, then chunks of a quarter and an eighth of its rows; 3000 x 1500: 106
-// and 93; at 1536 x 1536 (22 rows per CTA) 55.8 and 56.7, so below 24 rows one
-// wave stays.  16-bit storage waits less for memory and its SMs keep together:
+// storage at 4096 x 2048: 190 us a step in one wave, 163 with 75 % of the rows
+// in it, then chunks of a quarter and an eighth of its rows (164 with 65 % at
+// some sizes, 168 with 85 %); 2200 x 1800: 91.7 and 86.0; at 1536 x 1536 (22
+// rows per CTA) 55.8 and 56.7, so below 24 rows one wave stays.  16-bit storage waits less for memory and its SMs keep together:
 // 136 us in one wave, 131 with 90 % in it; at 2500 x 1300 60.9 either way.
 // FP64 is bound by its arithmetic (1500 x 1000: 506 us, 507 in levels).
-static ChunkLevels chunk_levels(int fmt, int h, int64_t wave, int tune_chunk, int max_rows) {
+static ChunkLevels chunk_levels(int fmt, int h, int one, int tune_chunk, int max_rows) {
     ChunkLevels L;
     memset(&L, 0, sizeof(L));
-    const int one = one_wave_rows(h, wave);
     const bool four = fmt != kFmtF64 && fmt != kFmtF16 && fmt != kFmtBF16;
     if (tune_chunk > 0 || fmt == kFmtF64 || one < (four ? 24 : 48) || one > max_rows) {
         L.rows[0] = std::min(tune_chunk > 0 ? tune_chunk : one, std::min(h, max_rows));
@@ -303,10 +332,10 @@ static ChunkLevels chunk_levels(int fmt, int h, int64_t wave, int tune_chunk, in
         return L;
     }
     const int n = (h + one - 1) / one;
-    L.rows[0] = std::max(8, int(int64_t(h) * (four ? 65 : 90) / (100 * int64_t(n))));
+    L.rows[0] = std::max(8, int(int64_t(h) * (four ? 75 : 90) / (100 * int64_t(n))));
     L.count[0] = n;
     L.rows[1] = std::max(8, one / 4);
-    L.count[1] = four ? int(int64_t(h) * 22 / (100 * int64_t(L.rows[1]))) : 0;
+    L.count[1] = four ? int(int64_t(h) * 15 / (100 * int64_t(L.rows[1]))) : 0;
     L.rows[2] = std::max(8, one / 8);
     const int left = h - n * L.rows[0] - L.count[1] * L.rows[1];
     L.count[2] = std::max(0, (left + L.rows[2] - 1) / L.rows[2]);
@@ -331,6 +360,8 @@ static cudaError_t build_plan(lbm_ctx* c) {
     const bool seams_inside = c->tune_plan == 2;
     plan_rects(c, edge_only, seams_inside, c->irect, &c->n_irect, c->brect, &c->nband);
     const bool hole = c->hole[0] < c->hole[1];
+    const bool perx = c->bc[0].kind == kPeriodic, pery = c->bc[2].kind == kPeriodic;
+    bool levels = false;  // shorter chunks after the interior's wave
     if (c->n_irect > 0) {
         c->i_ring = c->tune_ring ? c->tune_ring : kInteriorRing;
         const int per_sm = std::max(1, interior_occupancy(c->fmt, c->i_ring));
@@ -347,17 +378,17 @@ static cudaError_t build_plan(lbm_ctx* c) {
             // strips on sector boundaries for 4-byte storage where a CTA has
             // rows enough that its neighbours run apart in time (1536 x 1536:
             // 55.8 us a step, 57.4 without; 2000 x 1500: 72.1 and 75.1)
-            interior_strips(c->fmt, r[0], r[1], 0, &c->i_strip_x0[q], &c->i_strip_w[q], &strips[q]);
-            const bool four = elem_size_storage(c->fmt) == 4;
-            const int aligned = c->tune_aligned >= 0 ? c->tune_aligned
-                                : four && one_wave_rows(h, std::max<int64_t>(1, share / strips[q])) >= 16 ? 1
-                                                                                                         : 0;
-            if (aligned > 0)
+            auto rows_per_cta = [&](int aligned) {
                 interior_strips(c->fmt, r[0], r[1], aligned, &c->i_strip_x0[q], &c->i_strip_w[q], &strips[q]);
+                return one_wave_rows(c->fmt, r[1] - r[0], h, std::max<int64_t>(1, share / strips[q]),
+                                     double(c->num_sms) * double(share) / double(slots));
+            };
+            int aligned = std::max(0, c->tune_aligned), one = rows_per_cta(aligned);
+            if (c->tune_aligned < 0 && elem_size_storage(c->fmt) == 4 && one >= 16) one = rows_per_cta(aligned = 1);
             if (q == 0) c->i_aligned = aligned;
-            lev[q] = chunk_levels(c->fmt, h, std::max<int64_t>(1, share / strips[q]), c->tune_chunk,
-                                  interior_max_rows(c->fmt, c->pitch));
+            lev[q] = chunk_levels(c->fmt, h, one, c->tune_chunk, interior_max_rows(c->fmt, c->pitch));
             c->i_chunk[q] = lev[q].rows[0];
+            levels |= lev[q].count[1] + lev[q].count[2] > 0;
             nitems += interior_items(r, q, strips[q], lev[q], nullptr, 0);
         }
         if (nitems > INT32_MAX - 1) return cudaErrorInvalidConfiguration;
@@ -384,7 +415,17 @@ static cudaError_t build_plan(lbm_ctx* c) {
                                       c->plane, c->ny, &c->maps[q]);
         if (e != cudaSuccess) return e;
     }
-    c->edge_shape = c->has_interior ? kEdgeWide : edge_shape(c);
+    // edge tiles beside an interior: CTAs of an interior tile's size, each in
+    // the place of one, for the many band tiles of seams and holes beside short
+    // interior tiles (FP32 800 x 600 with a periodic axis 19.3 to 16.0 us a
+    // step, 1000 x 1000 with a hole 31.2 to 27.4) and where 4-byte storage keeps
+    // every place taken with shorter chunks (4096 x 2048 173.0 to 171.5); else
+    // wide ones, which compute less halo (800 x 700 16.0, 16.8 with small ones;
+    // FP16 2600 x 2400 with a hole 97 and 99).  So too in the launch that the
+    // image tiles share, whose CTAs are wide.
+    const bool crowded =
+        (levels && elem_size_storage(c->fmt) == 4) || (c->i_chunk[0] <= 12 && (perx || pery || hole));
+    c->edge_shape = !c->has_interior ? edge_shape(c) : crowded && !seams_inside ? kEdgeInterior : kEdgeWide;
     int n = 0;
     for (int b = 0; b < c->nband; ++b)
         n += edge_tiles_of_rect(c->brect[b], 0, nullptr, 0, false, c->edge_shape, bounded_sides(c, c->brect[b]));
@@ -401,7 +442,6 @@ static cudaError_t build_plan(lbm_ctx* c) {
         for (int q = 0; q < c->n_irect; ++q)
             m += edge_tiles_of_rect(c->irect[q], 0, h + m, ni - m, false, c->edge_shape, 0);
     // the images of the interior's nodes next to a periodic seam
-    const bool perx = c->bc[0].kind == kPeriodic, pery = c->bc[2].kind == kPeriodic;
     int nimg = 0;
     ImageTile* himg = nullptr;
     if (c->has_interior && seams_inside && (perx || pery)) {

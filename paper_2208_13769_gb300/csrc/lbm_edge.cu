@@ -98,7 +98,8 @@ cudaError_t launch_edge_t(const EdgeLaunch& L, int ntiles, const ImageTile* img,
     cfg.stream = s;
     cfg.attrs = at;
     cfg.numAttrs = mode == 0 && L.chain ? 1 : 0;
-    const int grid = int(total), threads = L.threads > 0 && mode == 0 ? L.threads : kEdgeThreads;
+    // (an image tile takes the threads of a wide edge tile)
+    const int grid = int(total), threads = L.threads > 0 && mode == 0 && n_img == 0 ? L.threads : kEdgeThreads;
     cfg.gridDim = dim3(unsigned(grid));
     cfg.blockDim = dim3(unsigned(threads));
     // the initialisation runs once: one variant, which handles a hole and

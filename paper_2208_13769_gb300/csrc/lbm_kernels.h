@@ -125,7 +125,8 @@ struct EdgeTile {
 struct EdgeShape {
     int threads, th;
 };
-constexpr EdgeShape kEdgeWide = {kEdgeThreads, 8};  // 28 x 4 output nodes
+constexpr EdgeShape kEdgeWide = {kEdgeThreads, 8};          // 28 x 4 output nodes
+constexpr EdgeShape kEdgeInterior = {kInteriorThreads, 8};  // CTAs of an interior tile's size: 12 x 4
 
 struct EdgeLaunch {
     const StepParams* params;  // device table, indexed by EdgeTile::inst
