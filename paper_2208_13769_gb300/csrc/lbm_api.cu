@@ -289,7 +289,7 @@ static EdgeShape edge_shape(const lbm_ctx* c) {
 static int short_rows(double load) {
     int best = 8;
     double least = INFINITY;
-    for (int r = 4; r <= 12; ++r) {
+    for (int r = 4; r <= 16; ++r) {
         const double x = load / r;
         const double g = x <= 2.0   ? 0.72
                          : x <= 3.0 ? 0.72 + 0.25 * (x - 2.0)
@@ -304,12 +304,32 @@ static int short_rows(double load) {
     return best;
 }
 
-// Rows per CTA of a rectangle of w x h nodes for a wave of `wave` CTAs per
-// strip on `sms` SMs.
-static int one_wave_rows(int fmt, int w, int h, int64_t wave, double sms) {
-    const int one = int((h + wave - 1) / wave);
-    if (fmt == kFmtF64) return std::max(one, 8);
-    return one > 10 ? one : short_rows(double(w) * h / (kInteriorThreads - 4) / std::max(1.0, sms));
+// The wave of a rectangle of w x h nodes in `strips` strips: rows per CTA for
+// at most `share` CTAs on `sms` SMs, and whether it is long enough for shorter
+// chunks after it (ChunkLevels).  A wave of 4-byte storage that is not takes
+// 4.45 CTAs per SM instead of the 6 or 7 that fit: memory is as busy with them,
+// and on the SMs that hold 4 the edge tiles run from the start instead of
+// after the first interior tiles end (FP32 pair / lo16 / plain us a step, full
+// and so: 1400 x 900 34.8 / 34.1 / 28.7 and 31.1 / 31.2 / 27.5, 1700 x 1438
+// 62.2 / 60.1 / 53.7 and 61.4 / 57.2 / 50.1; 2000 x 1500, 29 rows in the full
+// wave, 69.4 / 66.4 in levels and 73.9 / 68.7 so).  FP16 at 1400 x 900: 29.4
+// and 29.6.
+struct Wave {
+    int rows;
+    bool levels;
+};
+
+static Wave interior_wave(int fmt, int w, int h, int strips, int64_t share, double sms) {
+    auto rows = [&](int64_t ctas) {
+        const int64_t per = std::max<int64_t>(1, ctas / strips);
+        return int((h + per - 1) / per);
+    };
+    const int one = rows(share);
+    const bool four = elem_size_storage(fmt) == 4;
+    if (fmt == kFmtF64) return {std::max(one, 8), false};
+    if (one <= 10) return {short_rows(double(w) * h / (kInteriorThreads - 4) / std::max(1.0, sms)), false};
+    if (one >= (four ? 28 : 48)) return {one, true};
+    return {four ? rows(std::min(share, int64_t(4.45 * sms))) : one, false};
 }
 
 // The chunks of h rows.  One wave of equal chunks leaves SMs idle at the end:
@@ -319,14 +339,15 @@ static int one_wave_rows(int fmt, int w, int h, int64_t wave, double sms) {
 // storage at 4096 x 2048: 190 us a step in one wave, 163 with 75 % of the rows
 // in it, then chunks of a quarter and an eighth of its rows (164 with 65 % at
 // some sizes, 168 with 85 %); 2200 x 1800: 91.7 and 86.0; at 1536 x 1536 (22
-// rows per CTA) 55.8 and 56.7, so below 24 rows one wave stays.  16-bit storage waits less for memory and its SMs keep together:
-// 136 us in one wave, 131 with 90 % in it; at 2500 x 1300 60.9 either way.
+// rows per CTA) 55.8 and 56.7, so a shorter wave stays one.  16-bit storage
+// waits less for memory and its SMs keep together: 136 us in one wave, 131 with 90 % in it; at 2500 x 1300 60.9 either way.
 // FP64 is bound by its arithmetic (1500 x 1000: 506 us, 507 in levels).
-static ChunkLevels chunk_levels(int fmt, int h, int one, int tune_chunk, int max_rows) {
+static ChunkLevels chunk_levels(int fmt, int h, Wave wave, int tune_chunk, int max_rows) {
     ChunkLevels L;
     memset(&L, 0, sizeof(L));
-    const bool four = fmt != kFmtF64 && fmt != kFmtF16 && fmt != kFmtBF16;
-    if (tune_chunk > 0 || fmt == kFmtF64 || one < (four ? 24 : 48) || one > max_rows) {
+    const int one = wave.rows;
+    const bool four = elem_size_storage(fmt) == 4;
+    if (tune_chunk > 0 || !wave.levels || one > max_rows) {
         L.rows[0] = std::min(tune_chunk > 0 ? tune_chunk : one, std::min(h, max_rows));
         L.count[0] = (h + L.rows[0] - 1) / L.rows[0];
         return L;
@@ -378,15 +399,16 @@ static cudaError_t build_plan(lbm_ctx* c) {
             // strips on sector boundaries for 4-byte storage where a CTA has
             // rows enough that its neighbours run apart in time (1536 x 1536:
             // 55.8 us a step, 57.4 without; 2000 x 1500: 72.1 and 75.1)
-            auto rows_per_cta = [&](int aligned) {
+            auto wave_of = [&](int aligned) {
                 interior_strips(c->fmt, r[0], r[1], aligned, &c->i_strip_x0[q], &c->i_strip_w[q], &strips[q]);
-                return one_wave_rows(c->fmt, r[1] - r[0], h, std::max<int64_t>(1, share / strips[q]),
+                return interior_wave(c->fmt, r[1] - r[0], h, strips[q], share,
                                      double(c->num_sms) * double(share) / double(slots));
             };
-            int aligned = std::max(0, c->tune_aligned), one = rows_per_cta(aligned);
-            if (c->tune_aligned < 0 && elem_size_storage(c->fmt) == 4 && one >= 16) one = rows_per_cta(aligned = 1);
+            int aligned = std::max(0, c->tune_aligned);
+            Wave wave = wave_of(aligned);
+            if (c->tune_aligned < 0 && elem_size_storage(c->fmt) == 4 && wave.rows >= 16) wave = wave_of(aligned = 1);
             if (q == 0) c->i_aligned = aligned;
-            lev[q] = chunk_levels(c->fmt, h, one, c->tune_chunk, interior_max_rows(c->fmt, c->pitch));
+            lev[q] = chunk_levels(c->fmt, h, wave, c->tune_chunk, interior_max_rows(c->fmt, c->pitch));
             c->i_chunk[q] = lev[q].rows[0];
             levels |= lev[q].count[1] + lev[q].count[2] > 0;
             nitems += interior_items(r, q, strips[q], lev[q], nullptr, 0);
