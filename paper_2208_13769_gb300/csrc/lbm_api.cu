@@ -314,21 +314,27 @@ static int short_rows(double load) {
 // 62.2 / 60.1 / 53.7 and 61.4 / 57.2 / 50.1; 2000 x 1500, 29 rows in the full
 // wave, 69.4 / 66.4 in levels and 73.9 / 68.7 so).  FP16 at 1400 x 900: 29.4
 // and 29.6.
+// The extrapolated scheme keeps four more 4-byte carries and waits for memory
+// in every format: the same wave (FP16 1400 x 900 35.8 and 31.5, 1700 x 1438
+// 60.6 and 55.8), and where the full wave has 28 rows or more, chunks of 20
+// instead of levels (FP16 / plain / pair, levels and so: 2200 x 1800 95.4 /
+// 90.1 / 101.8 and 82.4 / 90.3 / 100.9, 3000 x 2900 187.7 / 183.3 / 207.3 and
+// 162.7 / 179.6 / 201.2).
 struct Wave {
     int rows;
     bool levels;
 };
 
-static Wave interior_wave(int fmt, int w, int h, int strips, int64_t share, double sms) {
+static Wave interior_wave(int fmt, bool xj, int w, int h, int strips, int64_t share, double sms) {
     auto rows = [&](int64_t ctas) {
         const int64_t per = std::max<int64_t>(1, ctas / strips);
         return int((h + per - 1) / per);
     };
     const int one = rows(share);
-    const bool four = elem_size_storage(fmt) == 4;
+    const bool four = xj || elem_size_storage(fmt) == 4;
     if (fmt == kFmtF64) return {std::max(one, 8), false};
     if (one <= 10) return {short_rows(double(w) * h / (kInteriorThreads - 4) / std::max(1.0, sms)), false};
-    if (one >= (four ? 28 : 48)) return {one, true};
+    if (one >= (four ? 28 : 48)) return xj ? Wave{20, false} : Wave{one, true};
     return {four ? rows(std::min(share, int64_t(4.45 * sms))) : one, false};
 }
 
@@ -401,7 +407,7 @@ static cudaError_t build_plan(lbm_ctx* c) {
             // 55.8 us a step, 57.4 without; 2000 x 1500: 72.1 and 75.1)
             auto wave_of = [&](int aligned) {
                 interior_strips(c->fmt, r[0], r[1], aligned, &c->i_strip_x0[q], &c->i_strip_w[q], &strips[q]);
-                return interior_wave(c->fmt, r[1] - r[0], h, strips[q], share,
+                return interior_wave(c->fmt, c->scheme == LBM_SCHEME_EXTRAPOLATED, r[1] - r[0], h, strips[q], share,
                                      double(c->num_sms) * double(share) / double(slots));
             };
             int aligned = std::max(0, c->tune_aligned);
