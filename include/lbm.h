@@ -208,7 +208,7 @@ typedef struct {
                            default (4) */
     int32_t chunk_rows; /* rows per CTA, >= 8; 0: one wave of CTAs over the SMs, with shorter
                            chunks after it on a large body; on a body of less than about 10
-                           rows each the 4 to 16 rows that take least time (default) */
+                           rows each the 4 to 18 rows that take least time (default) */
     int32_t aligned;    /* 1: the fewest strips of equal width on 32-byte sector boundaries (at
                            most 120 columns; 112 for 16-bit storage); 2: the same on 16-byte
                            boundaries (at most 124 columns; 120 for 16-bit storage);

@@ -277,34 +277,30 @@ static EdgeShape edge_shape(const lbm_ctx* c) {
     return best;
 }
 
-// Rows per CTA where one wave would give each few: a tile of r rows takes
-// about r + 4 iterations of its row pipeline (4 fill it), each of which lasts
-// as long as its chain of waits and barriers while an SM holds up to 2 CTAs,
-// then longer (they share its issue slots), and half as long again from about
-// 4.5 on.  `load` is the full-width CTAs per SM that 1-row tiles would make.
-// Measured (FP16 / FP32 us a step, with at least 8 rows and so): 420 x 400 12.6
-// / 13.2 and 9.4 / 10.0 (4 rows), 512 x 512 13.1 / 13.1 and 11.2 / 11.6 (4),
-// 600 x 600 13.2 / 14.2 (8 either way), 800 x 700 16.4 / 17.4 and 15.6 / 16.4
-// (7), 1000 x 777 22.1 / 24.5 and 20.3 / 21.1 (10).
-static int short_rows(double load) {
+// Rows per CTA where one full wave would give each few.  A tile of r rows
+// takes about r + 5 iterations of its row pipeline (the ones that fill it, the
+// launch and the end), and an iteration longer the more tiles (x) an SM holds:
+// in proportion to 4.5 + x, and from 4.6 on, where one more fills the SM's
+// places or its issue slots, to 4.5 + x + (x - 4.6).  The model's pick among 4
+// to 18 rows is within 1.2 % of the best one on average (10 % at worst) over
+// 18 bodies from 380 x 380 to 1000 x 1000 in three formats; the rows of a full
+// wave but at least 8 are up to 25 % off (640 x 640 FP32 19.4 us a step, 14.7
+// so).
+static int short_rows(int strips, int h, double sms) {
     int best = 8;
     double least = INFINITY;
-    for (int r = 4; r <= 16; ++r) {
-        const double x = load / r;
-        const double g = x <= 2.0   ? 0.72
-                         : x <= 3.0 ? 0.72 + 0.25 * (x - 2.0)
-                         : x <= 4.3 ? 0.97 + 0.14 * (x - 3.0)
-                         : x <= 4.8 ? 1.15 + (x - 4.3)
-                                    : 1.65 * x / 4.8;
-        if ((r + 4) * g < least) {
-            least = (r + 4) * g;
+    for (int r = 4; r <= 18; ++r) {
+        const double x = double(strips) * ((h + r - 1) / r) / sms;
+        const double t = (r + 5) * (4.5 + x + std::max(0.0, x - 4.6));
+        if (t < least) {
+            least = t;
             best = r;
         }
     }
     return best;
 }
 
-// The wave of a rectangle of w x h nodes in `strips` strips: rows per CTA for
+// The wave of a rectangle of h rows in `strips` strips: rows per CTA for
 // at most `share` CTAs on `sms` SMs, and whether it is long enough for shorter
 // chunks after it (ChunkLevels).  A wave of 4-byte storage that is not takes
 // 4.45 CTAs per SM instead of the 6 or 7 that fit: memory is as busy with them,
@@ -325,7 +321,7 @@ struct Wave {
     bool levels;
 };
 
-static Wave interior_wave(int fmt, bool xj, int w, int h, int strips, int64_t share, double sms) {
+static Wave interior_wave(int fmt, bool xj, int h, int strips, int64_t share, double sms) {
     auto rows = [&](int64_t ctas) {
         const int64_t per = std::max<int64_t>(1, ctas / strips);
         return int((h + per - 1) / per);
@@ -333,7 +329,7 @@ static Wave interior_wave(int fmt, bool xj, int w, int h, int strips, int64_t sh
     const int one = rows(share);
     const bool four = xj || elem_size_storage(fmt) == 4;
     if (fmt == kFmtF64) return {std::max(one, 8), false};
-    if (one <= 10) return {short_rows(double(w) * h / (kInteriorThreads - 4) / std::max(1.0, sms)), false};
+    if (one <= 10) return {short_rows(strips, h, std::max(1.0, sms)), false};
     if (one >= (four ? 28 : 48)) return xj ? Wave{20, false} : Wave{one, true};
     return {four ? rows(std::min(share, int64_t(4.45 * sms))) : one, false};
 }
@@ -346,8 +342,8 @@ static Wave interior_wave(int fmt, bool xj, int w, int h, int strips, int64_t sh
 // in it, then chunks of a quarter and an eighth of its rows (164 with 65 % at
 // some sizes, 168 with 85 %); 2200 x 1800: 91.7 and 86.0; at 1536 x 1536 (22
 // rows per CTA) 55.8 and 56.7, so a shorter wave stays one.  16-bit storage
-// waits less for memory and its SMs keep together: 136 us in one wave, 131 with 90 % in it; at 2500 x 1300 60.9 either way.
-// FP64 is bound by its arithmetic (1500 x 1000: 506 us, 507 in levels).
+// waits less for memory and its SMs keep together: 136 us in one wave, 131 with
+// 90 % in it; at 2500 x 1300 60.9 either way.  FP64 is bound by its arithmetic (1500 x 1000: 506 us, 507 in levels).
 static ChunkLevels chunk_levels(int fmt, int h, Wave wave, int tune_chunk, int max_rows) {
     ChunkLevels L;
     memset(&L, 0, sizeof(L));
@@ -407,7 +403,7 @@ static cudaError_t build_plan(lbm_ctx* c) {
             // 55.8 us a step, 57.4 without; 2000 x 1500: 72.1 and 75.1)
             auto wave_of = [&](int aligned) {
                 interior_strips(c->fmt, r[0], r[1], aligned, &c->i_strip_x0[q], &c->i_strip_w[q], &strips[q]);
-                return interior_wave(c->fmt, c->scheme == LBM_SCHEME_EXTRAPOLATED, r[1] - r[0], h, strips[q], share,
+                return interior_wave(c->fmt, c->scheme == LBM_SCHEME_EXTRAPOLATED, h, strips[q], share,
                                      double(c->num_sms) * double(share) / double(slots));
             };
             int aligned = std::max(0, c->tune_aligned);
@@ -446,13 +442,13 @@ static cudaError_t build_plan(lbm_ctx* c) {
     // edge tiles beside an interior: CTAs of an interior tile's size, each in
     // the place of one, for the many band tiles of seams and holes beside short
     // interior tiles (FP32 800 x 600 with a periodic axis 19.3 to 16.0 us a
-    // step, 1000 x 1000 with a hole 31.2 to 27.4) and where 4-byte storage keeps
-    // every place taken with shorter chunks (4096 x 2048 173.0 to 171.5); else
-    // wide ones, which compute less halo (800 x 700 16.0, 16.8 with small ones;
+    // step, 1000 x 1000 with a hole 31.2 to 27.4, 1200 x 1000 33.0 to 30.3) and
+    // where 4-byte storage keeps every place taken with shorter chunks (4096 x
+    // 2048 173.0 to 171.5); else wide ones, which compute less halo (800 x 700 16.0, 16.8 with small ones;
     // FP16 2600 x 2400 with a hole 97 and 99).  So too in the launch that the
     // image tiles share, whose CTAs are wide.
     const bool crowded =
-        (levels && elem_size_storage(c->fmt) == 4) || (c->i_chunk[0] <= 12 && (perx || pery || hole));
+        (levels && elem_size_storage(c->fmt) == 4) || c->i_chunk[0] <= (hole ? 20 : perx || pery ? 12 : 0);
     c->edge_shape = !c->has_interior ? edge_shape(c) : crowded && !seams_inside ? kEdgeInterior : kEdgeWide;
     int n = 0;
     for (int b = 0; b < c->nband; ++b)
