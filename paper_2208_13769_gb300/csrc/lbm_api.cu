@@ -17,7 +17,15 @@ using namespace lbm;
 
 namespace {
 
-constexpr int kGraphChunk = 64;  // steps per captured graph (even: keeps the ping-pong parity)
+// Steps per captured graph, a long and a short one (even: they keep the
+// ping-pong parity).  A mid-size body's step is shorter than its launches take
+// the host (512 x 512 FP32 18.5 us a step launched one by one, 12.0 in a
+// graph), so at most a short graph's steps are launched so; about 9 us pass
+// between two graphs of two branches (0.5 us a step if all were short).  A long
+// graph takes the host 0.6 ms to build, which a body's first call now spends
+// with that many steps in short graphs queued (640 x 384 FP16, a new body of
+// 500 steps: 7.3 ms, 6.9 so).
+constexpr int kGraphChunk = 64, kGraphShort = 16;
 constexpr int kSegMax = 144;  // widest row segment the interior kernel copies in bulk (elements)
 
 size_t elem_size_storage(int fmt) {
@@ -616,16 +624,17 @@ lbm_status lbm::ctx_ensure_initialized(lbm_ctx* c) {
     return LBM_OK;
 }
 
-// A graph of kGraphChunk plain steps starting at parity `par`.
-static lbm_status get_graph(lbm_ctx* c, int par, cudaGraphExec_t* out) {
-    if (c->graph[par]) {
-        *out = c->graph[par];
+// A graph of n plain steps (kGraphChunk or kGraphShort) starting at parity `par`.
+static lbm_status get_graph(lbm_ctx* c, int n, int par, cudaGraphExec_t* out) {
+    cudaGraphExec_t& slot = n == kGraphChunk ? c->graph[par] : c->graph_short[par];
+    if (slot) {
+        *out = slot;
         return LBM_OK;
     }
     cudaGraph_t g = nullptr;
     LBM_CUDA(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t err = cudaSuccess;
-    for (int k = 0; k < kGraphChunk && err == cudaSuccess; ++k) err = launch_step_kernels(c, 0, false, par ^ (k & 1));
+    for (int k = 0; k < n && err == cudaSuccess; ++k) err = launch_step_kernels(c, 0, false, par ^ (k & 1));
     cudaError_t e2 = cudaStreamEndCapture(c->stream, &g);
     if (err != cudaSuccess) {
         if (g) cudaGraphDestroy(g);
@@ -636,7 +645,7 @@ static lbm_status get_graph(lbm_ctx* c, int par, cudaGraphExec_t* out) {
     err = cudaGraphInstantiate(&ex, g, 0);
     cudaGraphDestroy(g);
     if (err != cudaSuccess) return ctx_fail_cuda(c, err);
-    c->graph[par] = ex;
+    slot = ex;
     *out = ex;
     return LBM_OK;
 }
@@ -655,6 +664,7 @@ lbm_status lbm::ctx_check_flag(lbm_ctx* c) {
 static void free_all(lbm_ctx* c) {
     for (int k = 0; k < 2; ++k) {
         if (c->graph[k]) cudaGraphExecDestroy(c->graph[k]);
+        if (c->graph_short[k]) cudaGraphExecDestroy(c->graph_short[k]);
         cudaFree(c->f[k]);
         cudaFree(c->a[k]);
         cudaFree(c->s[k]);
@@ -909,13 +919,22 @@ lbm_status lbm_step(lbm_ctx* c, int64_t nsteps) {
         --left;
         c->variant_warm = true;
     }
-    while (left > kGraphChunk) {
+    // a stream that the caller is capturing records up to kGraphChunk steps as
+    // plain launches (a second capture cannot begin on it)
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    LBM_CUDA(c, cudaStreamIsCapturing(c->stream, &capture));
+    const int shortest = capture == cudaStreamCaptureStatusNone ? kGraphShort : kGraphChunk;
+    int64_t queued = 0;
+    while (left > shortest) {
+        const bool built = c->graph[c->parity] != nullptr || queued >= kGraphChunk || shortest == kGraphChunk;
+        const int n = left > kGraphChunk && built ? kGraphChunk : kGraphShort;
         cudaGraphExec_t g;
-        st = get_graph(c, c->parity, &g);
+        st = get_graph(c, n, c->parity, &g);
         if (st != LBM_OK) return st;
         LBM_CUDA(c, cudaGraphLaunch(g, c->stream));
-        c->steps += kGraphChunk;  // kGraphChunk is even: parity unchanged
-        left -= kGraphChunk;
+        c->steps += n;  // even: parity unchanged
+        queued += n;
+        left -= n;
     }
     while (left > 1) {
         st = launch(c, 0, false);

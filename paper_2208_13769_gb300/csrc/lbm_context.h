@@ -83,7 +83,7 @@ struct lbm_ctx {
     int64_t steps = 0;
     bool sticky = false;
     bool variant_warm = false;
-    cudaGraphExec_t graph[2] = {nullptr, nullptr};
+    cudaGraphExec_t graph[2] = {nullptr, nullptr}, graph_short[2] = {nullptr, nullptr};
     // a rectangular hole: removed nodes x0 <= x < x1, y0 <= y < y1 (none
     // while x0 >= x1), and the traction on its faces at x0, x1, y0, y1
     int32_t hole[4] = {0, 0, 0, 0};
