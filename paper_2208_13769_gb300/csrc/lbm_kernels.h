@@ -158,6 +158,8 @@ struct ReadoutParams {
     const double* fields;  // 5 planes [ny][nx]: u_x, u_y, v_x, v_y, r
     EdgeBC bc[4];
     int32_t hole[4];  // removed nodes of a hole (x0 >= x1: none)
+    const int32_t* flag;  // the body's status flag, copied to host_flag (pinned
+    int32_t* host_flag;   // host memory) by the read-out; NULL: not copied
 };
 
 // Writes the fields selected by mask (LBM_FIELD_* bits) into out, each block
