@@ -652,10 +652,17 @@ static lbm_status get_graph(lbm_ctx* c, int n, int par, cudaGraphExec_t* out) {
 
 // Device flag bits: 1 non-finite value or J <= 0; 4 a bounded wait gave up;
 // 8 a bulk copy was refused for misalignment (an internal error).
+static lbm_status ctx_wait_flag(lbm_ctx* c);
+
 lbm_status lbm::ctx_check_flag(lbm_ctx* c) {
-    int32_t h = 0;
-    LBM_CUDA(c, cudaMemcpyAsync(&h, c->flag, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
+    LBM_CUDA(c, cudaMemcpyAsync(c->host_flag, c->flag, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
+    return ctx_wait_flag(c);
+}
+
+// The same where the flag's copy is queued already.
+static lbm_status ctx_wait_flag(lbm_ctx* c) {
     LBM_CUDA(c, cudaStreamSynchronize(c->stream));
+    const int32_t h = *static_cast<volatile int32_t*>(c->host_flag);
     if (h & 8) return ctx_fail_cuda(c, cudaErrorMisalignedAddress);
     if (h & 4) return LBM_E_TIMEOUT;
     return (h & 1) ? LBM_E_UNSTABLE : LBM_OK;
@@ -673,6 +680,7 @@ static void free_all(lbm_ctx* c) {
     cudaFree(c->u0);
     cudaFree(c->v0);
     cudaFree(c->flag);
+    cudaFreeHost(c->host_flag);
     cudaFree(c->counter);
     cudaFree(c->partials);
     cudaFree(c->diag);
@@ -798,6 +806,7 @@ lbm_status lbm_create(const lbm_desc* d, lbm_ctx** out) {
     if (err == cudaSuccess && d->u0) err = cudaMalloc(&c->u0, ubytes);
     if (err == cudaSuccess && d->v0) err = cudaMalloc(&c->v0, ubytes);
     if (err == cudaSuccess) err = cudaMalloc(&c->flag, sizeof(int32_t));
+    if (err == cudaSuccess) err = cudaHostAlloc(&c->host_flag, sizeof(int32_t), cudaHostAllocMapped);
     if (err == cudaSuccess) err = cudaMalloc(&c->counter, 2 * sizeof(int64_t));
     if (err == cudaSuccess) err = cudaMalloc(&c->partials, size_t(c->diag_blocks) * 8 * sizeof(double));
     if (err == cudaSuccess) err = cudaMalloc(&c->diag, 8 * sizeof(double));
@@ -1185,10 +1194,12 @@ lbm_status lbm_read_fields(lbm_ctx* c, uint32_t mask, double* out, int64_t out_l
         c->readout_cap = bytes;
     }
     ReadoutParams rp = make_readout(c);
+    rp.flag = c->flag;  // with the fields, instead of a copy of 4 bytes after theirs
+    rp.host_flag = c->host_flag;
     LBM_CUDA(c, launch_readout(rp, mask, c->readout, c->stream));
     LBM_CUDA(c, cudaMemcpyAsync(out, c->readout, bytes, cudaMemcpyDeviceToHost, c->stream));
     if (t_out) *t_out = double(c->steps) * c->dt;
-    return ctx_check_flag(c);
+    return ctx_wait_flag(c);
 }
 
 lbm_status lbm_diagnostics(lbm_ctx* c, double out[6]) {

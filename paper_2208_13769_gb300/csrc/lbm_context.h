@@ -64,6 +64,7 @@ struct lbm_ctx {
     double* u0 = nullptr;
     double* v0 = nullptr;
     int32_t* flag = nullptr;
+    int32_t* host_flag = nullptr;  // pinned: where the flag is read on the host
     int64_t* counter = nullptr;
     double* partials = nullptr;
     double* diag = nullptr;
