@@ -6,6 +6,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <memory>
 #include <new>
 
 #include "lbm.h"
@@ -393,6 +394,8 @@ static cudaError_t build_plan(lbm_ctx* c) {
     const bool hole = c->hole[0] < c->hole[1];
     const bool perx = c->bc[0].kind == kPeriodic, pery = c->bc[2].kind == kPeriodic;
     bool levels = false;  // shorter chunks after the interior's wave
+    std::unique_ptr<InteriorItem[]> items;
+    c->n_items = 0;
     if (c->n_irect > 0) {
         c->i_ring = c->tune_ring ? c->tune_ring : kInteriorRing;
         const int per_sm = std::max(1, interior_occupancy(c->fmt, c->i_ring));
@@ -424,21 +427,15 @@ static cudaError_t build_plan(lbm_ctx* c) {
             nitems += interior_items(r, q, strips[q], lev[q], nullptr, 0);
         }
         if (nitems > INT32_MAX - 1) return cudaErrorInvalidConfiguration;
-        InteriorItem* items = new (std::nothrow) InteriorItem[size_t(nitems)];
+        items.reset(new (std::nothrow) InteriorItem[size_t(nitems)]);
         if (!items) return cudaErrorMemoryAllocation;
         int64_t at = 0;
         for (int q = 0; q < c->n_irect; ++q)
-            at += interior_items(c->irect[q], q, strips[q], lev[q], items + at, nitems - at);
+            at += interior_items(c->irect[q], q, strips[q], lev[q], items.get() + at, nitems - at);
         // the longest first, so that the short ones even out the launch's end
-        std::stable_sort(items, items + nitems, [](const InteriorItem& a, const InteriorItem& b) {
+        std::stable_sort(items.get(), items.get() + nitems, [](const InteriorItem& a, const InteriorItem& b) {
             return std::abs(a.rows) > std::abs(b.rows);
         });
-        cudaError_t e = cudaMalloc(&c->ditems, sizeof(InteriorItem) * size_t(nitems));
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(c->ditems, items, sizeof(InteriorItem) * size_t(nitems), cudaMemcpyHostToDevice, c->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);  // items is freed below
-        delete[] items;
-        if (e != cudaSuccess) return e;
         c->n_items = int(nitems);
     }
     c->has_interior = c->n_irect > 0;  // a hole may leave the bands only
@@ -452,9 +449,9 @@ static cudaError_t build_plan(lbm_ctx* c) {
     // interior tiles (FP32 800 x 600 with a periodic axis 19.3 to 16.0 us a
     // step, 1000 x 1000 with a hole 31.2 to 27.4, 1200 x 1000 33.0 to 30.3) and
     // where 4-byte storage keeps every place taken with shorter chunks (4096 x
-    // 2048 173.0 to 171.5); else wide ones, which compute less halo (800 x 700 16.0, 16.8 with small ones;
-    // FP16 2600 x 2400 with a hole 97 and 99).  So too in the launch that the
-    // image tiles share, whose CTAs are wide.
+    // 2048 173.0 to 171.5); else wide ones, which compute less halo (800 x 700
+    // 16.0, 16.8 with small ones; FP16 2600 x 2400 with a hole 97 and 99).  So
+    // too in the launch that the image tiles share, whose CTAs are wide.
     const bool crowded =
         (levels && elem_size_storage(c->fmt) == 4) || c->i_chunk[0] <= (hole ? 20 : perx || pery ? 12 : 0);
     c->edge_shape = !c->has_interior ? edge_shape(c) : crowded && !seams_inside ? kEdgeInterior : kEdgeWide;
@@ -465,40 +462,46 @@ static cudaError_t build_plan(lbm_ctx* c) {
     if (hole)
         for (int q = 0; q < c->n_irect; ++q)
             ni += edge_tiles_of_rect(c->irect[q], 0, nullptr, 0, false, c->edge_shape, 0);
-    EdgeTile* h = new (std::nothrow) EdgeTile[size_t(ni)];
+    std::unique_ptr<EdgeTile[]> h(new (std::nothrow) EdgeTile[size_t(ni)]);
     if (!h) return cudaErrorMemoryAllocation;
     int m = 0;
     for (int b = 0; b < c->nband; ++b)
-        m += edge_tiles_of_rect(c->brect[b], 0, h + m, n - m, m == 0, c->edge_shape, bounded_sides(c, c->brect[b]));
+        m += edge_tiles_of_rect(c->brect[b], 0, h.get() + m, n - m, m == 0, c->edge_shape, bounded_sides(c, c->brect[b]));
     if (hole)
         for (int q = 0; q < c->n_irect; ++q)
-            m += edge_tiles_of_rect(c->irect[q], 0, h + m, ni - m, false, c->edge_shape, 0);
+            m += edge_tiles_of_rect(c->irect[q], 0, h.get() + m, ni - m, false, c->edge_shape, 0);
     // the images of the interior's nodes next to a periodic seam
     int nimg = 0;
-    ImageTile* himg = nullptr;
+    std::unique_ptr<ImageTile[]> himg;
     if (c->has_interior && seams_inside && (perx || pery)) {
         int box[4];
         seam_box(c, box);
         nimg = image_tiles_of_body(c->nx, c->ny, perx, pery, box, 0, nullptr, 0);
-        himg = new (std::nothrow) ImageTile[size_t(nimg)];
-        if (!himg) {
-            delete[] h;
-            return cudaErrorMemoryAllocation;
-        }
-        image_tiles_of_body(c->nx, c->ny, perx, pery, box, 0, himg, nimg);
+        himg.reset(new (std::nothrow) ImageTile[size_t(nimg)]);
+        if (!himg) return cudaErrorMemoryAllocation;
+        image_tiles_of_body(c->nx, c->ny, perx, pery, box, 0, himg.get(), nimg);
     }
     StepParams hp[2] = {make_params(c, 0), make_params(c, 1)};
-    cudaError_t e = cudaMalloc(&c->dtiles, sizeof(EdgeTile) * size_t(ni));
-    if (e == cudaSuccess) e = cudaMalloc(&c->dparams, sizeof(hp));
-    if (e == cudaSuccess) e = cudaMemcpyAsync(c->dtiles, h, sizeof(EdgeTile) * size_t(ni), cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(c->dparams, hp, sizeof(hp), cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess && nimg > 0) e = cudaMalloc(&c->dimg, sizeof(ImageTile) * size_t(nimg));
-    if (e == cudaSuccess && nimg > 0)
-        e = cudaMemcpyAsync(c->dimg, himg, sizeof(ImageTile) * size_t(nimg), cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);  // h and himg are freed below
-    delete[] h;
-    delete[] himg;
+    // one allocation and one copy for the lists and the parameters
+    const void* part[4] = {items.get(), h.get(), hp, himg.get()};
+    const size_t bytes[4] = {sizeof(InteriorItem) * size_t(c->n_items), sizeof(EdgeTile) * size_t(ni), sizeof(hp),
+                             sizeof(ImageTile) * size_t(nimg)};
+    size_t at[5] = {0};
+    for (int k = 0; k < 4; ++k) at[k + 1] = at[k] + (bytes[k] + 255) / 256 * 256;
+    std::unique_ptr<unsigned char[]> host(new (std::nothrow) unsigned char[at[4]]);
+    if (!host) return cudaErrorMemoryAllocation;
+    for (int k = 0; k < 4; ++k)
+        if (bytes[k] > 0) memcpy(host.get() + at[k], part[k], bytes[k]);
+    cudaFree(c->plan);  // of an attempt that failed
+    c->plan = nullptr;
+    cudaError_t e = cudaMalloc(&c->plan, at[4]);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(c->plan, host.get(), at[4], cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);  // the host's copy is freed
     if (e != cudaSuccess) return e;
+    c->ditems = reinterpret_cast<InteriorItem*>(c->plan + at[0]);
+    c->dtiles = reinterpret_cast<EdgeTile*>(c->plan + at[1]);
+    c->dparams = reinterpret_cast<StepParams*>(c->plan + at[2]);
+    c->dimg = reinterpret_cast<ImageTile*>(c->plan + at[3]);
     c->n_img = nimg;
     c->n_etiles = n;
     c->n_itiles = hole ? ni : 0;
@@ -606,6 +609,13 @@ static lbm_status launch(lbm_ctx* c, int mode, bool fields) {
     return LBM_OK;
 }
 
+static void drop_initial_fields(lbm_ctx* c) {
+    const int64_t ubytes = int64_t(2) * c->nx * c->ny * int64_t(sizeof(double));
+    c->device_bytes -= ubytes * ((c->u0 != nullptr) + (c->v0 != nullptr));
+    cudaFree(c->initial);
+    c->initial = c->u0 = c->v0 = nullptr;
+}
+
 lbm_status lbm::ctx_ensure_initialized(lbm_ctx* c) {
     if (c->initialized) return LBM_OK;
     lbm_status st = launch(c, 1, true);
@@ -614,12 +624,7 @@ lbm_status lbm::ctx_ensure_initialized(lbm_ctx* c) {
     // the initial fields are read only by the initialisation: give them back
     if (c->u0 || c->v0) {
         LBM_CUDA(c, cudaStreamSynchronize(c->stream));
-        const int64_t ubytes = int64_t(2) * c->nx * c->ny * int64_t(sizeof(double));
-        if (c->u0) c->device_bytes -= ubytes;
-        if (c->v0) c->device_bytes -= ubytes;
-        cudaFree(c->u0);
-        cudaFree(c->v0);
-        c->u0 = c->v0 = nullptr;
+        drop_initial_fields(c);
     }
     return LBM_OK;
 }
@@ -672,23 +677,12 @@ static void free_all(lbm_ctx* c) {
     for (int k = 0; k < 2; ++k) {
         if (c->graph[k]) cudaGraphExecDestroy(c->graph[k]);
         if (c->graph_short[k]) cudaGraphExecDestroy(c->graph_short[k]);
-        cudaFree(c->f[k]);
-        cudaFree(c->a[k]);
-        cudaFree(c->s[k]);
     }
-    cudaFree(c->fields);
-    cudaFree(c->u0);
-    cudaFree(c->v0);
-    cudaFree(c->flag);
+    cudaFree(c->arena);
+    cudaFree(c->initial);
     cudaFreeHost(c->host_flag);
-    cudaFree(c->counter);
-    cudaFree(c->partials);
-    cudaFree(c->diag);
     cudaFree(c->readout);
-    cudaFree(c->dparams);
-    cudaFree(c->dtiles);
-    cudaFree(c->ditems);
-    cudaFree(c->dimg);
+    cudaFree(c->plan);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
     if (c->side) cudaStreamDestroy(c->side);
@@ -796,20 +790,43 @@ lbm_status lbm_create(const lbm_desc* d, lbm_ctx** out) {
     const size_t fldbytes = size_t(5) * nodes * sizeof(double);
     const size_t ubytes = size_t(2) * nodes * sizeof(double);
     c->diag_blocks = diagnostics_blocks(nodes);
-    cudaError_t err = cudaSuccess;
-    for (int k = 0; k < 2 && err == cudaSuccess; ++k) {
-        err = cudaMalloc(&c->f[k], fbytes);
-        if (err == cudaSuccess) err = cudaMalloc(&c->a[k], abytes);
-        if (err == cudaSuccess) err = cudaMalloc(&c->s[k], sbytes);
+    // one allocation for all that lives as long as the context: an allocation
+    // and its release take the host 30 to 60 us each (640 x 384 FP16 created and
+    // destroyed in 640 and 550 us with eleven of them and the plan's, in 360 and
+    // 385 so)
+    size_t arena = 0;
+    auto place = [&](size_t bytes) {
+        const size_t at = arena;
+        arena += (bytes + 511) / 512 * 512;
+        return at;
+    };
+    size_t at_f[2], at_a[2], at_s[2];
+    for (int k = 0; k < 2; ++k) {
+        at_f[k] = place(fbytes);
+        at_a[k] = place(abytes);
+        at_s[k] = place(sbytes);
     }
-    if (err == cudaSuccess) err = cudaMalloc(&c->fields, fldbytes);
-    if (err == cudaSuccess && d->u0) err = cudaMalloc(&c->u0, ubytes);
-    if (err == cudaSuccess && d->v0) err = cudaMalloc(&c->v0, ubytes);
-    if (err == cudaSuccess) err = cudaMalloc(&c->flag, sizeof(int32_t));
+    const size_t at_fields = place(fldbytes), at_flag = place(sizeof(int32_t)), at_counter = place(2 * sizeof(int64_t)),
+                 at_partials = place(size_t(c->diag_blocks) * 8 * sizeof(double)), at_diag = place(8 * sizeof(double));
+    cudaError_t err = cudaMalloc(&c->arena, arena);
+    if (err == cudaSuccess) {
+        for (int k = 0; k < 2; ++k) {
+            c->f[k] = c->arena + at_f[k];
+            c->a[k] = c->arena + at_a[k];
+            c->s[k] = c->arena + at_s[k];
+        }
+        c->fields = reinterpret_cast<double*>(c->arena + at_fields);
+        c->flag = reinterpret_cast<int32_t*>(c->arena + at_flag);
+        c->counter = reinterpret_cast<int64_t*>(c->arena + at_counter);
+        c->partials = reinterpret_cast<double*>(c->arena + at_partials);
+        c->diag = reinterpret_cast<double*>(c->arena + at_diag);
+    }
+    if (err == cudaSuccess && (d->u0 || d->v0)) err = cudaMalloc(&c->initial, (d->u0 && d->v0 ? 2 : 1) * ubytes);
+    if (err == cudaSuccess) {
+        c->u0 = d->u0 ? c->initial : nullptr;
+        c->v0 = d->v0 ? c->initial + (d->u0 ? ubytes / sizeof(double) : 0) : nullptr;
+    }
     if (err == cudaSuccess) err = cudaHostAlloc(&c->host_flag, sizeof(int32_t), cudaHostAllocMapped);
-    if (err == cudaSuccess) err = cudaMalloc(&c->counter, 2 * sizeof(int64_t));
-    if (err == cudaSuccess) err = cudaMalloc(&c->partials, size_t(c->diag_blocks) * 8 * sizeof(double));
-    if (err == cudaSuccess) err = cudaMalloc(&c->diag, 8 * sizeof(double));
     if (err != cudaSuccess) {
         cudaGetLastError();
         free_all(c);
@@ -819,14 +836,7 @@ lbm_status lbm_create(const lbm_desc* d, lbm_ctx** out) {
     c->device_bytes = int64_t(2 * (fbytes + abytes + sbytes) + fldbytes + (d->u0 ? ubytes : 0) + (d->v0 ? ubytes : 0));
     // the state is cleared on the side stream while the initial fields are
     // uploaded on the main one (the copy engines and the SMs work at once)
-    for (int k = 0; k < 2 && err == cudaSuccess; ++k) {
-        err = cudaMemsetAsync(c->f[k], 0, fbytes, c->side);
-        if (err == cudaSuccess) err = cudaMemsetAsync(c->a[k], 0, abytes, c->side);
-        if (err == cudaSuccess) err = cudaMemsetAsync(c->s[k], 0, sbytes, c->side);
-    }
-    if (err == cudaSuccess) err = cudaMemsetAsync(c->fields, 0, fldbytes, c->side);
-    if (err == cudaSuccess) err = cudaMemsetAsync(c->flag, 0, sizeof(int32_t), c->side);
-    if (err == cudaSuccess) err = cudaMemsetAsync(c->counter, 0, 2 * sizeof(int64_t), c->side);
+    err = cudaMemsetAsync(c->arena, 0, arena, c->side);
     if (err == cudaSuccess && d->u0) err = cudaMemcpyAsync(c->u0, d->u0, ubytes, cudaMemcpyHostToDevice, c->stream);
     if (err == cudaSuccess && d->v0) err = cudaMemcpyAsync(c->v0, d->v0, ubytes, cudaMemcpyHostToDevice, c->stream);
     if (err == cudaSuccess) err = cudaStreamSynchronize(c->side);
@@ -1346,12 +1356,7 @@ lbm_status lbm_write_state(lbm_ctx* c, const void* in, int64_t in_len) {
     c->steps = h.steps;
     if (!c->initialized) {  // the restored state replaces the initialisation
         c->initialized = true;
-        const int64_t ubytes = int64_t(2) * c->nx * c->ny * int64_t(sizeof(double));
-        if (c->u0) c->device_bytes -= ubytes;
-        if (c->v0) c->device_bytes -= ubytes;
-        cudaFree(c->u0);
-        cudaFree(c->v0);
-        c->u0 = c->v0 = nullptr;
+        drop_initial_fields(c);
     }
     return LBM_OK;
 }

@@ -61,8 +61,10 @@ struct lbm_ctx {
     void* a[2] = {nullptr, nullptr};
     void* s[2] = {nullptr, nullptr};
     double* fields = nullptr;
+    double* initial = nullptr;  // u0 and v0, until the initialisation has read them
     double* u0 = nullptr;
     double* v0 = nullptr;
+    unsigned char* arena = nullptr;  // device: f, a, s, fields, flag, counter, partials and diag lie in it
     int32_t* flag = nullptr;
     int32_t* host_flag = nullptr;  // pinned: where the flag is read on the host
     int64_t* counter = nullptr;
@@ -97,6 +99,7 @@ struct lbm_ctx {
     int n_irect = 0;
     int irect[4][4];
     int i_chunk[4], i_strip_x0[4], i_strip_w[4];
+    unsigned char* plan = nullptr;        // device: ditems, dtiles, dparams and dimg lie in it
     lbm::InteriorItem* ditems = nullptr;  // device: the interior tiles
     int n_items = 0;
     int i_ring = 0, i_aligned = 0;
