@@ -345,11 +345,10 @@ LBM_API lbm_status lbm_batch_create(lbm_ctx* const* members, int32_t n, void* cu
 
 /* lbm_batch_create with a decomposition of the batch's interior tiles (no
  * counterpart in the paper; it changes the split of the work, never the
- * results): tuning->ring_slots, rows of the bulk-copy ring (4..8; 0: 4),
- * tuning->chunk_rows, rows per interior tile (>= 8; 0: about eight waves of
- * resident CTAs over the batch, 32..256 rows), and tuning->aligned, the
- * strip grid of each member (as for lbm_set_tuning; -1: 124-column strips
- * for 16-bit storage, strips on 32-byte sectors otherwise); plan is ignored
+ * results): tuning->ring_slots, rows of the pipeline in flight or in work
+ * (4..8; 0: 4), tuning->chunk_rows, rows per interior tile (>= 8; 0: about a
+ * wave's rows for most of them, then shorter tiles), and tuning->aligned, the
+ * strip grid of each member (as for lbm_set_tuning; -1: 2); plan is ignored
  * (each member keeps its own).  NULL: the defaults.
  * Errors as lbm_batch_create, and LBM_E_INVALID for a tuning out of range. */
 LBM_API lbm_status lbm_batch_create_tuned(lbm_ctx* const* members, int32_t n, void* cuda_stream,

@@ -295,7 +295,7 @@ static EdgeShape edge_shape(const lbm_ctx* c) {
 // 18 bodies from 380 x 380 to 1000 x 1000 in three formats; the rows of a full
 // wave but at least 8 are up to 25 % off (640 x 640 FP32 19.4 us a step, 14.7
 // so).
-static int short_rows(int strips, int h, double sms) {
+int lbm::short_rows(int strips, int h, double sms) {
     int best = 8;
     double least = INFINITY;
     for (int r = 4; r <= 18; ++r) {

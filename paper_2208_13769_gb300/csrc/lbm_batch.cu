@@ -56,7 +56,7 @@ struct lbm_batch {
     int n_img = 0;                // image tiles
     int chunk_rows = 0;
     int ring = kBatchRing;
-    int aligned = 1;  // strip grid of the interior tiles (interior_strips)
+    int aligned = 2;  // strip grid of the interior tiles (interior_strips)
     bool holed = false;           // some member has a hole
     int64_t steps = 0;
     bool warm = false;
@@ -99,8 +99,9 @@ void batch_free(lbm_batch* b) {
 // One batch time step from table parity q: the interior tiles on the batch's
 // stream and the edge tiles on the side stream, forked from and joined to
 // the batch's stream (the small edge CTAs fill the room the interior CTAs
-// leave), or, with seam images, the edge tiles and the images after the
-// interior on the batch's stream.
+// leave), and the images of members across periodic seams after the interior
+// (with the edge tiles in that launch too, after the interior: 12 bodies of
+// 128 to 2048 nodes a side in FP16 375 us a step, 367 so).
 cudaError_t batch_launch(lbm_batch* b, int q, bool fields) {
     const StepParams* tab = b->dtab + size_t(q) * size_t(b->n_entries);
     BatchInteriorLaunch I;
@@ -115,19 +116,13 @@ cudaError_t batch_launch(lbm_batch* b, int q, bool fields) {
     E.params = tab;
     E.tiles = b->dtiles;
     E.fields = fields ? 1 : 0;
-    if (b->n_img > 0) {
-        // members across periodic seams: the interior, then every member's
-        // edge tiles and seam images in one launch after it (the images copy
-        // what the interior launch wrote; the two launches barely overlapped
-        // anyway, six interior CTAs filling an SM's registers)
-        cudaError_t e = launch_batch_interior(b->fmt, I, b->ring, b->stream, nullptr);
-        if (e == cudaSuccess) e = launch_edge_images(b->fmt, E, b->n_edge, b->dimg, b->n_img, b->stream, b->holed, false);
-        return e;
-    }
     cudaError_t e = cudaEventRecord(b->ev_fork, b->stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(b->side, b->ev_fork, 0);
     if (e == cudaSuccess) e = launch_batch_interior(b->fmt, I, b->ring, b->stream, nullptr);
     if (e == cudaSuccess) e = launch_edge(b->fmt, E, b->n_edge, b->side, 0, b->holed, false);
+    // the seam images copy what the interior launch wrote
+    if (e == cudaSuccess && b->n_img > 0)
+        e = launch_edge_images(b->fmt, E, 0, b->dimg, b->n_img, b->stream, b->holed, false);
     if (e == cudaSuccess) e = cudaEventRecord(b->ev_join, b->side);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->ev_join, 0);
     return e;
@@ -165,11 +160,39 @@ lbm_status batch_graph(lbm_batch* b, int q, cudaGraphExec_t* out) {
     return LBM_OK;
 }
 
-// The batch's default strip grid: 124-column strips for 16-bit storage
-// (measured on the 256-body workload: 40 900 MLUPS against 38 700 with
-// strips on 32-byte sectors, which are at most 112 columns wide in a 2-byte
-// plane), sector-aligned strips otherwise (FP32: 36 700 against 36 100).
-int batch_default_aligned(int fmt) { return fmt == kFmtF16 || fmt == kFmtBF16 ? 0 : 1; }
+// The chunks of h rows of one member.  `one` is the rows per CTA if the batch
+// ran as one wave, `all` its rows over all strips.  As of a single long body,
+// most rows go to chunks of about a wave's rows and the rest to shorter ones,
+// which even out the end of the launch; fewer than 10 rows a wave are split as
+// a single short body's.  32 bodies of 64 to 1024 nodes a side in FP32 (93
+// rows) 247 us a step with chunks of 32 rows and 243 so, 12 of 128 to 2048 in
+// FP16 (185) 367 and 347, 20 of 64 to 700 in FP16 (35) 110 and 93, 6 of 64 to
+// 400 in FP32 (5) 36 and 23.
+ChunkLevels batch_levels(int h, int tune_chunk, double one, int64_t all, int sms, int max_rows) {
+    ChunkLevels L;
+    memset(&L, 0, sizeof(L));
+    int rows = tune_chunk;
+    if (rows == 0 && one < 10) rows = short_rows(1, int(all), sms);
+    if (rows > 0) {
+        L.rows[0] = std::min(rows, max_rows);
+        L.count[0] = (h + L.rows[0] - 1) / L.rows[0];
+        return L;
+    }
+    auto part = [&](double f) { return std::max(8, int(std::min(f * one, double(max_rows)))); };
+    L.rows[0] = std::min(part(0.75), h);
+    L.rows[1] = part(0.5);
+    L.rows[2] = part(1.0 / 3);
+    L.count[0] = std::max(1, int(0.75 * h / L.rows[0]));
+    const int left = h - L.count[0] * L.rows[0];
+    L.count[1] = std::min(left / L.rows[1], int(0.15 * h / L.rows[1]));
+    L.count[2] = (left - L.count[1] * L.rows[1] + L.rows[2] - 1) / L.rows[2];
+    return L;
+}
+
+// The batch's default strip grid: strips on 16-byte boundaries (12 bodies of
+// 128 to 2048 nodes a side in FP16 346 us a step, 357 without alignment, 380 on
+// sectors; 8 of 64 to 1024 in FP64 878, 883, 960; 32 in FP32 247, 258, 248).
+constexpr int kBatchAligned = 2;
 
 // Copies every member's status flag into one array (one launch and one
 // copy for the whole batch instead of one round trip per member).
@@ -269,8 +292,6 @@ lbm_status lbm_batch_create_tuned(lbm_ctx* const* members, int32_t n, void* cuda
         delete b;
         return LBM_E_OOM;
     }
-    // interior tiles: rows per chunk so that the batch holds about eight
-    // waves of resident CTAs (at least 32 rows, at most 256)
     int64_t all_interior = 0;
     for (int i = 0; i < n; ++i) {
         const lbm_ctx* c = b->m[size_t(i)];
@@ -281,7 +302,7 @@ lbm_status lbm_batch_create_tuned(lbm_ctx* const* members, int32_t n, void* cuda
         b->holed = b->holed || c->hole[0] < c->hole[1];
     }
     b->ring = tuning && tuning->ring_slots ? tuning->ring_slots : kBatchRing;
-    b->aligned = tuning && tuning->aligned >= 0 ? tuning->aligned : batch_default_aligned(b->fmt);
+    b->aligned = tuning && tuning->aligned >= 0 ? tuning->aligned : kBatchAligned;
     // the interior kernel's CTAs per SM with this ring (the first call also
     // sets its shared-memory limit, outside any capture)
     int resident = 0;
@@ -290,10 +311,9 @@ lbm_status lbm_batch_create_tuned(lbm_ctx* const* members, int32_t n, void* cuda
         memset(&L, 0, sizeof(L));
         if (e == cudaSuccess) e = launch_batch_interior(b->fmt, L, b->ring, b->stream, &resident);
     }
-    const int64_t wave = int64_t(b->m[0]->num_sms) * std::max(1, resident);
-    b->chunk_rows = tuning && tuning->chunk_rows
-                        ? tuning->chunk_rows
-                        : int(std::min<int64_t>(256, std::max<int64_t>(32, all_interior / (int64_t(120) * wave * 8))));
+    const int sms = b->m[0]->num_sms;
+    b->chunk_rows = tuning ? tuning->chunk_rows : 0;
+    const double one = double(all_interior) / (120.0 * sms * std::max(1, resident));
     cudaError_t e_maps = cudaSuccess;
     std::vector<StepParams> tab;
     std::vector<InteriorMaps> maps;
@@ -325,10 +345,8 @@ lbm_status lbm_batch_create_tuned(lbm_ctx* const* members, int32_t n, void* cuda
                 if (q < mri.n_irect) {
                     const int e = int(ent.size()) - 1;
                     const int h = p.rect[3] - p.rect[2];
-                    ChunkLevels lev;
-                    memset(&lev, 0, sizeof(lev));
-                    lev.rows[0] = std::min(b->chunk_rows, interior_max_rows(b->fmt, c->pitch));
-                    lev.count[0] = (h + lev.rows[0] - 1) / lev.rows[0];
+                    const ChunkLevels lev =
+                        batch_levels(h, b->chunk_rows, one, all_interior / 120, sms, interior_max_rows(b->fmt, c->pitch));
                     const int64_t cnt = interior_items(mri.irect[q], e, ns, lev, nullptr, 0);
                     const size_t at = items.size();
                     items.resize(at + size_t(cnt));
@@ -579,7 +597,7 @@ lbm_status lbm_batch_autotune(lbm_ctx* const* members, int32_t n, int64_t steps,
     // best of those
     const int rings[3] = {4, 5, 6};
     const int chunks[5] = {0, 32, 64, 128, 256};
-    const int al0 = batch_default_aligned(members[0]->fmt);
+    const int al0 = kBatchAligned;
     double best_t = INFINITY;
     lbm_tuning bt = {0, 0, al0, 0};
     cudaEvent_t e0 = nullptr, e1 = nullptr;

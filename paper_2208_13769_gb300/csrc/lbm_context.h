@@ -158,5 +158,8 @@ void seam_box(const lbm_ctx* c, int box[4]);
 lbm_status ctx_ensure_initialized(lbm_ctx* c);
 // Synchronises the context's stream and maps its device flag to a status.
 lbm_status ctx_check_flag(lbm_ctx* c);
+// Rows per interior tile where a full wave would give each few: of a rectangle
+// of h rows in `strips` strips on `sms` SMs.
+int short_rows(int strips, int h, double sms);
 
 }  // namespace lbm
