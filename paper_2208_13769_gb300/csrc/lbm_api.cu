@@ -351,23 +351,23 @@ static Wave interior_wave(int fmt, bool xj, int h, int strips, int64_t share, do
 // in it, then chunks of a quarter and an eighth of its rows (164 with 65 % at
 // some sizes, 168 with 85 %); 2200 x 1800: 91.7 and 86.0; at 1536 x 1536 (22
 // rows per CTA) 55.8 and 56.7, so a shorter wave stays one.  16-bit storage
-// waits less for memory and its SMs keep together: 136 us in one wave, 131 with
-// 90 % in it; at 2500 x 1300 60.9 either way.  FP64 is bound by its arithmetic (1500 x 1000: 506 us, 507 in levels).
-static ChunkLevels chunk_levels(int fmt, int h, Wave wave, int tune_chunk, int max_rows) {
+// waits less for memory and gains from 48 rows on: 3000 x 2900 152 us with 90 %
+// in the wave and 143 so; at 2500 x 1300 60.9 either way.  FP64 is bound by its
+// arithmetic (1500 x 1000: 506 us, 507 in levels).
+static ChunkLevels chunk_levels(int h, Wave wave, int tune_chunk, int max_rows) {
     ChunkLevels L;
     memset(&L, 0, sizeof(L));
     const int one = wave.rows;
-    const bool four = elem_size_storage(fmt) == 4;
     if (tune_chunk > 0 || !wave.levels || one > max_rows) {
         L.rows[0] = std::min(tune_chunk > 0 ? tune_chunk : one, std::min(h, max_rows));
         L.count[0] = (h + L.rows[0] - 1) / L.rows[0];
         return L;
     }
     const int n = (h + one - 1) / one;
-    L.rows[0] = std::max(8, int(int64_t(h) * (four ? 75 : 90) / (100 * int64_t(n))));
+    L.rows[0] = std::max(8, int(int64_t(h) * 75 / (100 * int64_t(n))));
     L.count[0] = n;
     L.rows[1] = std::max(8, one / 4);
-    L.count[1] = four ? int(int64_t(h) * 15 / (100 * int64_t(L.rows[1]))) : 0;
+    L.count[1] = int(int64_t(h) * 15 / (100 * int64_t(L.rows[1])));
     L.rows[2] = std::max(8, one / 8);
     const int left = h - n * L.rows[0] - L.count[1] * L.rows[1];
     L.count[2] = std::max(0, (left + L.rows[2] - 1) / L.rows[2]);
@@ -421,7 +421,7 @@ static cudaError_t build_plan(lbm_ctx* c) {
             Wave wave = wave_of(aligned);
             if (c->tune_aligned < 0 && elem_size_storage(c->fmt) == 4 && wave.rows >= 16) wave = wave_of(aligned = 1);
             if (q == 0) c->i_aligned = aligned;
-            lev[q] = chunk_levels(c->fmt, h, wave, c->tune_chunk, interior_max_rows(c->fmt, c->pitch));
+            lev[q] = chunk_levels(h, wave, c->tune_chunk, interior_max_rows(c->fmt, c->pitch));
             c->i_chunk[q] = lev[q].rows[0];
             levels |= lev[q].count[1] + lev[q].count[2] > 0;
             nitems += interior_items(r, q, strips[q], lev[q], nullptr, 0);

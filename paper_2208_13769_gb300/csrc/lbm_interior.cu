@@ -139,8 +139,9 @@ __host__ __device__ constexpr int ring_depth(int ring_slots) { return ring_slots
 // extrapolated scheme, whose carries are E = u(t) + F (the u* of stage A, in
 // the u-carry planes), D = ku jh(t) and F = ku (3 jh(t) - jh(t - dt)) (in
 // the source planes); else u* is A + ku m and the source planes hold the
-// last source.
-template <class TS, class TC, class UT, int NT, bool XJ, bool UNROLL3, bool REV>
+// last source.  PAIRS: FP32 operations by pairs in one instruction, where both
+// components of the displacement are FP32 pairs.
+template <class TS, class TC, class UT, int NT, bool XJ, bool UNROLL3, bool REV, bool PAIRS>
 __device__ __forceinline__ bool interior_tile(const StepParams& p, const InteriorMaps* maps, const TileGeom& tg,
                                               int bx, int y_begin, int y_end, double* fields) {
     using Slot = RingSlot<TS, TC, UT, NT, XJ>;
@@ -159,6 +160,9 @@ __device__ __forceinline__ bool interior_tile(const StepParams& p, const Interio
 
     LatConsts<TC> k;
     k.load(p);
+    // u* then lies by words: the high words of both components, the low ones
+    constexpr bool PK = PAIRS && sizeof(TC) == 4 && UT::layout != kCarryOne && !XJ;
+    float2* su2 = reinterpret_cast<float2*>(su);
     const int64_t pitch = p.pitch, plane = p.plane;
     const int t = threadIdx.x;
     const int rx0 = tg.rect[0], rx1 = tg.rect[1];
@@ -277,7 +281,13 @@ __device__ __forceinline__ bool interior_tile(const StepParams& p, const Interio
             const unsigned char* slot = ring + ra * Slot::BYTES;
             const unsigned char* pf = slot + e_own;
 #pragma unroll
-            for (int i = 0; i < 9; ++i) gcur[i] = Codec<TS, TC>::ld(Slot::pop(pf, i), i, p);
+            for (int i = 0; i < 9; ++i) {
+                if constexpr (PK && sizeof(TS) == 2)
+                    gcur[i] = float(Slot::pop(pf, i));
+                else
+                    gcur[i] = Codec<TS, TC>::ld(Slot::pop(pf, i), i, p);
+            }
+            if constexpr (PK && sizeof(TS) == 2) scale9(gcur, p.dec_scale);
             if constexpr (sizeof(TC) == 8) {  // FP64 keeps them as sums and differences of opposite ones
                 double f[9];
 #pragma unroll
@@ -290,15 +300,22 @@ __device__ __forceinline__ bool interior_tile(const StepParams& p, const Interio
                 su[(sA * 2 + 1) * NT + t] = A1;
             } else {
                 const TC* g = gcur;
-                TC m0, m1;
-                if constexpr (sizeof(TC) == 8) {
-                    momentum64(g, m0, m1);
+                if constexpr (PK) {
+                    const float2 D = sub2(f2(g[1], g[2]), f2(g[3], g[4]));
+                    const float2 m = add2(add2(D, f2(g[5] - g[6], g[5] - g[8])), f2(g[8] - g[7], g[6] - g[7]));
+                    su2[(sA * 2) * NT + t] = f2(A0.hi, A1.hi);
+                    su2[(sA * 2 + 1) * NT + t] = add2(f2(A0.lo, A1.lo), product2(f2(k.ku), m));
                 } else {
-                    m0 = (g[1] - g[3]) + (g[5] - g[6]) + (g[8] - g[7]);
-                    m1 = (g[2] - g[4]) + (g[5] - g[8]) + (g[6] - g[7]);
+                    TC m0, m1;
+                    if constexpr (sizeof(TC) == 8) {
+                        momentum64(g, m0, m1);
+                    } else {
+                        m0 = (g[1] - g[3]) + (g[5] - g[6]) + (g[8] - g[7]);
+                        m1 = (g[2] - g[4]) + (g[5] - g[8]) + (g[6] - g[7]);
+                    }
+                    su[(sA * 2) * NT + t] = A0.add(k.ku * m0);
+                    su[(sA * 2 + 1) * NT + t] = A1.add(k.ku * m1);
                 }
-                su[(sA * 2) * NT + t] = A0.add(k.ku * m0);
-                su[(sA * 2 + 1) * NT + t] = A1.add(k.ku * m1);
             }
         }
         __syncthreads();
@@ -314,10 +331,23 @@ __device__ __forceinline__ bool interior_tile(const StepParams& p, const Interio
             // the rows below and above (a - 2 sg and a in the walk)
             const UT* rm = su + ((rev ? sA : sC) * 2) * NT;
             const UT* rp = su + ((rev ? sC : sA) * 2) * NT;
-            const TC h11 = r0[tp].minus(r0[tm]) * k.inv_2dx;
-            const TC h21 = r0[NT + tp].minus(r0[NT + tm]) * k.inv_2dx;
-            const TC h12 = rp[t].minus(rm[t]) * k.inv_2dx;
-            const TC h22 = rp[NT + t].minus(rm[NT + t]) * k.inv_2dx;
+            TC h11, h12, h21, h22;
+            if constexpr (PK) {
+                const float2* q0 = reinterpret_cast<const float2*>(r0);
+                const float2* qm = reinterpret_cast<const float2*>(rm);
+                const float2* qp = reinterpret_cast<const float2*>(rp);
+                const float2 dx = add2(sub2(q0[tp], q0[tm]), sub2(q0[NT + tp], q0[NT + tm]));
+                const float2 dy = add2(sub2(qp[t], qm[t]), sub2(qp[NT + t], qm[NT + t]));
+                h11 = dx.x * k.inv_2dx;
+                h21 = dx.y * k.inv_2dx;
+                h12 = dy.x * k.inv_2dx;
+                h22 = dy.y * k.inv_2dx;
+            } else {
+                h11 = r0[tp].minus(r0[tm]) * k.inv_2dx;
+                h21 = r0[NT + tp].minus(r0[NT + tm]) * k.inv_2dx;
+                h12 = rp[t].minus(rm[t]) * k.inv_2dx;
+                h22 = rp[NT + t].minus(rm[NT + t]) * k.inv_2dx;
+            }
             TC q11, q12, q21, q22;
             const TC J = stress_remainder<TC>(h11, h12, h21, h22, k.lam, k.mu, q11, q12, q21, q22);
             bad |= not_positive(J);  // also catches a non-finite displacement gradient
@@ -381,42 +411,68 @@ __device__ __forceinline__ bool interior_tile(const StepParams& p, const Interio
                 TC dg;
                 collide64(f, j0, j1, sn0, sn1, k, fc, dg, r);
             } else {
-                // equilibrium, He forcing and BGK collision by opposite pairs
-                const TC tr15 = TC(1.5) * (pxx + pyy);
-                const TC E0 = TC(2) * r - tr15;
-                const TC Ex = TC(0.5) * r + TC(4.5) * pxx - tr15;
-                const TC Ey = TC(0.5) * r + TC(4.5) * pyy - tr15;
-                const TC Ed = -r + TC(4.5) * (pxx + pyy) - tr15;
-                const TC Ep = Ed + TC(9) * pxy, Em = Ed - TC(9) * pxy;
-                const TC w0 = wgt<TC>(0), w1 = wgt<TC>(1), w5 = wgt<TC>(5);
-                const TC b0 = TC(3) * (k.omega * j0 + k.force_pref * sn0);
-                const TC b1 = TC(3) * (k.omega * j1 + k.force_pref * sn1);
-                const TC ax = wmul<TS>(w1, k.omega * Ex), ay = wmul<TS>(w1, k.omega * Ey);
-                const TC ap = wmul<TS>(w5, k.omega * Ep), am = wmul<TS>(w5, k.omega * Em);
-                const TC bx = wmul<TS>(w1, b0), by = wmul<TS>(w1, b1);
-                const TC bp = wmul<TS>(w5, b0 + b1), bm = wmul<TS>(w5, b1 - b0);
-                fc[0] = k.one_m_omega * f[0] + wmul<TS>(w0, k.omega * E0);
-                fc[1] = k.one_m_omega * f[1] + (ax + bx);
-                fc[3] = k.one_m_omega * f[3] + (ax - bx);
-                fc[2] = k.one_m_omega * f[2] + (ay + by);
-                fc[4] = k.one_m_omega * f[4] + (ay - by);
-                fc[5] = k.one_m_omega * f[5] + (ap + bp);
-                fc[7] = k.one_m_omega * f[7] + (ap - bp);
-                fc[6] = k.one_m_omega * f[6] + (am + bm);
-                fc[8] = k.one_m_omega * f[8] + (am - bm);
+                if constexpr (PK) {
+                    collide2<TS>(f, r, pxx, pyy, pxy, f2(j0, j1), f2(sn0, sn1), k, fc);
+                } else {
+                    // equilibrium, He forcing and BGK collision by opposite pairs
+                    const TC tr15 = TC(1.5) * (pxx + pyy);
+                    const TC E0 = TC(2) * r - tr15;
+                    const TC Ex = TC(0.5) * r + TC(4.5) * pxx - tr15;
+                    const TC Ey = TC(0.5) * r + TC(4.5) * pyy - tr15;
+                    const TC Ed = -r + TC(4.5) * (pxx + pyy) - tr15;
+                    const TC Ep = Ed + TC(9) * pxy, Em = Ed - TC(9) * pxy;
+                    const TC w0 = wgt<TC>(0), w1 = wgt<TC>(1), w5 = wgt<TC>(5);
+                    const TC b0 = TC(3) * (k.omega * j0 + k.force_pref * sn0);
+                    const TC b1 = TC(3) * (k.omega * j1 + k.force_pref * sn1);
+                    const TC ax = wmul<TS>(w1, k.omega * Ex), ay = wmul<TS>(w1, k.omega * Ey);
+                    const TC ap = wmul<TS>(w5, k.omega * Ep), am = wmul<TS>(w5, k.omega * Em);
+                    const TC bx = wmul<TS>(w1, b0), by = wmul<TS>(w1, b1);
+                    const TC bp = wmul<TS>(w5, b0 + b1), bm = wmul<TS>(w5, b1 - b0);
+                    fc[0] = k.one_m_omega * f[0] + wmul<TS>(w0, k.omega * E0);
+                    fc[1] = k.one_m_omega * f[1] + (ax + bx);
+                    fc[3] = k.one_m_omega * f[3] + (ax - bx);
+                    fc[2] = k.one_m_omega * f[2] + (ay + by);
+                    fc[4] = k.one_m_omega * f[4] + (ay - by);
+                    fc[5] = k.one_m_omega * f[5] + (ap + bp);
+                    fc[7] = k.one_m_omega * f[7] + (ap - bp);
+                    fc[6] = k.one_m_omega * f[6] + (am + bm);
+                    fc[8] = k.one_m_omega * f[8] + (am - bm);
+                }
             }
+            if constexpr (PK && sizeof(TS) == 2) scale9(fc, p.enc_scale);
             const uint32_t o = off_a - 2 * dpitch;  // row a - 2 sg = gy
 #pragma unroll
-            for (int i = 0; i < 9; ++i) *elem(fd[i], o) = Codec<TS, TC>::st(fc[i], i, p);
+            for (int i = 0; i < 9; ++i) {
+                if constexpr (PK && sizeof(TS) == 2)
+                    *elem(fd[i], o) = TS(fc[i]);  // scaled above
+                else
+                    *elem(fd[i], o) = Codec<TS, TC>::st(fc[i], i, p);
+            }
 
             // carries: A' = u + ku (jh + s/2), u = u* + du;  s' = s
             // (XJ: E' = u + ku (3 jh - jh(t)) = E - F + 4 D', D' = ku jh,
             // F' = 3 D' - D)
-            const UT ux = su[(sC * 2) * NT + t], uy = su[(sC * 2 + 1) * NT + t];
+            UT ux, uy;
+            if constexpr (PK) {
+                const float2 uh = su2[(sC * 2) * NT + t], ul = su2[(sC * 2 + 1) * NT + t];
+                ux = UT{uh.x, ul.x};
+                uy = UT{uh.y, ul.y};
+            } else {
+                ux = su[(sC * 2) * NT + t];
+                uy = su[(sC * 2 + 1) * NT + t];
+            }
+            UT A0, A1;
             const TC ka0 = XJ ? k.ku * j0 : k.ku * (j0 + TC(0.5) * sn0);
             const TC ka1 = XJ ? k.ku * j1 : k.ku * (j1 + TC(0.5) * sn1);
-            const UT A0 = XJ ? ux.add(TC(4) * ka0 - fo0).renorm() : ux.add(du0 + ka0).renorm();
-            const UT A1 = XJ ? uy.add(TC(4) * ka1 - fo1).renorm() : uy.add(du1 + ka1).renorm();
+            if constexpr (PK) {
+                float2 hi = f2(ux.hi, uy.hi), lo = add2(f2(ux.lo, uy.lo), f2(du0 + ka0, du1 + ka1));
+                renorm2(hi, lo);
+                A0 = UT{hi.x, lo.x};
+                A1 = UT{hi.y, lo.y};
+            } else {
+                A0 = XJ ? ux.add(TC(4) * ka0 - fo0).renorm() : ux.add(du0 + ka0).renorm();
+                A1 = XJ ? uy.add(TC(4) * ka1 - fo1).renorm() : uy.add(du1 + ka1).renorm();
+            }
             auto put = [o](auto* at, auto v) { *elem(at, o) = v; };
             UT::store(A0, A1, ad0, ad1, p, put);
             *elem(sd[0], o) = XJ ? ka0 : sn0;
@@ -502,9 +558,9 @@ __global__ void __launch_bounds__(NT, MINB)
     const bool up = it.rows < 0;
     const int y1 = it.y0 + (up ? -it.rows : it.rows);
     if (alternate_walk<UNROLL3>() && up)
-        interior_tile<TS, TC, UT, NT, XJ, UNROLL3, true>(p, &maps, tg, it.strip, it.y0, y1, p.fields);
+        interior_tile<TS, TC, UT, NT, XJ, UNROLL3, true, true>(p, &maps, tg, it.strip, it.y0, y1, p.fields);
     else
-        interior_tile<TS, TC, UT, NT, XJ, UNROLL3, false>(p, &maps, tg, it.strip, it.y0, y1, p.fields);
+        interior_tile<TS, TC, UT, NT, XJ, UNROLL3, false, true>(p, &maps, tg, it.strip, it.y0, y1, p.fields);
 }
 
 // The interiors of a batch of bodies for one time step: one CTA per interior
@@ -535,10 +591,14 @@ __global__ void __launch_bounds__(NT, MINB) batch_interior_kernel(const __grid_c
     const bool up = it.rows < 0;
     const int y1 = it.y0 + (up ? -it.rows : it.rows);
     double* fields = L.fields ? sp.fields : nullptr;
+    // with 16-bit storage pairs let a 7th CTA on the SM, which costs the long
+    // tiles more than they save (128 bodies of 64 to 512 nodes a side: 281 us a
+    // step, 270 without); FP32 32 bodies of 64 to 1024 244 and 246
+    constexpr bool kPairs = sizeof(TS) == 4;
     if (alternate_walk<UNROLL3>() && up)
-        interior_tile<TS, TC, UT, NT, false, UNROLL3, true>(sp, maps, tg, it.strip, it.y0, y1, fields);
+        interior_tile<TS, TC, UT, NT, false, UNROLL3, true, kPairs>(sp, maps, tg, it.strip, it.y0, y1, fields);
     else
-        interior_tile<TS, TC, UT, NT, false, UNROLL3, false>(sp, maps, tg, it.strip, it.y0, y1, fields);
+        interior_tile<TS, TC, UT, NT, false, UNROLL3, false, kPairs>(sp, maps, tg, it.strip, it.y0, y1, fields);
 }
 
 template <class TS, class TC, class UT, int NT, bool XJ>

@@ -186,6 +186,85 @@ struct LatConsts {
     }
 };
 
+// Two FP32 operations in one instruction (fma.rn.f32x2 and its kin), which
+// halves what the two cost of the issue slots that bound the interior kernel
+// with 16-bit storage: 1000 x 777 FP16 20.3 us a step and 19.2 so, 3000 x 2900
+// 147.8 and 143.3; FP32 waits for memory (800 x 700 16.1 and 15.8, 4096 x 2048
+// 162.4 and 161.9).  Each half is rounded as the scalar instruction is.  The
+// forms below spell out which products are fused with an addition, so that
+// the kernel keeps the bits of the scalar code (the edge kernel's).
+__device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
+__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, f2(-b.x, -b.y)); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+// a b rounded on its own, for add2: a mul2 is fused with the add2 that takes
+// it, in spite of the rounding modifiers of both
+__device__ __forceinline__ float2 product2(float2 a, float2 b) {
+    return f2(__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y));
+}
+// the nine populations times their scales (one for each weight)
+__device__ __forceinline__ void scale9(float* f, const float* scale) {
+    f[0] = __fmul_rn(f[0], scale[0]);
+#pragma unroll
+    for (int i = 1; i < 9; i += 2) {
+        const float2 v = mul2(f2(f[i], f[i + 1]), f2(scale[i < 5 ? 1 : 5]));
+        f[i] = v.x;
+        f[i + 1] = v.y;
+    }
+}
+// UPair::renorm of both components: hi the high words, lo the low ones
+__device__ __forceinline__ void renorm2(float2& hi, float2& lo) {
+    const float2 s = add2(hi, lo), b = sub2(s, hi);
+    lo = add2(sub2(hi, sub2(s, b)), sub2(lo, b));
+    hi = s;
+}
+// Equilibrium, He forcing and BGK collision in FP32, by pairs: directions (1,
+// 2) and their opposites (3, 4), (5, 6) and (7, 8); j, s: jh and s.
+template <class TS>
+__device__ __forceinline__ void collide2(const float* f, float r, float pxx, float pyy, float pxy, float2 j, float2 s,
+                                         const LatConsts<float>& k, float* fc) {
+    const float tr = __fadd_rn(pxx, pyy), hr = __fmul_rn(0.5f, r);
+    const float E0 = __fmaf_rn(-1.5f, tr, __fmul_rn(2.0f, r));
+    const float2 Exy = fma2(f2(-1.5f), f2(tr), add2(f2(hr), product2(f2(4.5f), f2(pxx, pyy))));
+    const float Ed = __fmaf_rn(-1.5f, tr, __fmaf_rn(4.5f, tr, -r));
+    const float2 Epm = f2(__fmaf_rn(9.0f, pxy, Ed), __fmaf_rn(-9.0f, pxy, Ed));
+    const float w0 = wgt<float>(0), w1 = wgt<float>(1), w5 = wgt<float>(5);
+    const float2 om = f2(k.omega), o1 = f2(k.one_m_omega);
+    const float2 b = mul2(f2(3.0f), fma2(f2(k.force_pref), s, mul2(om, j)));
+    const float2 bd = f2(__fadd_rn(b.x, b.y), __fsub_rn(b.y, b.x));
+    const float2 e1 = mul2(om, Exy), e5 = mul2(om, Epm);
+    const float e0 = __fmul_rn(k.omega, E0);
+    float2 p1, q1, p5, q5;  // w (omega E + b) and w (omega E - b)
+    if constexpr (sizeof(TS) == 4) {
+        auto wm = [](float w, float2 x) { return fma2(f2(w), x, mul2(f2(-w * 0x1p-27f), x)); };  // wmul
+        const float2 a1 = wm(w1, e1), a5 = wm(w5, e5), b1 = wm(w1, b), b5 = wm(w5, bd);
+        p1 = add2(a1, b1);
+        q1 = sub2(a1, b1);
+        p5 = add2(a5, b5);
+        q5 = sub2(a5, b5);
+        fc[0] = __fmaf_rn(k.one_m_omega, f[0], wmul<TS>(w0, e0));
+    } else {
+        const float2 b1 = mul2(f2(w1), b), b5 = mul2(f2(w5), bd);
+        p1 = fma2(f2(w1), e1, b1);
+        q1 = fma2(f2(w1), e1, f2(-b1.x, -b1.y));
+        p5 = fma2(f2(w5), e5, b5);
+        q5 = fma2(f2(w5), e5, f2(-b5.x, -b5.y));
+        fc[0] = __fmaf_rn(w0, e0, __fmul_rn(k.one_m_omega, f[0]));
+    }
+    const float2 c12 = fma2(o1, f2(f[1], f[2]), p1), c34 = fma2(o1, f2(f[3], f[4]), q1);
+    const float2 c56 = fma2(o1, f2(f[5], f[6]), p5), c78 = fma2(o1, f2(f[7], f[8]), q5);
+    fc[1] = c12.x;
+    fc[2] = c12.y;
+    fc[3] = c34.x;
+    fc[4] = c34.y;
+    fc[5] = c56.x;
+    fc[6] = c56.y;
+    fc[7] = c78.x;
+    fc[8] = c78.y;
+}
+
 // The FP64 collision on sums and differences of opposite populations, g =
 // {f0, f1 + f3, f2 + f4, f5 + f7, f6 + f8, f1 - f3, f2 - f4, f5 - f7, f6 -
 // f8}: the moments, equilibrium and forcing need only these, each pair's
