@@ -5,9 +5,8 @@
 // interior tiles of every member (one CTA per tile, longest first) on the
 // batch's stream, and the edge tiles of every member, each CTA reading its
 // member's parameters from a device table.  The edge launch runs on a side
-// stream at the same time, or, when some member's interior runs across a
-// periodic seam, after the interior launch with the seam-image copies
-// appended to it.
+// stream at the same time; when some member's interior runs across a periodic
+// seam, a launch of the seam-image copies follows the interior's.
 // So small and uneven bodies share the GPU instead of each paying launches
 // per step, and chunks of 64 steps replay as one CUDA graph.  Every node of
 // every member goes through the same tile code and arithmetic as when the

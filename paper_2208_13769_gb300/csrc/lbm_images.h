@@ -12,8 +12,9 @@ namespace lbm {
 // Along a periodic axis the 3 outer rows / columns of every state plane hold
 // copies of the nodes across the seam (lbm_params.h).  The edge kernel
 // writes the copies of the nodes it advances; where the interior kernel
-// advances the nodes next to a seam, CTAs of the edge launch that follows
-// the interior launch copy them.  A tile is a box of image positions [x0, x1) x [y0, y1) of one
+// advances the nodes next to a seam, CTAs of a launch of the edge kernel that
+// follows the interior launch (with the step's edge tiles, or of images alone)
+// copy them.  A tile is a box of image positions [x0, x1) x [y0, y1) of one
 // instance (entry of the parameter table), at most kImageThreads positions,
 // each copied from the node (x mod nx, y mod ny) in every plane of the
 // instance's destination state (populations, u-carry, source carry).
@@ -41,7 +42,7 @@ struct ImageLaunch {
 
 struct EdgeLaunch;
 // A step's edge tiles (n_edge of them, as launch_edge with mode 0) and its
-// seam images (n_img tiles, a device list indexing the same parameter table
+// seam images (n_edge may be 0; n_img tiles, a device list indexing the same parameter table
 // as the edge tiles, whose f_dst / a_dst / s_dst are the state being
 // written) in one launch, for a step whose interior kernel ran across a
 // periodic seam: it follows the interior launch on the same stream (the

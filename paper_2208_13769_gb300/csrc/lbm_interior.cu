@@ -710,10 +710,12 @@ int interior_occupancy_t(int ring_slots) {
 }
 
 // Per format: the minimum CTAs per SM (the register cap) and the row loop's
-// form, as measured on the 4096 x 2048 body: FP16 / BF16 gain 4.5 % from the
-// unrolled loop at 80 registers, plain-carry FP32 3 % at 72 registers (7
-// CTAs per SM); the compensated carry has no registers to spare and runs the
-// rotating loop (the unrolled one was 3 % slower at 80 registers).
+// form: FP16 / BF16 run the unrolled loop (72 registers, so 7 CTAs of one body
+// fit an SM; held to 6 by their shared memory, 1000 x 1000 with a hole took
+// 23.5 us a step instead of 22.4 and 2200 x 1800 69.7 instead of 72.8), plain-
+// carry FP32 too at 72 registers (3 % at 4096 x 2048); the compensated carry
+// has no registers to spare and runs the rotating loop (the unrolled one gained
+// nothing for one body and made batches slower).
 int interior_occupancy(int fmt, int ring_slots) {
     switch (fmt) {
         case kFmtF64: return interior_occupancy_t<double, double, UPlain<double>, 128, 3, false>(ring_slots);
