@@ -229,7 +229,8 @@ typedef struct {
 LBM_API lbm_status lbm_set_tuning(lbm_ctx* ctx, const lbm_tuning* tuning);
 
 /* The decomposition in use once the context has run (rows per CTA and ring
- * depth as planned), else the one requested. */
+ * depth as planned, by default at least 8 rows so that lbm_set_tuning takes
+ * them), else the one requested. */
 LBM_API lbm_status lbm_get_tuning(const lbm_ctx* ctx, lbm_tuning* tuning);
 
 /* Autotuner: times `steps` graph-replayed steps of scratch contexts with

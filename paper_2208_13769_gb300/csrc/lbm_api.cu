@@ -938,11 +938,15 @@ lbm_status lbm_step(lbm_ctx* c, int64_t nsteps) {
         --left;
         c->variant_warm = true;
     }
-    // a stream that the caller is capturing records up to kGraphChunk steps as
-    // plain launches (a second capture cannot begin on it)
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    LBM_CUDA(c, cudaStreamIsCapturing(c->stream, &capture));
-    const int shortest = capture == cudaStreamCaptureStatusNone ? kGraphShort : kGraphChunk;
+    // up to kGraphChunk steps are plain launches on a stream on which no capture
+    // can begin: one that the caller is capturing, or the legacy default stream
+    bool plain = left <= kGraphShort || c->stream == cudaStreamLegacy;
+    if (!plain) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        LBM_CUDA(c, cudaStreamIsCapturing(c->stream, &capture));
+        plain = capture != cudaStreamCaptureStatusNone;
+    }
+    const int shortest = plain ? kGraphChunk : kGraphShort;
     int64_t queued = 0;
     while (left > shortest) {
         const bool built = c->graph[c->parity] != nullptr || queued >= kGraphChunk || shortest == kGraphChunk;
@@ -1087,7 +1091,8 @@ lbm_status lbm_get_tuning(const lbm_ctx* c, lbm_tuning* t) {
     if (!c || !t) return LBM_E_INVALID;
     if (c->planned && c->has_interior) {
         t->ring_slots = c->i_ring;
-        t->chunk_rows = c->i_chunk[0];
+        // short tiles as the least that lbm_set_tuning takes
+        t->chunk_rows = c->tune_chunk > 0 ? c->i_chunk[0] : std::max(8, c->i_chunk[0]);
         t->aligned = c->i_aligned;
         t->plan = 2;
     } else {

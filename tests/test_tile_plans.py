@@ -54,6 +54,18 @@ def test_default_interior_plans_match_fixed_rows(nx, ny, storage, carry, scheme)
     _same(got, _run(prob, 18, storage, carry, scheme, lbm.lbm_tuning(0, 0, -1, 1)), storage, "edge tiles")
 
 
+def test_reported_tuning_of_short_tiles_is_accepted():
+    """The default plan of a short-tiled body, read back, sets another one's."""
+    prob = _problem(420, 400, MIXED)
+    with lbm.Body(prob, storage="f32") as a:
+        a.step(9)
+        used, ref = lbm.lbm_get_tuning(a.ctx), a.read()
+    assert used.plan == 2 and used.chunk_rows >= 8
+    with lbm.Body(prob, storage="f32", tuning=used) as b:
+        b.step(9)
+        _same(b.read(), ref, "f32", "read back")
+
+
 # band tiles of interior tiles' size (seams, a hole beside short tiles), and
 # the three tile shapes of bodies that run as edge tiles only
 @pytest.mark.parametrize("storage", ["f64", "f32", "f16"])
@@ -78,6 +90,16 @@ def test_graphs_of_both_lengths_match_single_steps(nx, ny):
                 b.step(1)
             assert lbm.lbm_get_info(a.ctx)[0] == lbm.lbm_get_info(b.ctx)[0]
             _same(a.read(), b.read(), "f32", n)
+
+
+def test_steps_on_the_legacy_stream_run():
+    """No capture begins on the legacy default stream (handle 1): its calls of
+    up to 64 steps are launches."""
+    prob = _problem(420, 400, MIXED)
+    with lbm.Body(prob, storage="f32", stream=1) as a, lbm.Body(prob, storage="f32") as b:
+        a.step(33)
+        b.step(33)
+        _same(a.read(), b.read(), "f32", "legacy stream")
 
 
 def test_steps_recorded_by_a_caller_replay():
