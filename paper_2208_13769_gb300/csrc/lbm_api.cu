@@ -19,14 +19,17 @@ using namespace lbm;
 namespace {
 
 // Steps per captured graph, a long and a short one (even: they keep the
-// ping-pong parity).  A mid-size body's step is shorter than its launches take
-// the host (512 x 512 FP32 18.5 us a step launched one by one, 12.0 in a
-// graph), so at most a short graph's steps are launched so; about 9 us pass
-// between two graphs of two branches (0.5 us a step if all were short).  A long
-// graph takes the host 0.6 ms to build, which a body's first call now spends
-// with that many steps in short graphs queued (640 x 384 FP16, a new body of
-// 500 steps: 7.3 ms, 6.9 so).
+// ping-pong parity).  A small or mid-size body's step is shorter than its
+// launches take the host (512 x 512 FP32 18.5 us a step launched one by one,
+// 12.0 in a graph), so at most a short graph's steps are launched so; about 9
+// us pass between two graphs of two branches (0.5 us a step if all were short).
+// A long graph takes the host 0.6 ms to build, which a body's first call spends
+// with work queued: 64 steps in short graphs (640 x 384 FP16, a new body of 500
+// steps: 7.3 ms, 6.9 so), or of a larger body, whose steps outlast their
+// launches, 16 plain ones (4096 x 2048: 20 steps in 3.4 ms, 3.7 with a short
+// graph built first).
 constexpr int kGraphChunk = 64, kGraphShort = 16;
+constexpr int64_t kShortGraphNodes = int64_t(1) << 20;
 constexpr int kSegMax = 144;  // widest row segment the interior kernel copies in bulk (elements)
 
 size_t elem_size_storage(int fmt) {
@@ -325,6 +328,13 @@ int lbm::short_rows(int strips, int h, double sms) {
 // instead of levels (FP16 / plain / pair, levels and so: 2200 x 1800 95.4 /
 // 90.1 / 101.8 and 82.4 / 90.3 / 100.9, 3000 x 2900 187.7 / 183.3 / 207.3 and
 // 162.7 / 179.6 / 201.2).
+// A long wave of any format is cut into tiles of 18 rows: the tiles in work at
+// a time then lie in a band of a few hundred rows instead of all over the
+// body, which memory answers faster, and the launch ends evenly (levels and
+// so: 8192 x 8192 FP16 1288 and 985 us a step, lo16 1352 and 1145, 6000 x 6000
+// pair 741 and 671, plain 648 and 637; 10 to 22 rows within 3 %, 64 rows 1098
+// and 1263; below the lines, 4096 x 2048 FP16 134.4 and 137.9, 2200 x 1800
+// lo16 84.5 and 91.1).
 struct Wave {
     int rows;
     bool levels;
@@ -339,7 +349,9 @@ static Wave interior_wave(int fmt, bool xj, int h, int strips, int64_t share, do
     const bool four = xj || elem_size_storage(fmt) == 4;
     if (fmt == kFmtF64) return {std::max(one, 8), false};
     if (one <= 10) return {short_rows(strips, h, std::max(1.0, sms)), false};
-    if (one >= (four ? 28 : 48)) return xj ? Wave{20, false} : Wave{one, true};
+    if (one >= 28 && xj) return {20, false};
+    if (one >= (fmt == kFmtF32C || fmt == kFmtF32H ? 64 : 100)) return {18, false};
+    if (one >= (four ? 28 : 48)) return {one, true};
     return {four ? rows(std::min(share, int64_t(4.45 * sms))) : one, false};
 }
 
@@ -940,17 +952,25 @@ lbm_status lbm_step(lbm_ctx* c, int64_t nsteps) {
     }
     // up to kGraphChunk steps are plain launches on a stream on which no capture
     // can begin: one that the caller is capturing, or the legacy default stream
-    bool plain = left <= kGraphShort || c->stream == cudaStreamLegacy;
-    if (!plain) {
+    bool capturable = true, small = false;
+    if (left > kGraphShort) {
         cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-        LBM_CUDA(c, cudaStreamIsCapturing(c->stream, &capture));
-        plain = capture != cudaStreamCaptureStatusNone;
+        if (c->stream != cudaStreamLegacy) LBM_CUDA(c, cudaStreamIsCapturing(c->stream, &capture));
+        capturable = c->stream != cudaStreamLegacy && capture == cudaStreamCaptureStatusNone;
+        small = capturable && int64_t(c->nx) * c->ny < kShortGraphNodes;
     }
-    const int shortest = plain ? kGraphChunk : kGraphShort;
     int64_t queued = 0;
-    while (left > shortest) {
-        const bool built = c->graph[c->parity] != nullptr || queued >= kGraphChunk || shortest == kGraphChunk;
-        const int n = left > kGraphChunk && built ? kGraphChunk : kGraphShort;
+    while (left > (small ? kGraphShort : kGraphChunk)) {
+        const bool built =
+            c->graph[c->parity] != nullptr || !capturable || queued >= (small ? kGraphChunk : kGraphShort);
+        const int n = left > kGraphChunk && built ? kGraphChunk : small ? kGraphShort : 1;
+        if (n == 1) {
+            st = launch(c, 0, false);
+            if (st != LBM_OK) return st;
+            ++queued;
+            --left;
+            continue;
+        }
         cudaGraphExec_t g;
         st = get_graph(c, n, c->parity, &g);
         if (st != LBM_OK) return st;

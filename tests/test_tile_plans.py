@@ -40,12 +40,13 @@ def _same(got, ref, storage, what):
 
 # one full wave of 11 to 27 rows (4-byte storage: 4.45 tiles per SM), fewer
 # rows (short tiles), 28 and more (a wave with shorter tiles after it; the
-# extrapolated scheme: 20 rows), 48 and more in 16-bit storage, with the last
-# strip a few columns wide
+# extrapolated scheme: 20 rows), 48 and more in 16-bit storage, 64 and 100 and
+# more (18 rows), with the last strip a few columns wide
 @pytest.mark.parametrize("nx,ny,storage,carry,scheme", [
     (420, 400, "f32", True, 1), (640, 640, "f32", "lo16", 0), (1000, 140, "f16", None, 1), (700, 601, "f64", None, 1),
     (126, 7001, "f32", True, 1), (250, 7000, "f32", False, 1), (130, 13501, "f32", "lo16", 1), (130, 13501, "f32", True, 2),
-    (130, 13501, "f16", None, 2), (131, 23003, "f16", None, 1), (129, 23003, "bf16", None, 0)])
+    (130, 13501, "f16", None, 2), (131, 23003, "f16", None, 1), (129, 23003, "bf16", None, 0),
+    (130, 30011, "f32", "lo16", 1), (129, 54007, "f16", None, 0)])
 def test_default_interior_plans_match_fixed_rows(nx, ny, storage, carry, scheme):
     prob = _problem(nx, ny, W.clamped_free_edges())
     got = _run(prob, 18, storage, carry, scheme)
