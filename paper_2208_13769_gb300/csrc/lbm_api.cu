@@ -19,17 +19,18 @@ using namespace lbm;
 namespace {
 
 // Steps per captured graph, a long and a short one (even: they keep the
-// ping-pong parity).  A small or mid-size body's step is shorter than its
-// launches take the host (512 x 512 FP32 18.5 us a step launched one by one,
-// 12.0 in a graph), so at most a short graph's steps are launched so; about 9
-// us pass between two graphs of two branches (0.5 us a step if all were short).
-// A long graph takes the host 0.6 ms to build, which a body's first call spends
-// with work queued: 64 steps in short graphs (640 x 384 FP16, a new body of 500
-// steps: 7.3 ms, 6.9 so), or of a larger body, whose steps outlast their
-// launches, 16 plain ones (4096 x 2048: 20 steps in 3.4 ms, 3.7 with a short
-// graph built first).
+// ping-pong parity).  Steps launched one by one leave gaps between their two
+// streams, and a small body's are shorter than their launches take the host (a
+// step of 512 x 512 FP32 18.5 us so, 12.0 in a graph; 4096 x 2048 FP16 142 and
+// 134), so at most a short graph's steps are launched so where the graphs
+// exist; about 9 us pass between two graphs of two branches (0.5 us a step of
+// 512 x 512 if all were short).  A graph takes the host 9 us a step to build: a
+// body whose steps outlast that gets its graphs once 16 plain steps are queued
+// (4096 x 2048: 20 steps in 3.4 ms, 3.7 with a short graph built first), a
+// smaller one the short graph at once and the long one with 64 steps queued
+// (640 x 384 FP16, a new body of 500 steps: 7.3 ms, 6.9 so).
 constexpr int kGraphChunk = 64, kGraphShort = 16;
-constexpr int64_t kShortGraphNodes = int64_t(1) << 20;
+constexpr int64_t kShortGraphNodes = int64_t(1) << 20;  // a step of about 20 us
 constexpr int kSegMax = 144;  // widest row segment the interior kernel copies in bulk (elements)
 
 size_t elem_size_storage(int fmt) {
@@ -960,10 +961,14 @@ lbm_status lbm_step(lbm_ctx* c, int64_t nsteps) {
         small = capturable && int64_t(c->nx) * c->ny < kShortGraphNodes;
     }
     int64_t queued = 0;
-    while (left > (small ? kGraphShort : kGraphChunk)) {
-        const bool built =
-            c->graph[c->parity] != nullptr || !capturable || queued >= (small ? kGraphChunk : kGraphShort);
-        const int n = left > kGraphChunk && built ? kGraphChunk : small ? kGraphShort : 1;
+    while (left > (capturable ? kGraphShort : kGraphChunk)) {
+        const int q = c->parity;
+        int n = 1;
+        if (left > kGraphChunk &&
+            (c->graph[q] != nullptr || !capturable || queued >= (small ? kGraphChunk : kGraphShort)))
+            n = kGraphChunk;
+        else if (c->graph_short[q] != nullptr || small || queued >= kGraphShort)
+            n = kGraphShort;
         if (n == 1) {
             st = launch(c, 0, false);
             if (st != LBM_OK) return st;
