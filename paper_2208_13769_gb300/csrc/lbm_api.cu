@@ -367,15 +367,11 @@ static Wave interior_wave(int fmt, bool xj, int h, int strips, int64_t share, do
 // waits less for memory and gains from 48 rows on: 3000 x 2900 152 us with 90 %
 // in the wave and 143 so; at 2500 x 1300 60.9 either way.  FP64 is bound by its
 // arithmetic (1500 x 1000: 506 us, 507 in levels).
-static ChunkLevels chunk_levels(int h, Wave wave, int tune_chunk, int max_rows) {
+static ChunkLevels chunk_levels(int h, Wave wave, int tune_chunk) {
+    const int one = wave.rows;
+    if (tune_chunk > 0 || !wave.levels) return equal_chunks(h, tune_chunk > 0 ? tune_chunk : one);
     ChunkLevels L;
     memset(&L, 0, sizeof(L));
-    const int one = wave.rows;
-    if (tune_chunk > 0 || !wave.levels || one > max_rows) {
-        L.rows[0] = std::min(tune_chunk > 0 ? tune_chunk : one, std::min(h, max_rows));
-        L.count[0] = (h + L.rows[0] - 1) / L.rows[0];
-        return L;
-    }
     const int n = (h + one - 1) / one;
     L.rows[0] = std::max(8, int(int64_t(h) * 75 / (100 * int64_t(n))));
     L.count[0] = n;
@@ -434,7 +430,7 @@ static cudaError_t build_plan(lbm_ctx* c) {
             Wave wave = wave_of(aligned);
             if (c->tune_aligned < 0 && elem_size_storage(c->fmt) == 4 && wave.rows >= 16) wave = wave_of(aligned = 1);
             if (q == 0) c->i_aligned = aligned;
-            lev[q] = chunk_levels(h, wave, c->tune_chunk, interior_max_rows(c->fmt, c->pitch));
+            lev[q] = bounded_chunks(chunk_levels(h, wave, c->tune_chunk), h, interior_max_rows(c->fmt, c->pitch));
             c->i_chunk[q] = lev[q].rows[0];
             levels |= lev[q].count[1] + lev[q].count[2] > 0;
             nitems += interior_items(r, q, strips[q], lev[q], nullptr, 0);

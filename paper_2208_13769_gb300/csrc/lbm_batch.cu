@@ -167,17 +167,13 @@ lbm_status batch_graph(lbm_batch* b, int q, cudaGraphExec_t* out) {
 // rows) 247 us a step with chunks of 32 rows and 243 so, 12 of 128 to 2048 in
 // FP16 (185) 367 and 347, 20 of 64 to 700 in FP16 (35) 110 and 93, 6 of 64 to
 // 400 in FP32 (5) 36 and 23.
-ChunkLevels batch_levels(int h, int tune_chunk, double one, int64_t all, int sms, int max_rows) {
-    ChunkLevels L;
-    memset(&L, 0, sizeof(L));
+ChunkLevels batch_levels(int h, int tune_chunk, double one, int64_t all, int sms) {
     int rows = tune_chunk;
     if (rows == 0 && one < 10) rows = short_rows(1, int(all), sms);
-    if (rows > 0) {
-        L.rows[0] = std::min(rows, max_rows);
-        L.count[0] = (h + L.rows[0] - 1) / L.rows[0];
-        return L;
-    }
-    auto part = [&](double f) { return std::max(8, int(std::min(f * one, double(max_rows)))); };
+    if (rows > 0) return equal_chunks(h, rows);
+    ChunkLevels L;
+    memset(&L, 0, sizeof(L));
+    auto part = [&](double f) { return std::max(8, int(std::min(f * one, double(1 << 20)))); };
     L.rows[0] = std::min(part(0.75), h);
     L.rows[1] = part(0.5);
     L.rows[2] = part(1.0 / 3);
@@ -344,8 +340,8 @@ lbm_status lbm_batch_create_tuned(lbm_ctx* const* members, int32_t n, void* cuda
                 if (q < mri.n_irect) {
                     const int e = int(ent.size()) - 1;
                     const int h = p.rect[3] - p.rect[2];
-                    const ChunkLevels lev =
-                        batch_levels(h, b->chunk_rows, one, all_interior / 120, sms, interior_max_rows(b->fmt, c->pitch));
+                    const ChunkLevels lev = bounded_chunks(batch_levels(h, b->chunk_rows, one, all_interior / 120, sms), h,
+                                                           interior_max_rows(b->fmt, c->pitch));
                     const int64_t cnt = interior_items(mri.irect[q], e, ns, lev, nullptr, 0);
                     const size_t at = items.size();
                     items.resize(at + size_t(cnt));

@@ -812,14 +812,6 @@ cudaError_t interior_maps(int fmt, bool xj, const void* f, const void* a, const 
     return ok ? cudaSuccess : cudaErrorNotSupported;
 }
 
-// The widest element of a plane that interior_tile addresses by a 32-bit
-// byte offset is 8 bytes in FP64 and 4 otherwise; a tile spans its rows and
-// 4 more.
-int interior_max_rows(int fmt, int64_t pitch) {
-    const int64_t row = pitch * (fmt == kFmtF64 ? 8 : 4);
-    return int(std::max<int64_t>(8, (int64_t(1) << 32) / row - 8));
-}
-
 cudaError_t launch_interior(int fmt, const StepParams& p0, const InteriorRects& R, const InteriorMaps& maps, cudaStream_t s,
                             bool fields) {
     StepParams p = p0;

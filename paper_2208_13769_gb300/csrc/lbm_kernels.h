@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include "lbm_params.h"
+#include "lbm_tile_rows.h"
 
 namespace lbm {
 
@@ -59,11 +60,6 @@ struct InteriorRects {
     const InteriorItem* items;  // device list, one per CTA
     int32_t total;
 };
-// The rows of a rectangle as chunks: count[k] chunks of rows[k] rows for each
-// level k in turn (the last of them clipped to the rectangle).
-struct ChunkLevels {
-    int32_t rows[4], count[4];
-};
 // The tiles of a rectangle: its chunks in order, every strip of each; chunks
 // of odd index walk up, so that the chunks on either side of a boundary read
 // its halo rows together.  Returns their number (written to out, at most cap,
@@ -81,9 +77,10 @@ struct alignas(128) InteriorMaps {
 // The maps of the state (f, a, s); xj: of the extrapolated scheme.
 cudaError_t interior_maps(int fmt, bool xj, const void* f, const void* a, const void* s, int64_t pitch, int64_t plane,
                           int ny, InteriorMaps* out);
-// The most rows an interior tile may have at this pitch (its byte offsets
-// are 32-bit).
-int interior_max_rows(int fmt, int64_t pitch);
+// The most rows an interior tile of this format may have at this pitch.
+inline int interior_max_rows(int fmt, int64_t pitch) {
+    return interior_max_rows(pitch, fmt == kFmtF64 ? 8 : 4, kInteriorThreads);
+}
 // One step of the interior: a launch of R.total CTAs over the rectangles.
 cudaError_t launch_interior(int fmt, const StepParams& p, const InteriorRects& R, const InteriorMaps& maps, cudaStream_t s,
                             bool fields);
