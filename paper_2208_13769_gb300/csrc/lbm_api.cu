@@ -407,7 +407,7 @@ static cudaError_t build_plan(lbm_ctx* c) {
     c->n_items = 0;
     if (c->n_irect > 0) {
         c->i_ring = c->tune_ring ? c->tune_ring : kInteriorRing;
-        const int per_sm = std::max(1, interior_occupancy(c->fmt, c->i_ring));
+        const int per_sm = std::max(1, interior_occupancy(c->fmt, c->scheme == LBM_SCHEME_EXTRAPOLATED, c->i_ring));
         const int64_t slots = int64_t(c->num_sms) * per_sm;
         const int64_t all_area = interior_nodes(c);
         int strips[4];
@@ -1097,7 +1097,7 @@ lbm_status lbm_set_tuning(lbm_ctx* c, const lbm_tuning* t) {
     if (!c || !t) return LBM_E_INVALID;
     if (c->sticky) return LBM_E_CUDA;
     if (c->planned) return LBM_E_STATE;
-    if ((t->ring_slots != 0 && (t->ring_slots < 4 || t->ring_slots > 8)) ||
+    if ((t->ring_slots != 0 && (t->ring_slots < 4 || t->ring_slots > kMaxRing)) ||
         (t->chunk_rows != 0 && (t->chunk_rows < 8 || t->chunk_rows > (1 << 20))) || t->aligned < -1 ||
         t->aligned > 2 || t->plan < 0 || t->plan > 2)
         return LBM_E_INVALID;

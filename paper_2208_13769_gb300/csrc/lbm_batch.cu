@@ -218,7 +218,7 @@ lbm_status lbm_batch_create_tuned(lbm_ctx* const* members, int32_t n, void* cuda
     if (!out) return LBM_E_INVALID;
     *out = nullptr;
     if (!members || n < 1) return LBM_E_INVALID;
-    if (tuning && ((tuning->ring_slots != 0 && (tuning->ring_slots < 4 || tuning->ring_slots > 8)) ||
+    if (tuning && ((tuning->ring_slots != 0 && (tuning->ring_slots < 4 || tuning->ring_slots > kMaxRing)) ||
                    (tuning->chunk_rows != 0 && (tuning->chunk_rows < 8 || tuning->chunk_rows > (1 << 20))) ||
                    tuning->aligned < -1 || tuning->aligned > 2))
         return LBM_E_INVALID;

@@ -607,16 +607,20 @@ size_t interior_smem_bytes(int ring_slots) {
            size_t(RingSlot<TS, TC, UT, NT, XJ>::BYTES) * size_t(ring_depth(ring_slots));
 }
 
+// The kernel's limit of dynamic shared memory, on the current device, that of
+// the deepest ring: the same whatever ring a body or a batch runs with, so that
+// planning one never lowers it under another's launches, on any device and from
+// any thread.  (A launch takes what its own ring needs.)
+template <class TS, class TC, class UT, int NT, bool XJ, class Kernel>
+cudaError_t allow_any_ring(Kernel kern) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                int(interior_smem_bytes<TS, TC, UT, NT, XJ>(kMaxRing)));
+}
+
 template <class TS, class TC, class UT, int NT, int MINB, bool UNROLL3, bool XJ>
 cudaError_t launch_interior_x(const StepParams& p, const InteriorRects& R, const InteriorMaps& maps, cudaStream_t s) {
     auto kern = interior_step_kernel<TS, TC, UT, NT, MINB, XJ, UNROLL3>;
     const size_t sm = interior_smem_bytes<TS, TC, UT, NT, XJ>(p.ring_slots);
-    static size_t configured = 0;
-    if (sm > configured) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
-        if (e != cudaSuccess) return e;
-        configured = sm;
-    }
     if (R.total <= 0) return cudaSuccess;
     kern<<<R.total, NT, sm, s>>>(p, R, maps);
     return cudaGetLastError();
@@ -634,15 +638,10 @@ template <class TS, class TC, class UT, int NT, int MINB, bool UNROLL3>
 cudaError_t launch_batch_interior_t(const BatchInteriorLaunch& L, int ring_slots, cudaStream_t s, int* resident) {
     auto kern = batch_interior_kernel<TS, TC, UT, NT, MINB, UNROLL3>;
     const size_t sm = interior_smem_bytes<TS, TC, UT, NT, false>(ring_slots);
-    static size_t configured = 0;
-    if (sm > configured) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
-        if (e != cudaSuccess) return e;
-        configured = sm;
-    }
     if (resident) {  // CTAs per SM of this kernel with this ring
         *resident = 0;
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(resident, kern, NT, sm);
+        cudaError_t e = allow_any_ring<TS, TC, UT, NT, false>(kern);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(resident, kern, NT, sm);
         if (e != cudaSuccess) return e;
     }
     if (L.nitems <= 0) return cudaSuccess;
@@ -699,14 +698,19 @@ void interior_strips(int fmt, int rx0, int rx1, int aligned, int* strip_x0, int*
     *nstrips = (rx1 - xg + W - 1) / W;  // the first and last strips may be partial
 }
 
+// (of the kernel of the other schemes for the extrapolated one too: the plans'
+// figures stand for it)
 template <class TS, class TC, class UT, int NT, int MINB, bool UNROLL3>
-int interior_occupancy_t(int ring_slots) {
+int interior_occupancy_t(bool xj, int ring_slots) {
     auto kern = interior_step_kernel<TS, TC, UT, NT, MINB, false, UNROLL3>;
-    const size_t sm = interior_smem_bytes<TS, TC, UT, NT, false>(ring_slots);
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm)) != cudaSuccess) return 0;
+    cudaError_t e = allow_any_ring<TS, TC, UT, NT, false>(kern);
+    if (e == cudaSuccess && xj)
+        e = allow_any_ring<TS, TC, UT, NT, true>(interior_step_kernel<TS, TC, UT, NT, MINB, true, false>);
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, NT, sm) != cudaSuccess) return 0;
-    return n;
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, NT,
+                                                          interior_smem_bytes<TS, TC, UT, NT, false>(ring_slots));
+    return e == cudaSuccess ? n : 0;
 }
 
 // Per format: the minimum CTAs per SM (the register cap) and the row loop's
@@ -716,14 +720,14 @@ int interior_occupancy_t(int ring_slots) {
 // carry FP32 too at 72 registers (3 % at 4096 x 2048); the compensated carry
 // has no registers to spare and runs the rotating loop (the unrolled one gained
 // nothing for one body and made batches slower).
-int interior_occupancy(int fmt, int ring_slots) {
+int interior_occupancy(int fmt, bool xj, int ring_slots) {
     switch (fmt) {
-        case kFmtF64: return interior_occupancy_t<double, double, UPlain<double>, 128, 3, false>(ring_slots);
-        case kFmtF32: return interior_occupancy_t<float, float, UPlain<float>, 128, 7, true>(ring_slots);
-        case kFmtF32C: return interior_occupancy_t<float, float, UComp, 128, 6, false>(ring_slots);
-        case kFmtF32H: return interior_occupancy_t<float, float, UCompH, 128, 6, false>(ring_slots);
-        case kFmtF16: return interior_occupancy_t<__half, float, UComp, 128, 6, true>(ring_slots);
-        default: return interior_occupancy_t<__nv_bfloat16, float, UComp, 128, 6, true>(ring_slots);
+        case kFmtF64: return interior_occupancy_t<double, double, UPlain<double>, 128, 3, false>(xj, ring_slots);
+        case kFmtF32: return interior_occupancy_t<float, float, UPlain<float>, 128, 7, true>(xj, ring_slots);
+        case kFmtF32C: return interior_occupancy_t<float, float, UComp, 128, 6, false>(xj, ring_slots);
+        case kFmtF32H: return interior_occupancy_t<float, float, UCompH, 128, 6, false>(xj, ring_slots);
+        case kFmtF16: return interior_occupancy_t<__half, float, UComp, 128, 6, true>(xj, ring_slots);
+        default: return interior_occupancy_t<__nv_bfloat16, float, UComp, 128, 6, true>(xj, ring_slots);
     }
 }
 

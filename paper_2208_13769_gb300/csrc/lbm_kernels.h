@@ -25,13 +25,15 @@ enum Format : int {
 // has kInteriorThreads threads, one per column of its strip and halo.
 constexpr int kInteriorThreads = 128;
 // CTAs of the interior kernel resident per SM with this ring (0 on error);
-// also sets the kernel's dynamic shared-memory limit, so call it before any
-// stream capture.
-int interior_occupancy(int fmt, int ring_slots);
+// also sets the kernel's dynamic shared-memory limit on the current device (xj:
+// that of the extrapolated scheme's kernel too), so each context calls it
+// before its first launch_interior and before any stream capture.
+int interior_occupancy(int fmt, bool xj, int ring_slots);
 // Rows of the interior kernel's ring by default, those in flight and the one
 // in work (4 measured fastest for single bodies and for batches).
 constexpr int kInteriorRing = 4;
 constexpr int kBatchRing = 4;
+constexpr int kMaxRing = 8;
 // The strip grid of the interior kernel over columns [rx0, rx1): origin of
 // strip 0, output columns per strip, number of strips.  aligned 1: the
 // fewest strips of equal width (at most 120 columns, 112 for 16-bit storage)
@@ -95,9 +97,10 @@ struct BatchInteriorLaunch {
     int32_t fields;            // also write u, v, r to params.fields
     int32_t nitems;            // tiles in the list
 };
-// The setting of the dynamic shared-memory limit happens on the first call
-// (also with nitems == 0), which must precede any stream capture; resident
-// (may be NULL) receives the kernel's CTAs per SM with this ring.
+// resident (may be NULL) receives the kernel's CTAs per SM with this ring; a
+// call with it sets the kernel's dynamic shared-memory limit on the current
+// device, so each batch makes one (nitems may be 0) before its first launch and
+// before any stream capture.
 cudaError_t launch_batch_interior(int fmt, const BatchInteriorLaunch& L, int ring_slots, cudaStream_t s,
                                   int* resident);
 
