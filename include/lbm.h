@@ -156,7 +156,8 @@ LBM_API lbm_status lbm_set_boundary(lbm_ctx* ctx, int32_t edge, int32_t kind, co
 LBM_API lbm_status lbm_set_hole(lbm_ctx* ctx, const int32_t hole[4], const double traction[8]);
 
 /* Advances nsteps (>= 0) time steps (Algorithm 1, one iteration each) on
- * the context's stream, replayed as CUDA graphs of 64 steps for long runs.
+ * the context's stream, more than a few as CUDA graphs of 16 and 64 steps, or,
+ * while the caller is capturing that stream, recorded as plain launches.
  * A step is the fused stream-collide-constitutive update in one launch of
  * the interior kernel and one of the edge tiles on a side stream (or the
  * edge tiles alone for a small body), plus, where the interior kernel runs

@@ -645,22 +645,10 @@ static lbm_status get_graph(lbm_ctx* c, int n, int par, cudaGraphExec_t* out) {
         *out = slot;
         return LBM_OK;
     }
-    cudaGraph_t g = nullptr;
-    LBM_CUDA(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
-    cudaError_t err = cudaSuccess;
-    for (int k = 0; k < n && err == cudaSuccess; ++k) err = launch_step_kernels(c, 0, false, par ^ (k & 1));
-    cudaError_t e2 = cudaStreamEndCapture(c->stream, &g);
-    if (err != cudaSuccess) {
-        if (g) cudaGraphDestroy(g);
-        return ctx_fail_cuda(c, err);
-    }
-    if (e2 != cudaSuccess) return ctx_fail_cuda(c, e2);
-    cudaGraphExec_t ex = nullptr;
-    err = cudaGraphInstantiate(&ex, g, 0);
-    cudaGraphDestroy(g);
-    if (err != cudaSuccess) return ctx_fail_cuda(c, err);
-    slot = ex;
-    *out = ex;
+    LBM_CUDA(c, build_graph(&c->stream, c->owns_stream, n, &slot, [&](int k) {
+                 return launch_step_kernels(c, 0, false, par ^ (k & 1));
+             }));
+    *out = slot;
     return LBM_OK;
 }
 
@@ -733,7 +721,6 @@ lbm_status lbm_create(const lbm_desc* d, lbm_ctx** out) {
     }
     c->stream = static_cast<cudaStream_t>(d->cuda_stream);
     if (!c->stream) {
-        // graphs cannot be captured on the legacy default stream: own one
         if (cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking) != cudaSuccess) {
             cudaGetLastError();
             delete c;
@@ -947,21 +934,14 @@ lbm_status lbm_step(lbm_ctx* c, int64_t nsteps) {
         --left;
         c->variant_warm = true;
     }
-    // up to kGraphChunk steps are plain launches on a stream on which no capture
-    // can begin: one that the caller is capturing, or the legacy default stream
-    bool capturable = true, small = false;
-    if (left > kGraphShort) {
-        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-        if (c->stream != cudaStreamLegacy) LBM_CUDA(c, cudaStreamIsCapturing(c->stream, &capture));
-        capturable = c->stream != cudaStreamLegacy && capture == cudaStreamCaptureStatusNone;
-        small = capturable && int64_t(c->nx) * c->ny < kShortGraphNodes;
-    }
+    bool graphs = false;
+    if (left > kGraphShort) LBM_CUDA(c, stream_takes_graphs(c->stream, &graphs));
+    const bool small = int64_t(c->nx) * c->ny < kShortGraphNodes;
     int64_t queued = 0;
-    while (left > (capturable ? kGraphShort : kGraphChunk)) {
+    while (graphs && left > kGraphShort) {
         const int q = c->parity;
         int n = 1;
-        if (left > kGraphChunk &&
-            (c->graph[q] != nullptr || !capturable || queued >= (small ? kGraphChunk : kGraphShort)))
+        if (left > kGraphChunk && (c->graph[q] != nullptr || queued >= (small ? kGraphChunk : kGraphShort)))
             n = kGraphChunk;
         else if (c->graph_short[q] != nullptr || small || queued >= kGraphShort)
             n = kGraphShort;

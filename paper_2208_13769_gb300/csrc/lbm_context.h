@@ -162,4 +162,43 @@ lbm_status ctx_check_flag(lbm_ctx* c);
 // of h rows in `strips` strips on `sms` SMs.
 int short_rows(int strips, int h, double sms);
 
+// Whether step graphs can be built and launched on stream s now: not while the
+// caller is capturing it (its steps are then recorded as plain launches).
+inline cudaError_t stream_takes_graphs(cudaStream_t s, bool* yes) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    const cudaError_t e = s == cudaStreamLegacy ? cudaSuccess : cudaStreamIsCapturing(s, &capture);
+    *yes = e == cudaSuccess && capture == cudaStreamCaptureStatusNone;
+    return e;
+}
+
+// Builds the graph of n steps, enqueued on *stream by step(0), ..., step(n - 1).
+// The capture runs on a non-blocking stream of the library's, which *stream
+// names meanwhile: no capture can begin on the legacy default stream, and one
+// on a blocking stream of the caller's would make other threads' work on the
+// legacy stream fail.
+template <class Step>
+cudaError_t build_graph(cudaStream_t* stream, bool owned, int n, cudaGraphExec_t* out, Step&& step) {
+    const cudaStream_t callers = *stream;
+    cudaStream_t own = callers;
+    cudaError_t err = cudaSuccess;
+    if (!owned) err = cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking);
+    cudaGraph_t g = nullptr;
+    cudaGraphExec_t ex = nullptr;
+    if (err == cudaSuccess) {
+        *stream = own;
+        err = cudaStreamBeginCapture(own, cudaStreamCaptureModeThreadLocal);
+        if (err == cudaSuccess) {
+            for (int k = 0; k < n && err == cudaSuccess; ++k) err = step(k);
+            const cudaError_t end = cudaStreamEndCapture(own, &g);
+            if (err == cudaSuccess) err = end;
+        }
+        *stream = callers;
+        if (!owned) cudaStreamDestroy(own);
+    }
+    if (err == cudaSuccess) err = cudaGraphInstantiate(&ex, g, 0);
+    if (g) cudaGraphDestroy(g);
+    if (err == cudaSuccess) *out = ex;
+    return err;
+}
+
 }  // namespace lbm
