@@ -175,18 +175,22 @@ inline cudaError_t stream_takes_graphs(cudaStream_t s, bool* yes) {
 // The capture runs on a non-blocking stream of the library's, which *stream
 // names meanwhile: no capture can begin on the legacy default stream, and one
 // on a blocking stream of the caller's would make other threads' work on the
-// legacy stream fail.
+// legacy stream fail.  The thread's capture mode is relaxed meanwhile: a caller
+// may be capturing a stream that this work is not on, which an instantiation
+// in another mode would invalidate.
 template <class Step>
 cudaError_t build_graph(cudaStream_t* stream, bool owned, int n, cudaGraphExec_t* out, Step&& step) {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaError_t err = cudaThreadExchangeStreamCaptureMode(&mode);
+    if (err != cudaSuccess) return err;
     const cudaStream_t callers = *stream;
     cudaStream_t own = callers;
-    cudaError_t err = cudaSuccess;
     if (!owned) err = cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking);
     cudaGraph_t g = nullptr;
     cudaGraphExec_t ex = nullptr;
     if (err == cudaSuccess) {
         *stream = own;
-        err = cudaStreamBeginCapture(own, cudaStreamCaptureModeThreadLocal);
+        err = cudaStreamBeginCapture(own, cudaStreamCaptureModeRelaxed);
         if (err == cudaSuccess) {
             for (int k = 0; k < n && err == cudaSuccess; ++k) err = step(k);
             const cudaError_t end = cudaStreamEndCapture(own, &g);
@@ -197,6 +201,7 @@ cudaError_t build_graph(cudaStream_t* stream, bool owned, int n, cudaGraphExec_t
     }
     if (err == cudaSuccess) err = cudaGraphInstantiate(&ex, g, 0);
     if (g) cudaGraphDestroy(g);
+    cudaThreadExchangeStreamCaptureMode(&mode);
     if (err == cudaSuccess) *out = ex;
     return err;
 }

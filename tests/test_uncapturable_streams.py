@@ -63,7 +63,7 @@ def test_building_graphs_leaves_other_threads_legacy_work_alone():
     torch.zeros(1, device="cuda")
     h = ctypes.c_void_p()
     assert cuda.cuStreamCreate(ctypes.byref(h), 0) == 0  # CU_STREAM_DEFAULT: blocking
-    stop, errors, launches = threading.Event(), [], [0]
+    stop, running, errors, launches = threading.Event(), threading.Event(), [], [0]
 
     def work():
         x = torch.zeros(1000, device="cuda")
@@ -71,12 +71,14 @@ def test_building_graphs_leaves_other_threads_legacy_work_alone():
             while not stop.is_set():
                 x.add_(1.0)
                 launches[0] += 1
+                running.set()
         except Exception as e:  # noqa: BLE001
             errors.append(e)
 
     t = threading.Thread(target=work)
     t.start()
     try:
+        assert running.wait(60)  # its kernel is loaded
         with lbm.Body(_prob(70, 60), storage="f32") as b:
             b.step(200)
             ref = b.read()
@@ -90,3 +92,29 @@ def test_building_graphs_leaves_other_threads_legacy_work_alone():
         assert cuda.cuStreamDestroy_v2(h) == 0
     assert not errors, errors
     assert launches[0] > 100
+
+
+@pytest.mark.parametrize("mode", ["relaxed", "thread_local", "global"])
+@pytest.mark.parametrize("own", [True, False])
+@pytest.mark.parametrize("n", [20, 200])
+def test_building_graphs_inside_a_capture_of_another_stream(mode, own, n):
+    """A body steps on its own stream (the library's or the caller's) while the
+    thread captures another one: neither disturbs the other."""
+    import torch
+    s, t = torch.cuda.Stream(), torch.cuda.Stream()
+    x = torch.zeros(10, device="cuda")
+    with lbm.Body(_prob(420, 400), storage="f32", stream=0 if own else t.cuda_stream) as a, \
+            lbm.Body(_prob(420, 400), storage="f32") as b:
+        a.step(5)  # the plan's allocations come before the capture
+        lbm.lbm_sync(a.ctx)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s, capture_error_mode=mode):
+            x.add_(1.0)
+            a.step(n)
+            x.add_(1.0)
+        b.step(5 + n)
+        _same(a.read(), b.read())
+        with torch.cuda.stream(s):
+            g.replay()
+        s.synchronize()
+        assert float(x[0]) == 2.0
