@@ -140,22 +140,9 @@ lbm_status batch_graph(lbm_batch* b, int q, cudaGraphExec_t* out) {
         *out = b->graph[q];
         return LBM_OK;
     }
-    cudaGraph_t g = nullptr;
-    BATCH_CUDA(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-    cudaError_t err = cudaSuccess;
-    for (int k = 0; k < kBatchGraphChunk && err == cudaSuccess; ++k) err = batch_launch(b, q ^ (k & 1), false);
-    const cudaError_t e2 = cudaStreamEndCapture(b->stream, &g);
-    if (err != cudaSuccess) {
-        if (g) cudaGraphDestroy(g);
-        return batch_fail(b, err);
-    }
-    if (e2 != cudaSuccess) return batch_fail(b, e2);
-    cudaGraphExec_t ex = nullptr;
-    err = cudaGraphInstantiate(&ex, g, 0);
-    cudaGraphDestroy(g);
-    if (err != cudaSuccess) return batch_fail(b, err);
-    b->graph[q] = ex;
-    *out = ex;
+    BATCH_CUDA(b, build_graph(&b->stream, b->owns_stream, kBatchGraphChunk, &b->graph[q],
+                              [&](int k) { return batch_launch(b, q ^ (k & 1), false); }));
+    *out = b->graph[q];
     return LBM_OK;
 }
 
@@ -475,7 +462,9 @@ lbm_status lbm_batch_step(lbm_batch* b, int64_t nsteps) {
         --left;
         b->warm = true;
     }
-    while (left > kBatchGraphChunk) {
+    bool graphs = false;
+    if (left > kBatchGraphChunk) BATCH_CUDA(b, stream_takes_graphs(b->stream, &graphs));
+    while (graphs && left > kBatchGraphChunk) {
         cudaGraphExec_t g;
         const lbm_status st = batch_graph(b, int(b->steps & 1), &g);
         if (st != LBM_OK) return st;

@@ -118,3 +118,50 @@ def test_building_graphs_inside_a_capture_of_another_stream(mode, own, n):
             g.replay()
         s.synchronize()
         assert float(x[0]) == 2.0
+
+
+@pytest.mark.parametrize("n", [66, 150])
+def test_long_batch_calls_on_the_legacy_stream(n):
+    probs = [_prob(200, 130, 1), _prob(131, 90, 2)]
+    bodies = [lbm.Body(p, storage="f32", stream=1) for p in probs]
+    others = [lbm.Body(p, storage="f32") for p in probs]
+    try:
+        with lbm.Batch(bodies, stream=1) as a, lbm.Batch(others) as b:
+            for k in (n, 3, n):
+                a.step(k)
+                b.step(k)
+            a.sync()
+            b.sync()
+        for x, y in zip(bodies, others):
+            _same(x.read(), y.read())
+    finally:
+        for x in bodies + others:
+            x.close()
+
+
+@pytest.mark.parametrize("before", [6, 200])
+def test_long_batch_calls_recorded_by_a_caller(before):
+    import torch
+    s = torch.cuda.Stream()
+    probs = [_prob(200, 130, 1), _prob(131, 90, 2)]
+    bodies = [lbm.Body(p, storage="f32", stream=s.cuda_stream) for p in probs]
+    others = [lbm.Body(p, storage="f32") for p in probs]
+    try:
+        with lbm.Batch(bodies, stream=s.cuda_stream) as a, lbm.Batch(others) as b:
+            a.step(before)
+            a.sync()
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=s, capture_error_mode="thread_local"):
+                a.step(150)
+            with torch.cuda.stream(s):
+                g.replay()
+            s.synchronize()
+            a.step(100)
+            b.step(before + 250)
+            a.sync()
+            b.sync()
+        for x, y in zip(bodies, others):
+            _same(x.read(), y.read())
+    finally:
+        for x in bodies + others:
+            x.close()
