@@ -270,11 +270,13 @@ void lbm::plan_rects(const lbm_ctx* c, bool edge_only, bool seams_inside, int ir
 // Otherwise a tile is bound by latency and the waves of 3 CTAs per SM decide:
 // 12 x 12 where they are fewer (301 x 203 in FP32: 442 tiles instead of 561,
 // 7.6 us instead of 9.9; 350 x 350: 12.4 and 14.0), else 28 x 4 (256 x 256,
-// two waves of either: 9.2 and 9.0).
+// two waves of either: 9.2 and 9.0), but with a hole, whose tiles are uneven,
+// 12 x 12 again if there are several waves (300 x 300 10.1 us, 10.4 with 28 x 4;
+// FP16 10.3 and 10.7).
 static EdgeShape edge_shape(const lbm_ctx* c) {
     const EdgeShape shapes[3] = {kEdgeWide, {kEdgeThreads, 16}, {kEdgeThreads / 2, 8}};
     const int64_t ops[3] = {570, 830, 320};
-    const bool f64 = c->fmt == kFmtF64;
+    const bool f64 = c->fmt == kFmtF64, hole = c->hole[0] < c->hole[1];
     EdgeShape best = kEdgeWide;
     int64_t least = INT64_MAX;
     for (int k = 0; k < (f64 ? 3 : 2); ++k) {
@@ -282,7 +284,7 @@ static EdgeShape edge_shape(const lbm_ctx* c) {
         for (int b = 0; b < c->nband; ++b)
             n += edge_tiles_of_rect(c->brect[b], 0, nullptr, 0, false, shapes[k], bounded_sides(c, c->brect[b]));
         const int64_t per = int64_t(c->num_sms) * (f64 ? 1 : 3), cost = (n + per - 1) / per * (f64 ? ops[k] : 1);
-        if (cost < least) {
+        if (cost < least || (cost == least && cost > 1 && hole && !f64)) {
             least = cost;
             best = shapes[k];
         }

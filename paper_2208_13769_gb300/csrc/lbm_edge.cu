@@ -29,12 +29,6 @@ static_assert(sizeof(StepParams) % 16 == 0, "StepParams is copied to shared memo
 template <class TS, class TC, class UT, int MODE, bool HOLE, bool XJ>
 __global__ void __launch_bounds__(kEdgeThreads, sizeof(TC) == 8 ? 2 : 3)
     edge_tile_kernel(const __grid_constant__ EdgeLaunch L, const __grid_constant__ ImageLaunch I) {
-    // the next launch may start; in FP64 only once this one is done, so that
-    // its tiles find the SMs free (started early, two of them share an SM's
-    // FP64 units while others idle: 64 x 64 in 12.8 us a step, 6.7 so, 8.0
-    // without the overlap)
-    constexpr bool early = sizeof(TC) == 4;
-    if (early) grid_launch_dependents();
     constexpr int N = kEdgeThreads;
     static_assert(kImageThreads <= N, "an image tile fits an edge CTA");
     if (I.tiles != nullptr && int(blockIdx.x) >= I.n_edge) {  // a seam-image CTA (uniform per CTA)
@@ -77,7 +71,11 @@ __global__ void __launch_bounds__(kEdgeThreads, sizeof(TC) == 8 ? 2 : 3)
     __syncthreads();
     edge_tile_body<TS, TC, UT, MODE, HOLE, XJ>(tile, sp, L.fields != 0, su, sq, MODE == 1 ? sinit : nullptr,
                                                 s_edge);
-    if (!early) grid_launch_dependents();
+    // the next launch may start (in FP32 edge_tile_body lets it earlier): in FP64
+    // only once this one is done, so that its tiles find the SMs free (started
+    // early, two of them share an SM's FP64 units while others idle: 64 x 64 in
+    // 12.8 us a step, 6.7 so, 8.0 without the overlap)
+    if (sizeof(TC) == 8) grid_launch_dependents();
 }
 
 // ---------------------------------------------------------------- launchers

@@ -162,15 +162,51 @@ __device__ __noinline__ void corner_link(TS* fdst, Geo g, const StepParams& p, c
     store_img(fdst + oi * g.plane, g, gx + ex(i), gy + ey(i), Codec<TS, TC>::st(val, oi, p));
 }
 
-// The boundary rules of Sec. 6 for a node on a bounded edge or next to the
-// hole, written into the ghost cells the links lead to.  edges: bits 0..3,
-// the node lies on x-, x+, y-, y+; faces: bits 0..3, next to the hole's face
-// at x0, x1, y0, y1; near_hole: within one node of the hole.  Out of line:
-// few nodes take it, and the tile's registers are spoken for.
+// A node's post-collision populations, moments and Q.
 template <class TC>
 struct BackNode {
     TC fc[9], r, pxx, pxy, pyy, q[4];
 };
+
+// Every link of node (gx, gy) into the hole: Eq. (abbcon) across the face it
+// crosses, or both faces at a corner.  In FP32 a tile waits for instructions
+// more than for arithmetic, and one small loop for all directions is faster
+// than code for each face (wall_links, which saves operations and is kept for
+// FP64): a 128 x 128 plate with a hole 7.9 us a step with that, 7.7 so.
+template <class TS, class TC>
+__device__ __forceinline__ void hole_links(TS* fdst, const Geo& g, const StepParams& p, int gx, int gy,
+                                           const BackNode<TC>& n, TC inv_c2) {
+#pragma unroll 1
+    for (int i = 1; i < 9; ++i) {
+        const int dx = gx + ex(i), dy = gy + ey(i);
+        if (!in_hole(p.hole, dx, dy)) continue;
+        const bool cx = ex(i) != 0 && in_hole(p.hole, dx, gy);
+        const bool cy = ey(i) != 0 && in_hole(p.hole, gx, dy);
+        const int sx = (cx || !cy) ? ex(i) : 0, sy = (cy || !cx) ? ey(i) : 0;
+        TC T0 = TC(0), T1 = TC(0);
+        if (sx != 0) {  // the face at x0 (entered along +x) or at x1
+            const int fa = sx > 0 ? 0 : 1;
+            T0 += TC(p.hole_T[2 * fa]);
+            T1 += TC(p.hole_T[2 * fa + 1]);
+        }
+        if (sy != 0) {  // the face at y0 or at y1
+            const int fa = sy > 0 ? 2 : 3;
+            T0 += TC(p.hole_T[2 * fa]);
+            T1 += TC(p.hole_T[2 * fa + 1]);
+        }
+        const TC inv_len = (sx != 0 && sy != 0) ? TC(0.70710678118654752440) : TC(1);
+        const TC val = abb_value<TS, TC>(i, n.fc[i], sx, sy, inv_len, T0, T1, n.r, n.pxx, n.pxy, n.pyy, n.q[0], n.q[1],
+                                         n.q[2], n.q[3], inv_c2);
+        const int oi = opp(i);
+        store_back(fdst + oi * g.plane, g, dx, dy, Codec<TS, TC>::st(val, oi, p));
+    }
+}
+
+// The boundary rules of Sec. 6 for a node on a bounded edge or next to the
+// hole, written into the ghost cells the links lead to.  edges: bits 0..3,
+// the node lies on x-, x+, y-, y+; faces: bits 0..3, next to the hole's face
+// at x0, x1, y0, y1; near_hole: within one node of the hole (then on no edge).
+// Out of line: few nodes take it, and the tile's registers are spoken for.
 template <class TS, class TC, class UT, bool HOLE>
 __device__ __noinline__ void boundary_links(TS* fdst, Geo g, const StepParams& p, const EdgeNow<TC, UT>* s_edge,
                                             int gx, int gy, unsigned edges, unsigned faces, bool near_hole,
@@ -189,6 +225,10 @@ __device__ __noinline__ void boundary_links(TS* fdst, Geo g, const StepParams& p
     if (exh) edge(P1(), Z0(), 1, !eyl, !eyh);
     if (eyl) edge(Z0(), M1(), 2, !exl, !exh);
     if (eyh) edge(Z0(), P1(), 3, !exl, !exh);
+    if (HOLE && sizeof(TC) == 4 && near_hole) {
+        hole_links<TS, TC>(fdst, g, p, gx, gy, n, inv_c2);
+        return;
+    }
     if (HOLE && near_hole) {
         auto face = [&](auto SX, auto SY, int fa) {
             constexpr int sx = decltype(SX)::value, sy = decltype(SY)::value;
@@ -261,6 +301,11 @@ __device__ __forceinline__ void edge_tile_body(const EdgeTile& tile, const StepP
     // is read here and used once stage A has issued its loads, so that the
     // two memory round trips overlap
     grid_wait();  // before the first read of what the previous step wrote
+    // the next launch may start now: not before this wait, which would let the
+    // one after it start too, and tiles of three steps then crowd some SMs while
+    // others run empty (an FP32 plate of 301 x 203 with a hole 10.3 us a step,
+    // 8.3 so; of 150 x 150 9.0 and 7.3; 256 x 256 8.2 either way)
+    if (sizeof(TC) == 4) grid_launch_dependents();
     int64_t n_now = 0;
     if (MODE == 0 && t < 4) n_now = p.counter[p.parity] + 1;
 
