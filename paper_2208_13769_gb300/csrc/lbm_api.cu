@@ -324,7 +324,11 @@ int lbm::short_rows(int strips, int h, double sms) {
 // and so: 1400 x 900 34.8 / 34.1 / 28.7 and 31.1 / 31.2 / 27.5, 1700 x 1438
 // 62.2 / 60.1 / 53.7 and 61.4 / 57.2 / 50.1; 2000 x 1500, 29 rows in the full
 // wave, 69.4 / 66.4 in levels and 73.9 / 68.7 so).  FP16 at 1400 x 900: 29.4
-// and 29.6.
+// and 29.6.  FP32 pairs, which move most bytes, gain from levels from 20 rows on
+// (2048 x 1024 56.4 and 52.1, 1536 x 1536 61.0 and 57.2, 1900 x 1500 71.1 and
+// 66.4; 1700 x 1500, periodic along y, 64.4 and 63.9; lo16 and plain carries
+// lose up to 3 and 8 % there, and so do pairs with a hole: 1600 x 1500 54.3 and
+// 58.6).
 // The extrapolated scheme keeps four more 4-byte carries and waits for memory
 // in every format: the same wave (FP16 1400 x 900 35.8 and 31.5, 1700 x 1438
 // 60.6 and 55.8), and where the full wave has 28 rows or more, chunks of 20
@@ -343,7 +347,7 @@ struct Wave {
     bool levels;
 };
 
-static Wave interior_wave(int fmt, bool xj, int h, int strips, int64_t share, double sms) {
+static Wave interior_wave(int fmt, bool xj, bool hole, int h, int strips, int64_t share, double sms) {
     auto rows = [&](int64_t ctas) {
         const int64_t per = std::max<int64_t>(1, ctas / strips);
         return int((h + per - 1) / per);
@@ -354,7 +358,7 @@ static Wave interior_wave(int fmt, bool xj, int h, int strips, int64_t share, do
     if (one <= 10) return {short_rows(strips, h, std::max(1.0, sms)), false};
     if (one >= 28 && xj) return {20, false};
     if (one >= (fmt == kFmtF32C || fmt == kFmtF32H ? 64 : 100)) return {18, false};
-    if (one >= (four ? 28 : 48)) return {one, true};
+    if (one >= (fmt == kFmtF32C && !xj && !hole ? 20 : (four ? 28 : 48))) return {one, true};
     return {four ? rows(std::min(share, int64_t(4.45 * sms))) : one, false};
 }
 
@@ -425,7 +429,7 @@ static cudaError_t build_plan(lbm_ctx* c) {
             // 55.8 us a step, 57.4 without; 2000 x 1500: 72.1 and 75.1)
             auto wave_of = [&](int aligned) {
                 interior_strips(c->fmt, r[0], r[1], aligned, &c->i_strip_x0[q], &c->i_strip_w[q], &strips[q]);
-                return interior_wave(c->fmt, c->scheme == LBM_SCHEME_EXTRAPOLATED, h, strips[q], share,
+                return interior_wave(c->fmt, c->scheme == LBM_SCHEME_EXTRAPOLATED, hole, h, strips[q], share,
                                      double(c->num_sms) * double(share) / double(slots));
             };
             int aligned = std::max(0, c->tune_aligned);
