@@ -334,7 +334,12 @@ int lbm::short_rows(int strips, int h, double sms) {
 // 60.6 and 55.8), and where the full wave has 28 rows or more, chunks of 20
 // instead of levels (FP16 / plain / pair, levels and so: 2200 x 1800 95.4 /
 // 90.1 / 101.8 and 82.4 / 90.3 / 100.9, 3000 x 2900 187.7 / 183.3 / 207.3 and
-// 162.7 / 179.6 / 201.2).
+// 162.7 / 179.6 / 201.2).  In FP32 pairs it is slower with one wave than it was
+// without the carries in the ring; with a ring of 5 rows (kDeepRing) and as few
+// whole waves of equal tiles as give them 20 rows or fewer it is not (one wave
+// before, these rules, and so: 1536 x 1536 66.4 / 67.5 / 65.2, 2048 x 1024 59.0
+// / 61.4 / 59.3, 1000 x 1000 34.4 / 35.6 / 28.5, 2200 x 1800 99.3 / 101.0 /
+// 98.3, 3000 x 2900 206 / 199 / 195).
 // A long wave of any format is cut into tiles of 18 rows: the tiles in work at
 // a time then lie in a band of a few hundred rows instead of all over the
 // body, which memory answers faster, and the launch ends evenly (levels and
@@ -342,12 +347,13 @@ int lbm::short_rows(int strips, int h, double sms) {
 // pair 741 and 671, plain 648 and 637; 10 to 22 rows within 3 %, 64 rows 1098
 // and 1263; below the lines, 4096 x 2048 FP16 134.4 and 137.9, 2200 x 1800
 // lo16 84.5 and 91.1).
+constexpr int kDeepRing = 5;
 struct Wave {
     int rows;
     bool levels;
 };
 
-static Wave interior_wave(int fmt, bool xj, bool hole, int h, int strips, int64_t share, double sms) {
+static Wave interior_wave(int fmt, bool xj, bool deep, bool hole, int h, int strips, int64_t share, double sms) {
     auto rows = [&](int64_t ctas) {
         const int64_t per = std::max<int64_t>(1, ctas / strips);
         return int((h + per - 1) / per);
@@ -355,6 +361,7 @@ static Wave interior_wave(int fmt, bool xj, bool hole, int h, int strips, int64_
     const int one = rows(share);
     const bool four = xj || elem_size_storage(fmt) == 4;
     if (fmt == kFmtF64) return {std::max(one, 8), false};
+    if (deep) return {rows(share * ((one + 19) / 20)), false};
     if (one <= 10) return {short_rows(strips, h, std::max(1.0, sms)), false};
     if (one >= 28 && xj) return {20, false};
     if (one >= (fmt == kFmtF32C || fmt == kFmtF32H ? 64 : 100)) return {18, false};
@@ -412,10 +419,17 @@ static cudaError_t build_plan(lbm_ctx* c) {
     std::unique_ptr<InteriorItem[]> items;
     c->n_items = 0;
     if (c->n_irect > 0) {
-        c->i_ring = c->tune_ring ? c->tune_ring : kInteriorRing;
-        const int per_sm = std::max(1, interior_occupancy(c->fmt, c->scheme == LBM_SCHEME_EXTRAPOLATED, c->i_ring));
-        const int64_t slots = int64_t(c->num_sms) * per_sm;
         const int64_t all_area = interior_nodes(c);
+        const bool xj = c->scheme == LBM_SCHEME_EXTRAPOLATED;
+        c->i_ring = c->tune_ring ? c->tune_ring : kInteriorRing;
+        // the extrapolated scheme in FP32 pairs moves most bytes a row: a deeper
+        // ring, of which 4 CTAs fit an SM, where they have 12 rows or more each
+        // (interior_wave; not with a hole: 1400 x 1000 38.2 us a step, 39.2 so)
+        if (c->tune_ring == 0 && xj && !hole && c->fmt == kFmtF32C && all_area >= int64_t(4 * 120 * 11) * c->num_sms)
+            c->i_ring = kDeepRing;
+        const bool deep = xj && !hole && c->fmt == kFmtF32C && c->i_ring == kDeepRing;
+        const int per_sm = std::max(1, interior_occupancy(c->fmt, xj, c->i_ring));
+        const int64_t slots = int64_t(c->num_sms) * per_sm;
         int strips[4];
         ChunkLevels lev[4];
         int64_t nitems = 0;
@@ -429,12 +443,13 @@ static cudaError_t build_plan(lbm_ctx* c) {
             // 55.8 us a step, 57.4 without; 2000 x 1500: 72.1 and 75.1)
             auto wave_of = [&](int aligned) {
                 interior_strips(c->fmt, r[0], r[1], aligned, &c->i_strip_x0[q], &c->i_strip_w[q], &strips[q]);
-                return interior_wave(c->fmt, c->scheme == LBM_SCHEME_EXTRAPOLATED, hole, h, strips[q], share,
+                return interior_wave(c->fmt, xj, deep, hole, h, strips[q], share,
                                      double(c->num_sms) * double(share) / double(slots));
             };
             int aligned = std::max(0, c->tune_aligned);
             Wave wave = wave_of(aligned);
-            if (c->tune_aligned < 0 && elem_size_storage(c->fmt) == 4 && wave.rows >= 16) wave = wave_of(aligned = 1);
+            if (c->tune_aligned < 0 && elem_size_storage(c->fmt) == 4 && (wave.rows >= 16 || deep))
+                wave = wave_of(aligned = 1);
             if (q == 0) c->i_aligned = aligned;
             lev[q] = bounded_chunks(chunk_levels(h, wave, c->tune_chunk), h, interior_max_rows(c->fmt, c->pitch));
             c->i_chunk[q] = lev[q].rows[0];

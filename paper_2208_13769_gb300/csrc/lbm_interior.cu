@@ -698,19 +698,21 @@ void interior_strips(int fmt, int rx0, int rx1, int aligned, int* strip_x0, int*
     *nstrips = (rx1 - xg + W - 1) / W;  // the first and last strips may be partial
 }
 
-// (of the kernel of the other schemes for the extrapolated one too: the plans'
-// figures stand for it)
-template <class TS, class TC, class UT, int NT, int MINB, bool UNROLL3>
-int interior_occupancy_t(bool xj, int ring_slots) {
-    auto kern = interior_step_kernel<TS, TC, UT, NT, MINB, false, UNROLL3>;
-    cudaError_t e = allow_any_ring<TS, TC, UT, NT, false>(kern);
-    if (e == cudaSuccess && xj)
-        e = allow_any_ring<TS, TC, UT, NT, true>(interior_step_kernel<TS, TC, UT, NT, MINB, true, false>);
+template <class TS, class TC, class UT, int NT, bool XJ, class Kernel>
+int interior_occupancy_k(Kernel kern, int ring_slots) {
     int n = 0;
+    cudaError_t e = allow_any_ring<TS, TC, UT, NT, XJ>(kern);
     if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, NT,
-                                                          interior_smem_bytes<TS, TC, UT, NT, false>(ring_slots));
+                                                          interior_smem_bytes<TS, TC, UT, NT, XJ>(ring_slots));
     return e == cudaSuccess ? n : 0;
+}
+template <class TS, class TC, class UT, int NT, int MINB, bool UNROLL3>
+int interior_occupancy_t(bool xj, int ring_slots) {
+    return xj ? interior_occupancy_k<TS, TC, UT, NT, true>(interior_step_kernel<TS, TC, UT, NT, MINB, true, false>,
+                                                           ring_slots)
+              : interior_occupancy_k<TS, TC, UT, NT, false>(interior_step_kernel<TS, TC, UT, NT, MINB, false, UNROLL3>,
+                                                            ring_slots);
 }
 
 // Per format: the minimum CTAs per SM (the register cap) and the row loop's

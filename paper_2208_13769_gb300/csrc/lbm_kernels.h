@@ -24,10 +24,10 @@ enum Format : int {
 // lie at least 2 nodes from bounded edges and 3 from periodic seams.  A CTA
 // has kInteriorThreads threads, one per column of its strip and halo.
 constexpr int kInteriorThreads = 128;
-// CTAs of the interior kernel resident per SM with this ring (0 on error);
-// also sets the kernel's dynamic shared-memory limit on the current device (xj:
-// that of the extrapolated scheme's kernel too), so each context calls it
-// before its first launch_interior and before any stream capture.
+// CTAs of the interior kernel (xj: of the extrapolated scheme's) resident per
+// SM with this ring (0 on error); also sets the kernel's dynamic shared-memory
+// limit on the current device, so each context calls it before its first
+// launch_interior and before any stream capture.
 int interior_occupancy(int fmt, bool xj, int ring_slots);
 // Rows of the interior kernel's ring by default, those in flight and the one
 // in work (4 measured fastest for single bodies and for batches).
