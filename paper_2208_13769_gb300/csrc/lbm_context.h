@@ -66,7 +66,7 @@ struct lbm_ctx {
     double* v0 = nullptr;
     unsigned char* arena = nullptr;  // device: f, a, s, fields, flag, counter, partials and diag lie in it
     int32_t* flag = nullptr;
-    int32_t* host_flag = nullptr;  // pinned: where the flag is read on the host
+    int32_t* host_flag = nullptr;  // pinned: the flag as of the last read, or none yet
     int64_t* counter = nullptr;
     double* partials = nullptr;
     double* diag = nullptr;
