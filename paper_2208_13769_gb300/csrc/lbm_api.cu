@@ -512,7 +512,7 @@ static cudaError_t build_plan(lbm_ctx* c) {
         image_tiles_of_body(c->nx, c->ny, perx, pery, box, 0, himg.get(), nimg);
     }
     StepParams hp[2] = {make_params(c, 0), make_params(c, 1)};
-    // one allocation and one copy for the lists and the parameters
+    // one place and one copy for the lists and the parameters
     const void* part[4] = {items.get(), h.get(), hp, himg.get()};
     const size_t bytes[4] = {sizeof(InteriorItem) * size_t(c->n_items), sizeof(EdgeTile) * size_t(ni), sizeof(hp),
                              sizeof(ImageTile) * size_t(nimg)};
@@ -524,14 +524,19 @@ static cudaError_t build_plan(lbm_ctx* c) {
         if (bytes[k] > 0) memcpy(host.get() + at[k], part[k], bytes[k]);
     cudaFree(c->plan);  // of an attempt that failed
     c->plan = nullptr;
-    cudaError_t e = cudaMalloc(&c->plan, at[4]);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(c->plan, host.get(), at[4], cudaMemcpyHostToDevice, c->stream);
+    unsigned char* to = c->plan_room;
+    cudaError_t e = cudaSuccess;
+    if (at[4] > c->plan_room_bytes) {
+        e = cudaMalloc(&c->plan, at[4]);
+        to = c->plan;
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(to, host.get(), at[4], cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);  // the host's copy is freed
     if (e != cudaSuccess) return e;
-    c->ditems = reinterpret_cast<InteriorItem*>(c->plan + at[0]);
-    c->dtiles = reinterpret_cast<EdgeTile*>(c->plan + at[1]);
-    c->dparams = reinterpret_cast<StepParams*>(c->plan + at[2]);
-    c->dimg = reinterpret_cast<ImageTile*>(c->plan + at[3]);
+    c->ditems = reinterpret_cast<InteriorItem*>(to + at[0]);
+    c->dtiles = reinterpret_cast<EdgeTile*>(to + at[1]);
+    c->dparams = reinterpret_cast<StepParams*>(to + at[2]);
+    c->dimg = reinterpret_cast<ImageTile*>(to + at[3]);
     c->n_img = nimg;
     c->n_etiles = n;
     c->n_itiles = hole ? ni : 0;
@@ -838,6 +843,17 @@ lbm_status lbm_create(const lbm_desc* d, lbm_ctx** out) {
     }
     const size_t at_fields = place(fldbytes), at_flag = place(sizeof(int32_t)), at_counter = place(2 * sizeof(int64_t)),
                  at_partials = place(size_t(c->diag_blocks) * 8 * sizeof(double)), at_diag = place(8 * sizeof(double));
+    // Room for the plan, so that the first step does not allocate: 28 bytes for
+    // 48 nodes or more of a body that runs as edge tiles only, which leaves
+    // enough for the tiles of larger ones without a hole.  (An allocation is
+    // cheap where another of less than 2 MB is alive and shares its block, else
+    // 30 to 85 us: 400 x 300 FP32 planned and initialised in 180 us with one,
+    // 123 so.  The initial fields of a body under 256 x 256 are such an
+    // allocation, and a plan of its own keeps their block: 64 x 64 97 and 37 us.)
+    const size_t initial = (d->u0 ? ubytes : 0) + (d->v0 ? ubytes : 0);
+    if (initial == 0 || initial >= size_t(2) << 20)
+        c->plan_room_bytes = 16384 + size_t(std::min<int64_t>(int64_t(nodes), int64_t(3) << 17)) * 3 / 4;
+    const size_t at_plan = place(c->plan_room_bytes);
     cudaError_t err = cudaMalloc(&c->arena, arena);
     if (err == cudaSuccess) {
         for (int k = 0; k < 2; ++k) {
@@ -850,6 +866,7 @@ lbm_status lbm_create(const lbm_desc* d, lbm_ctx** out) {
         c->counter = reinterpret_cast<int64_t*>(c->arena + at_counter);
         c->partials = reinterpret_cast<double*>(c->arena + at_partials);
         c->diag = reinterpret_cast<double*>(c->arena + at_diag);
+        c->plan_room = c->arena + at_plan;
     }
     if (err == cudaSuccess && (d->u0 || d->v0)) err = cudaMalloc(&c->initial, (d->u0 && d->v0 ? 2 : 1) * ubytes);
     if (err == cudaSuccess) {

@@ -64,7 +64,7 @@ struct lbm_ctx {
     double* initial = nullptr;  // u0 and v0, until the initialisation has read them
     double* u0 = nullptr;
     double* v0 = nullptr;
-    unsigned char* arena = nullptr;  // device: f, a, s, fields, flag, counter, partials and diag lie in it
+    unsigned char* arena = nullptr;  // device: f, a, s, fields, flag, counter, partials, diag and plan_room lie in it
     int32_t* flag = nullptr;
     int32_t* host_flag = nullptr;  // pinned: the flag as of the last read, or none yet
     int64_t* counter = nullptr;
@@ -99,7 +99,10 @@ struct lbm_ctx {
     int n_irect = 0;
     int irect[4][4];
     int i_chunk[4], i_strip_x0[4], i_strip_w[4];
-    unsigned char* plan = nullptr;        // device: ditems, dtiles, dparams and dimg lie in it
+    // device: ditems, dtiles, dparams and dimg lie in the arena's room for them,
+    // or, where they need more, in an allocation of their own
+    unsigned char *plan_room = nullptr, *plan = nullptr;
+    size_t plan_room_bytes = 0;
     lbm::InteriorItem* ditems = nullptr;  // device: the interior tiles
     int n_items = 0;
     int i_ring = 0, i_aligned = 0;
