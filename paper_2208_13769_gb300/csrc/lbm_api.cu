@@ -13,24 +13,12 @@
 #include "lbm_context.h"
 #include "lbm_init_grid.h"
 #include "lbm_kernels.h"
+#include "lbm_step_graphs.h"
 
 using namespace lbm;
 
 namespace {
 
-// Steps per captured graph, a long and a short one (even: they keep the
-// ping-pong parity).  Steps launched one by one leave gaps between their two
-// streams, and a small body's are shorter than their launches take the host (a
-// step of 512 x 512 FP32 18.5 us so, 12.0 in a graph; 4096 x 2048 FP16 142 and
-// 134), so at most a short graph's steps are launched so where the graphs
-// exist; about 9 us pass between two graphs of two branches (0.5 us a step of
-// 512 x 512 if all were short).  A graph takes the host 9 us a step to build: a
-// body whose steps outlast that gets its graphs once 16 plain steps are queued
-// (4096 x 2048: 20 steps in 3.4 ms, 3.7 with a short graph built first), a
-// smaller one the short graph at once and the long one with 64 steps queued
-// (640 x 384 FP16, a new body of 500 steps: 7.3 ms, 6.9 so).
-constexpr int kGraphChunk = 64, kGraphShort = 16;
-constexpr int64_t kShortGraphNodes = int64_t(1) << 20;  // a step of about 20 us
 constexpr int kSegMax = 144;  // widest row segment the interior kernel copies in bulk (elements)
 
 size_t elem_size_storage(int fmt) {
@@ -989,12 +977,8 @@ lbm_status lbm_step(lbm_ctx* c, int64_t nsteps) {
     const bool small = int64_t(c->nx) * c->ny < kShortGraphNodes;
     int64_t queued = 0;
     while (graphs && left > kGraphShort) {
-        const int q = c->parity;
-        int n = 1;
-        if (left > kGraphChunk && (c->graph[q] != nullptr || queued >= (small ? kGraphChunk : kGraphShort)))
-            n = kGraphChunk;
-        else if (c->graph_short[q] != nullptr || small || queued >= kGraphShort)
-            n = kGraphShort;
+        const int n = next_steps(left, queued, c->steps, small, c->graph[c->parity] != nullptr,
+                                 c->graph_short[c->parity] != nullptr);
         if (n == 1) {
             st = launch(c, 0, false);
             if (st != LBM_OK) return st;
