@@ -1176,8 +1176,9 @@ lbm_status lbm_autotune(const lbm_desc* d, const int32_t edge_kind[4], int64_t s
         if (st == LBM_OK) st = lbm_set_material(c, 0.3, 0.3, 1.0, 1.0, nullptr);
         for (int e = 0; e < 4 && st == LBM_OK; ++e)
             st = lbm_set_boundary(c, e, edge_kind[e], nullptr, nullptr, nullptr);
-        // warm: initialisation, a plain step, the graphs of both parities
-        if (st == LBM_OK) st = lbm_step(c, 2 * kGraphChunk + 2);
+        // warm: initialisation, plain steps, both graphs of the timed call's parity
+        if (st == LBM_OK) st = lbm_step(c, kWarmFirst);
+        if (st == LBM_OK) st = lbm_step(c, kWarmRest);
         double ms = INFINITY;
         if (st == LBM_OK) {
             DeviceGuard guard(c->device);

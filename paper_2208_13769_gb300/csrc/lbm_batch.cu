@@ -22,12 +22,13 @@
 #include "lbm.h"
 #include "lbm_context.h"
 #include "lbm_kernels.h"
+#include "lbm_step_graphs.h"
 
 using namespace lbm;
 
 namespace {
 
-constexpr int kBatchGraphChunk = 64;  // steps per captured graph (even)
+constexpr int kBatchGraphChunk = kGraphChunk;  // steps per captured graph (even)
 
 }  // namespace
 
@@ -602,8 +603,8 @@ lbm_status lbm_batch_autotune(lbm_ctx* const* members, int32_t n, int64_t steps,
             }
             lbm_batch* b = nullptr;
             status = lbm_batch_create_tuned(scratch.data(), n, st, &t, &b);
-            // warm: a plain step and the graphs of both parities
-            if (status == LBM_OK) status = lbm_batch_step(b, 2 * kBatchGraphChunk + 2);
+            // warm: a plain step and the graph of the timed call's parity
+            if (status == LBM_OK) status = lbm_batch_step(b, kBatchWarm);
             if (status == LBM_OK) status = lbm_batch_sync(b, nullptr);
             double ms = INFINITY;
             if (status == LBM_OK) {

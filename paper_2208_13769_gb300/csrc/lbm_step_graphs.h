@@ -35,4 +35,10 @@ inline int next_steps(int64_t left, int64_t queued, int64_t steps, bool small, b
     return 1;
 }
 
+// The autotuners' untimed calls: after kWarmFirst and then kWarmRest steps of a
+// new body, or kBatchWarm of a new batch (whose graphs take 64 steps each), the
+// graphs of the parity at which the timed call starts exist, and every longer
+// launch of it replays one.
+constexpr int64_t kWarmFirst = 2, kWarmRest = 3 * kGraphChunk + 2, kBatchWarm = 2 * kGraphChunk + 3;
+
 }  // namespace lbm
