@@ -403,6 +403,7 @@ static cudaError_t build_plan(lbm_ctx* c) {
     plan_rects(c, edge_only, seams_inside, c->irect, &c->n_irect, c->brect, &c->nband);
     const bool hole = c->hole[0] < c->hole[1];
     const bool perx = c->bc[0].kind == kPeriodic, pery = c->bc[2].kind == kPeriodic;
+    const bool images = seams_inside && (perx || pery);
     bool levels = false;  // shorter chunks after the interior's wave
     std::unique_ptr<InteriorItem[]> items;
     c->n_items = 0;
@@ -472,7 +473,7 @@ static cudaError_t build_plan(lbm_ctx* c) {
     // too in the launch that the image tiles share, whose CTAs are wide.
     const bool crowded =
         (levels && elem_size_storage(c->fmt) == 4) || c->i_chunk[0] <= (hole ? 20 : perx || pery ? 12 : 0);
-    c->edge_shape = !c->has_interior ? edge_shape(c) : crowded && !seams_inside ? kEdgeInterior : kEdgeWide;
+    c->edge_shape = !c->has_interior ? edge_shape(c) : crowded && !images ? kEdgeInterior : kEdgeWide;
     int n = 0;
     for (int b = 0; b < c->nband; ++b)
         n += edge_tiles_of_rect(c->brect[b], 0, nullptr, 0, false, c->edge_shape, bounded_sides(c, c->brect[b]));
@@ -491,7 +492,7 @@ static cudaError_t build_plan(lbm_ctx* c) {
     // the images of the interior's nodes next to a periodic seam
     int nimg = 0;
     std::unique_ptr<ImageTile[]> himg;
-    if (c->has_interior && seams_inside && (perx || pery)) {
+    if (c->has_interior && images) {
         int box[4];
         seam_box(c, box);
         nimg = image_tiles_of_body(c->nx, c->ny, perx, pery, box, 0, nullptr, 0);
