@@ -148,16 +148,22 @@ lbm_status batch_graph(lbm_batch* b, int q, cudaGraphExec_t* out) {
 }
 
 // The chunks of h rows of one member.  `one` is the rows per CTA if the batch
-// ran as one wave, `all` its rows over all strips.  As of a single long body,
+// ran as one wave, `all` its rows over all strips (in FP64, which is bound by
+// its operations, over full strips of its nodes).  As of a single long body,
 // most rows go to chunks of about a wave's rows and the rest to shorter ones,
-// which even out the end of the launch; fewer than 10 rows a wave are split as
-// a single short body's.  32 bodies of 64 to 1024 nodes a side in FP32 (93
-// rows) 247 us a step with chunks of 32 rows and 243 so, 12 of 128 to 2048 in
-// FP16 (185) 367 and 347, 20 of 64 to 700 in FP16 (35) 110 and 93, 6 of 64 to
-// 400 in FP32 (5) 36 and 23.
-ChunkLevels batch_levels(int h, int tune_chunk, double one, int64_t all, int sms) {
+// which even out the end of the launch; fewer than 12 rows a wave are split as
+// a single short body's, and short members of a batch of many, whose tiles even
+// out the end by themselves, into chunks of about 32 rows.  32 bodies of 64 to
+// 1024 nodes a side in FP32 (93 rows) 247 us a step with chunks of 32 rows and
+// 243 so, 12 of 128 to 2048 in FP16 (185) 367 and 347, 20 of 64 to 700 in FP16
+// (35) 110 and 92, 6 of 64 to 400 in FP32 (5) 36 and 21; 256 bodies of 32 to 128
+// nodes a side (22 rows) 122 us a step in FP32 lo16 in levels and 115 in chunks
+// of 32 rows, FP16 101 and 95; 128 of them (11 rows) in FP16 57 in such chunks
+// and 49 in short ones.
+ChunkLevels batch_levels(bool f64, int h, int tune_chunk, double one, int64_t all, int sms) {
     int rows = tune_chunk;
-    if (rows == 0 && one < 10) rows = short_rows(1, int(all), sms);
+    if (rows == 0 && one < 12) rows = short_rows(1, int(all), sms);
+    if (rows == 0 && !f64 && h <= 128 && one < 43) rows = (h + (h + 31) / 32 - 1) / ((h + 31) / 32);
     if (rows > 0) return equal_chunks(h, rows);
     ChunkLevels L;
     memset(&L, 0, sizeof(L));
@@ -275,17 +281,22 @@ lbm_status lbm_batch_create_tuned(lbm_ctx* const* members, int32_t n, void* cuda
         delete b;
         return LBM_E_OOM;
     }
-    int64_t all_interior = 0;
+    b->ring = tuning && tuning->ring_slots ? tuning->ring_slots : kBatchRing;
+    b->aligned = tuning && tuning->aligned >= 0 ? tuning->aligned : kBatchAligned;
+    const bool f64 = b->fmt == kFmtF64;
+    double all_rows = 0;  // of the interiors (batch_levels)
     for (int i = 0; i < n; ++i) {
         const lbm_ctx* c = b->m[size_t(i)];
         Rects& r = mr[size_t(i)];
         plan_rects(c, c->tune_plan == 1, true, r.irect, &r.n_irect, r.brect, &r.nband);
-        for (int k = 0; k < r.n_irect; ++k)
-            all_interior += int64_t(r.irect[k][1] - r.irect[k][0]) * (r.irect[k][3] - r.irect[k][2]);
+        for (int k = 0; k < r.n_irect; ++k) {
+            int x0, w, ns;
+            interior_strips(b->fmt, r.irect[k][0], r.irect[k][1], b->aligned, &x0, &w, &ns);
+            const int h = r.irect[k][3] - r.irect[k][2];
+            all_rows += f64 ? double(r.irect[k][1] - r.irect[k][0]) * h / 120.0 : double(ns) * h;
+        }
         b->holed = b->holed || c->hole[0] < c->hole[1];
     }
-    b->ring = tuning && tuning->ring_slots ? tuning->ring_slots : kBatchRing;
-    b->aligned = tuning && tuning->aligned >= 0 ? tuning->aligned : kBatchAligned;
     // the interior kernel's CTAs per SM with this ring (the first call also
     // sets its shared-memory limit, outside any capture)
     int resident = 0;
@@ -296,7 +307,7 @@ lbm_status lbm_batch_create_tuned(lbm_ctx* const* members, int32_t n, void* cuda
     }
     const int sms = b->m[0]->num_sms;
     b->chunk_rows = tuning ? tuning->chunk_rows : 0;
-    const double one = double(all_interior) / (120.0 * sms * std::max(1, resident));
+    const double one = all_rows / (double(sms) * std::max(1, resident));
     cudaError_t e_maps = cudaSuccess;
     std::vector<StepParams> tab;
     std::vector<InteriorMaps> maps;
@@ -328,8 +339,9 @@ lbm_status lbm_batch_create_tuned(lbm_ctx* const* members, int32_t n, void* cuda
                 if (q < mri.n_irect) {
                     const int e = int(ent.size()) - 1;
                     const int h = p.rect[3] - p.rect[2];
-                    const ChunkLevels lev = bounded_chunks(batch_levels(h, b->chunk_rows, one, all_interior / 120, sms), h,
-                                                           interior_max_rows(b->fmt, c->pitch));
+                    const ChunkLevels lev =
+                        bounded_chunks(batch_levels(f64, h, b->chunk_rows, one, int64_t(all_rows), sms), h,
+                                       interior_max_rows(b->fmt, c->pitch));
                     const int64_t cnt = interior_items(mri.irect[q], e, ns, lev, nullptr, 0);
                     const size_t at = items.size();
                     items.resize(at + size_t(cnt));
