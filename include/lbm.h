@@ -401,6 +401,14 @@ LBM_API lbm_status lbm_batch_destroy(lbm_batch* batch);
  * Errors: LBM_E_INVALID, LBM_E_OOM, LBM_E_CUDA. */
 LBM_API lbm_status lbm_selftest_bounded_wait(uint32_t polls, void* cuda_stream, int32_t* timed_out);
 
+/* Self-test of the FP64 arithmetic that the kernels do by hand (no counterpart
+ * in the paper), on `count` (1 .. 2^30) pseudo-random numbers of a seed: out[0]
+ * is the largest error of the reciprocal of J in units in the last place (below
+ * 0.57), out[1] the number of quotients of the read-out whose bits differ from
+ * the division's (0).  Allocates 16 device bytes; synchronises cuda_stream
+ * (NULL: legacy stream).  Errors: LBM_E_INVALID, LBM_E_OOM, LBM_E_CUDA. */
+LBM_API lbm_status lbm_selftest_quotients(int64_t count, uint64_t seed, void* cuda_stream, double out[2]);
+
 /* ------------------------------------------------------------------------
  * Allocation-free diagnostics (no counterpart in the paper).
  *

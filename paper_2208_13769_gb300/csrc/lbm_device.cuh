@@ -113,10 +113,13 @@ __device__ __forceinline__ T feq_odd_over_w(int i, T j0, T j1, T inv_c) {
 // 1 / J, J = det F near 1 for any admissible deformation.  FP32: the
 // hardware's approximate reciprocal, one instruction on the critical path of
 // stage B (its error, about an ulp, is far inside the FP32 path's
-// tolerance); FP64: the hardware's seed (20 bits or more) and one step of
-// Householder's third-order iteration, x (1 + e + e^2) with e = 1 - J x,
-// which leaves e^3 < 2^-60 and the roundings of three operations (the
-// correctly rounded reciprocal takes more than twice as many).
+// tolerance); FP64: the hardware's seed, which has 20 mantissa bits of the
+// reciprocal of J's first 20 and so an error below 2^-19, and one step of
+// Householder's third-order iteration, x (1 + e + e^2) with e = 1 - J x, which
+// leaves e^3 < 2^-57 and the roundings of three operations: below 0.57 units in
+// the last place (0.5084 at most over 2^29 values, lbm_selftest_quotients).  A
+// correction of the last bit takes two operations more and 1 to 3 % of the FP64
+// step, CUDA's correctly rounded reciprocal more than twice as many.
 __device__ __forceinline__ float rcp_j(float x) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -127,6 +130,20 @@ __device__ __forceinline__ double rcp_j(double x) {
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
     const double e = fma(-x, r, 1.0);
     return fma(r, fma(e, e, e), r);
+}
+
+// a / j for i = 1 / j (rounded to nearest): Markstein's correction of the
+// quotient a i by its residual, which rounds to nearest as the division does,
+// in 3 operations.  A zero is a i itself; infinities, NaN and what lies near
+// the ends of the exponents take the division.
+__device__ __forceinline__ double over(double a, double j, double i) {
+    const double q = a * i;
+    auto middle = [](double v) {  // 2^-500 < |v| < 2^500
+        return (unsigned(__double2hiint(v)) & 0x7fffffffu) - 0x20b00000u < 0x3e800000u;
+    };
+    const bool zero = ((unsigned(__double2hiint(a)) & 0x7fffffffu) | unsigned(__double2loint(a))) == 0;
+    if (!((middle(q) || zero) && middle(j))) return a / j;
+    return zero ? q : fma(fma(-q, j, a), i, q);
 }
 
 // !(J > 0), NaN included.  FP64: on the bits, since a comparison would take

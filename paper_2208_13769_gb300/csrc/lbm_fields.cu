@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include "lbm_device.cuh"
 #include "lbm_kernels.h"
 
 namespace lbm {
@@ -45,20 +46,6 @@ __device__ double du_fd(const ReadoutParams& p, int x, int y, int dx, int dy, in
     else
         ghost = 2.0 * u0 - u1;
     return (k == 0) ? (u1 - ghost) : (ghost - u1);
-}
-
-// a / j for i = 1 / j (rounded to nearest): Markstein's correction of the
-// quotient a i by its residual, which rounds to nearest as the division does,
-// in 3 operations.  A zero is a i itself; infinities, NaN and what lies near
-// the ends of the exponents take the division.
-__device__ __forceinline__ double over(double a, double j, double i) {
-    const double q = a * i;
-    auto middle = [](double v) {  // 2^-500 < |v| < 2^500
-        return (unsigned(__double2hiint(v)) & 0x7fffffffu) - 0x20b00000u < 0x3e800000u;
-    };
-    const bool zero = ((unsigned(__double2hiint(a)) & 0x7fffffffu) | unsigned(__double2loint(a))) == 0;
-    if (!((middle(q) || zero) && middle(j))) return a / j;
-    return zero ? q : fma(fma(-q, j, a), i, q);
 }
 
 struct Local {

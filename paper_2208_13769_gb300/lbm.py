@@ -115,6 +115,7 @@ _SIGNATURES = {
     "lbm_batch_get_info": (C.c_int, [C.c_void_p, C.POINTER(C.c_int64), C.POINTER(C.c_int32),
                                      C.POINTER(C.c_int32)]),
     "lbm_batch_destroy": (C.c_int, [C.c_void_p]),
+    "lbm_selftest_quotients": (C.c_int, [C.c_int64, C.c_uint64, C.c_void_p, C.POINTER(C.c_double)]),
     "lbm_selftest_bounded_wait": (C.c_int, [C.c_uint32, C.c_void_p, C.POINTER(C.c_int32)]),
     "lbm_set_tuning": (C.c_int, [C.c_void_p, C.POINTER(lbm_tuning)]),
     "lbm_get_tuning": (C.c_int, [C.c_void_p, C.POINTER(lbm_tuning)]),
@@ -322,6 +323,15 @@ def lbm_selftest_bounded_wait(polls: int, stream: int = 0) -> int:
     _check(lib().lbm_selftest_bounded_wait(int(polls), C.c_void_p(stream or None), C.byref(out)),
            "lbm_selftest_bounded_wait")
     return int(out.value)
+
+
+def lbm_selftest_quotients(count: int, seed: int, stream: int = 0):
+    """(largest error of the kernels' FP64 reciprocal in units in the last
+    place, quotients of the read-out that differ from the division's)."""
+    out = (C.c_double * 2)()
+    _check(lib().lbm_selftest_quotients(int(count), int(seed), C.c_void_p(stream or None), out),
+           "lbm_selftest_quotients")
+    return float(out[0]), int(out[1])
 
 
 def lbm_set_hole(ctx, hole, traction=None):
