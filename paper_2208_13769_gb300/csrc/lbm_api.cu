@@ -19,7 +19,7 @@ using namespace lbm;
 
 namespace {
 
-constexpr int kSegMax = 144;  // widest row segment the interior kernel copies in bulk (elements)
+constexpr int kRowPad = 160;  // columns of a plane's row beyond its kPadCols and nodes, at least
 
 size_t elem_size_storage(int fmt) {
     switch (fmt) {
@@ -795,11 +795,11 @@ lbm_status lbm_create(const lbm_desc* d, lbm_ctx** out) {
         c->bc[e].times[2] = INFINITY;
     }
     // plane layout: kPadCols columns / kPadRows rows of padding on each side,
-    // pitch a multiple of 64 elements covering the widest bulk-copied row
-    // segment of the interior kernel (a strip starting as far right as
-    // column nx - 1 reads a segment of up to kSegMax elements from 8 columns
-    // left of it)
-    const int64_t need = kPadCols + int64_t(d->nx) + kSegMax + 16;
+    // pitch a multiple of 64 elements.  (The kernels need 3 columns after the
+    // nodes, and what a tensor copy reads beyond the pitch is zeros; saved states
+    // hold whole planes and are taken back by contexts of the same pitch, so the
+    // wider padding stays.)
+    const int64_t need = kPadCols + int64_t(d->nx) + kRowPad;
     c->pitch = (need + 63) / 64 * 64;
     c->plane = c->pitch * (int64_t(d->ny) + 2 * kPadRows);
     if (c->plane > 0x7fffffffLL) {  // the interior kernel indexes a plane with 32-bit offsets

@@ -257,12 +257,7 @@ enum CarryLayout : int {
 // keeps o * sizeof(T) below 2^32).
 template <class T>
 __device__ __forceinline__ T* elem(T* base, uint32_t o) {
-    using B = typename std::conditional<std::is_const<T>::value, const char, char>::type;
-    return reinterpret_cast<T*>(reinterpret_cast<B*>(base) + o * uint32_t(sizeof(T)));
-}
-template <class T>
-__device__ __forceinline__ T* elem(T* base, int64_t o) {
-    return base + o;
+    return reinterpret_cast<T*>(reinterpret_cast<char*>(base) + o * uint32_t(sizeof(T)));
 }
 
 template <class T>
@@ -270,29 +265,24 @@ struct UPlain {  // u kept in T itself (FP64 or FP32)
     static constexpr int layout = kCarryOne;
     T v;
     // a component's plane
-    template <class P>
-    struct ViewT {
-        P* w;
-        __device__ __forceinline__ ViewT shifted(int64_t o) const { return ViewT{w + o}; }
+    struct View {
+        T* w;
+        __device__ __forceinline__ View shifted(int64_t o) const { return View{w + o}; }
     };
-    using View = ViewT<T>;
-    using CView = ViewT<const T>;
+    struct CView {
+        const T* w;
+    };
     __device__ __forceinline__ static View view(void* a, int comp, int64_t plane) {
         return View{static_cast<T*>(a) + comp * plane};
     }
     __device__ __forceinline__ static CView cview(const void* a, int comp, int64_t plane) {
         return CView{static_cast<const T*>(a) + comp * plane};
     }
-    // the stored words as loaded (decode() turns them into the value; a
-    // prefetch keeps them raw so that nothing waits for the load early)
+    // the stored words, which decode() turns into the value
     using Raw = UPlain;
-    template <class O>
-    __device__ __forceinline__ static Raw load_raw(const CView& c, O o) {
-        return UPlain{*elem(c.w, o)};
-    }
     __device__ __forceinline__ static UPlain decode(const Raw& r, const StepParams&) { return r; }
     __device__ __forceinline__ static UPlain load(const CView& c, int64_t o, const StepParams& p) {
-        return decode(load_raw(c, o), p);
+        return decode(Raw{c.w[o]}, p);
     }
     template <class Put>
     __device__ __forceinline__ static void store(const UPlain& x, const UPlain& y, const View& cx, const View& cy,
@@ -332,7 +322,6 @@ struct UPair {
     struct CView {
         const float* hi;
         const Lo* lo;
-        __device__ __forceinline__ CView shifted(int64_t o) const { return CView{hi + o, lo + o}; }
     };
     // first float of component comp: after 2 planes of floats per component,
     // or after 1.5 (a multiple of 32 floats: plane is a multiple of 64)
@@ -351,10 +340,6 @@ struct UPair {
         float hi;
         Lo lo;
     };
-    template <class O>
-    __device__ __forceinline__ static Raw load_raw(const CView& c, O o) {
-        return Raw{*elem(c.hi, o), *elem(c.lo, o)};
-    }
     __device__ __forceinline__ static UPair decode(const Raw& r, const StepParams& p) {
         if constexpr (LO16)
             return UPair{r.hi, __fmul_rn(__half2float(r.lo), p.lo_scale[1])};
@@ -362,7 +347,7 @@ struct UPair {
             return UPair{r.hi, r.lo};
     }
     __device__ __forceinline__ static UPair load(const CView& c, int64_t o, const StepParams& p) {
-        return decode(load_raw(c, o), p);
+        return decode(Raw{c.hi[o], c.lo[o]}, p);
     }
     __device__ __forceinline__ Lo lo_word(const StepParams& p) const {
         if constexpr (LO16) {

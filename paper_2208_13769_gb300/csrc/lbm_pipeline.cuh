@@ -63,9 +63,6 @@ __device__ __forceinline__ void tensor_load(uint32_t dst, const void* map, int x
         "l"(map), "r"(x), "r"(row), "r"(plane), "r"(bar)
         : "memory");
 }
-__device__ __forceinline__ void prefetch_tensor_map(const void* map) {
-    asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
-}
 // A tensor map that the host wrote to global memory, before this thread's
 // first copy by it.
 __device__ __forceinline__ void acquire_tensor_map(const void* map) {
