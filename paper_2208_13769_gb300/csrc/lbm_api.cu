@@ -458,10 +458,13 @@ static cudaError_t build_plan(lbm_ctx* c) {
         c->n_items = int(nitems);
     }
     c->has_interior = c->n_irect > 0;  // a hole may leave the bands only
-    for (int q = 0; q < 2 && c->has_interior; ++q) {
+    // (of a body without an interior too, whose batches run one)
+    c->maps_ok = true;
+    for (int q = 0; q < 2; ++q) {
         cudaError_t e = interior_maps(c->fmt, c->scheme == LBM_SCHEME_EXTRAPOLATED, c->f[q], c->a[q], c->s[q], c->pitch,
                                       c->plane, c->ny, &c->maps[q]);
-        if (e != cudaSuccess) return e;
+        if (e != cudaSuccess && c->has_interior) return e;
+        c->maps_ok = c->maps_ok && e == cudaSuccess;
     }
     // edge tiles beside an interior: CTAs of an interior tile's size, each in
     // the place of one, for the many band tiles of seams and holes beside short
@@ -502,30 +505,33 @@ static cudaError_t build_plan(lbm_ctx* c) {
     }
     StepParams hp[2] = {make_params(c, 0), make_params(c, 1)};
     // one place and one copy for the lists and the parameters
-    const void* part[4] = {items.get(), h.get(), hp, himg.get()};
-    const size_t bytes[4] = {sizeof(InteriorItem) * size_t(c->n_items), sizeof(EdgeTile) * size_t(ni), sizeof(hp),
-                             sizeof(ImageTile) * size_t(nimg)};
-    size_t at[5] = {0};
-    for (int k = 0; k < 4; ++k) at[k + 1] = at[k] + (bytes[k] + 255) / 256 * 256;
-    std::unique_ptr<unsigned char[]> host(new (std::nothrow) unsigned char[at[4]]);
+    constexpr int kParts = 5;
+    const void* part[kParts] = {items.get(), h.get(), hp, himg.get(), c->maps};
+    const size_t bytes[kParts] = {sizeof(InteriorItem) * size_t(c->n_items), sizeof(EdgeTile) * size_t(ni), sizeof(hp),
+                                  sizeof(ImageTile) * size_t(nimg), sizeof(c->maps)};
+    size_t at[kParts + 1] = {0};
+    for (int k = 0; k < kParts; ++k) at[k + 1] = at[k] + (bytes[k] + 255) / 256 * 256;
+    const size_t all = at[kParts];
+    std::unique_ptr<unsigned char[]> host(new (std::nothrow) unsigned char[all]);
     if (!host) return cudaErrorMemoryAllocation;
-    for (int k = 0; k < 4; ++k)
+    for (int k = 0; k < kParts; ++k)
         if (bytes[k] > 0) memcpy(host.get() + at[k], part[k], bytes[k]);
     cudaFree(c->plan);  // of an attempt that failed
     c->plan = nullptr;
     unsigned char* to = c->plan_room;
     cudaError_t e = cudaSuccess;
-    if (at[4] > c->plan_room_bytes) {
-        e = cudaMalloc(&c->plan, at[4]);
+    if (all > c->plan_room_bytes) {
+        e = cudaMalloc(&c->plan, all);
         to = c->plan;
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(to, host.get(), at[4], cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(to, host.get(), all, cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);  // the host's copy is freed
     if (e != cudaSuccess) return e;
     c->ditems = reinterpret_cast<InteriorItem*>(to + at[0]);
     c->dtiles = reinterpret_cast<EdgeTile*>(to + at[1]);
     c->dparams = reinterpret_cast<StepParams*>(to + at[2]);
     c->dimg = reinterpret_cast<ImageTile*>(to + at[3]);
+    c->dmaps = reinterpret_cast<InteriorMaps*>(to + at[4]);
     c->n_img = nimg;
     c->n_etiles = n;
     c->n_itiles = hole ? ni : 0;

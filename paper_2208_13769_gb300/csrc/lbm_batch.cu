@@ -44,7 +44,7 @@ struct lbm_batch {
     int fmt = 0;
     int n_entries = 0;           // parameter-table entries per parity
     StepParams* dtab = nullptr;  // [2][n_entries]: entry q * n_entries + e at parity base_parity ^ q
-    InteriorMaps* dmaps = nullptr;     // [2][n_entries]: the entries' tensor maps
+    InteriorMaps* dmaps = nullptr;  // [2][n_entries]: the entries' tensor maps, copied from the members
     InteriorItem* ditems = nullptr;  // interior tiles, longest first
     EdgeTile* dtiles = nullptr;   // edge tiles of every member
     ImageTile* dimg = nullptr;    // seam images of the members with a periodic axis
@@ -310,7 +310,7 @@ lbm_status lbm_batch_create_tuned(lbm_ctx* const* members, int32_t n, void* cuda
     const double one = all_rows / (double(sms) * std::max(1, resident));
     cudaError_t e_maps = cudaSuccess;
     std::vector<StepParams> tab;
-    std::vector<InteriorMaps> maps;
+    std::vector<const InteriorMaps*> maps;  // on the device, in the members' plans
     std::vector<EdgeTile> tiles;
     std::vector<ImageTile> imgs;
     std::vector<InteriorItem> items;
@@ -356,7 +356,8 @@ lbm_status lbm_batch_create_tuned(lbm_ctx* const* members, int32_t n, void* cuda
             const size_t k = e % ent.size();
             const lbm_ctx* c = b->m[size_t(owner[k])];
             const int par = b->base_parity[size_t(owner[k])] ^ int(e / ent.size());
-            if (e_maps == cudaSuccess) e_maps = interior_maps(b->fmt, false, c->f[par], c->a[par], c->s[par], c->pitch, c->plane, c->ny, &maps[e]);
+            maps[e] = c->dmaps + par;
+            if (!c->maps_ok) e_maps = cudaErrorNotSupported;
         }
         for (size_t e = 0; e < ent.size(); ++e) {
             tab[e] = ent[e];
@@ -411,9 +412,14 @@ lbm_status lbm_batch_create_tuned(lbm_ctx* const* members, int32_t n, void* cuda
     b->n_img = int(imgs.size());
     if (e == cudaSuccess) e = e_maps;
     if (e == cudaSuccess) e = cudaMalloc(&b->dtab, sizeof(StepParams) * tab.size());
-    if (e == cudaSuccess) e = cudaMalloc(&b->dmaps, sizeof(InteriorMaps) * maps.size());
+    // (the list of the members' maps after the table that they are copied to)
+    if (e == cudaSuccess) e = cudaMalloc(&b->dmaps, (sizeof(InteriorMaps) + sizeof(maps[0])) * maps.size());
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(b->dmaps, maps.data(), sizeof(InteriorMaps) * maps.size(), cudaMemcpyHostToDevice, b->stream);
+        e = cudaMemcpyAsync(b->dmaps + maps.size(), maps.data(), sizeof(maps[0]) * maps.size(), cudaMemcpyHostToDevice,
+                            b->stream);
+    if (e == cudaSuccess)
+        e = gather_interior_maps(reinterpret_cast<const InteriorMaps* const*>(b->dmaps + maps.size()), b->dmaps,
+                                 int(maps.size()), b->stream);
     if (e == cudaSuccess) e = cudaMalloc(&b->dflagptr, sizeof(int32_t*) * size_t(n));
     if (e == cudaSuccess) e = cudaMalloc(&b->dflagval, sizeof(int32_t) * size_t(n));
     std::vector<int32_t*> flagptr;

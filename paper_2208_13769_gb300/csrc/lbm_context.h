@@ -99,8 +99,8 @@ struct lbm_ctx {
     int n_irect = 0;
     int irect[4][4];
     int i_chunk[4], i_strip_x0[4], i_strip_w[4];
-    // device: ditems, dtiles, dparams and dimg lie in the arena's room for them,
-    // or, where they need more, in an allocation of their own
+    // device: ditems, dtiles, dparams, dimg and dmaps lie in the arena's room for
+    // them, or, where they need more, in an allocation of their own
     unsigned char *plan_room = nullptr, *plan = nullptr;
     size_t plan_room_bytes = 0;
     lbm::InteriorItem* ditems = nullptr;  // device: the interior tiles
@@ -112,7 +112,9 @@ struct lbm_ctx {
     int nband = 0;
     int brect[12][4];
     lbm::StepParams* dparams = nullptr;  // device: make_params(parity 0), make_params(parity 1)
-    lbm::InteriorMaps maps[2];                // the interior's copies, source state of parity 0 and 1
+    lbm::InteriorMaps maps[2];           // the interior's copies, source state of parity 0 and 1
+    lbm::InteriorMaps* dmaps = nullptr;  // device: maps, for the batches that the body joins
+    bool maps_ok = false;
     lbm::EdgeTile* dtiles = nullptr;     // device: tiles of the edge bands
     int n_etiles = 0;
     lbm::EdgeShape edge_shape = lbm::kEdgeWide;

@@ -818,6 +818,26 @@ cudaError_t interior_maps(int fmt, bool xj, const void* f, const void* a, const 
     return ok ? cudaSuccess : cudaErrorNotSupported;
 }
 
+namespace {
+
+constexpr int kMapWords = int(sizeof(InteriorMaps) / sizeof(int4));
+
+__global__ void gather_maps(const InteriorMaps* const* from, InteriorMaps* to) {
+    reinterpret_cast<int4*>(to + blockIdx.x)[threadIdx.x] =
+        reinterpret_cast<const int4*>(from[blockIdx.x])[threadIdx.x];
+    release_tensor_maps();
+}
+
+}  // namespace
+
+// (Encoded and uploaded by the host for each batch, the maps of 256 members took
+// 140 us of the 454 in which it was made; read where the members hold them, by a
+// list, small batches' steps took up to 4 % longer.)
+cudaError_t gather_interior_maps(const InteriorMaps* const* from, InteriorMaps* to, int n, cudaStream_t s) {
+    gather_maps<<<unsigned(n), kMapWords, 0, s>>>(from, to);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_interior(int fmt, const StepParams& p0, const InteriorRects& R, const InteriorMaps& maps, cudaStream_t s,
                             bool fields) {
     StepParams p = p0;

@@ -79,6 +79,9 @@ struct alignas(128) InteriorMaps {
 // The maps of the state (f, a, s); xj: of the extrapolated scheme.
 cudaError_t interior_maps(int fmt, bool xj, const void* f, const void* a, const void* s, int64_t pitch, int64_t plane,
                           int ny, InteriorMaps* out);
+// Copies n maps on the device, to[k] = *from[k] (device lists), for the interior
+// launches after it: a batch's table of its members' maps.
+cudaError_t gather_interior_maps(const InteriorMaps* const* from, InteriorMaps* to, int n, cudaStream_t s);
 // The most rows an interior tile of this format may have at this pitch.
 inline int interior_max_rows(int fmt, int64_t pitch) {
     return interior_max_rows(pitch, fmt == kFmtF64 ? 8 : 4, kInteriorThreads);
@@ -92,7 +95,7 @@ cudaError_t launch_interior(int fmt, const StepParams& p, const InteriorRects& R
 // (a member's rectangle, with its strip grid).
 struct BatchInteriorLaunch {
     const StepParams* params;  // device table, indexed by InteriorItem::inst
-    const InteriorMaps* maps;       // device table of the entries' tensor maps, indexed as params
+    const InteriorMaps* maps;  // device table of the entries' tensor maps, indexed as params
     const InteriorItem* items; // device list of interior tiles, one per CTA
     int32_t fields;            // also write u, v, r to params.fields
     int32_t nitems;            // tiles in the list

@@ -63,8 +63,13 @@ __device__ __forceinline__ void tensor_load(uint32_t dst, const void* map, int x
         "l"(map), "r"(x), "r"(row), "r"(plane), "r"(bar)
         : "memory");
 }
-// A tensor map that the host wrote to global memory, before this thread's
-// first copy by it.
+// This thread's stores to tensor maps in global memory, for the kernels after
+// this one that acquire them.
+__device__ __forceinline__ void release_tensor_maps() {
+    asm volatile("fence.proxy.tensormap::generic.release.sys;" ::: "memory");
+}
+// A tensor map that the host or an earlier kernel wrote to global memory, before
+// this thread's first copy by it.
 __device__ __forceinline__ void acquire_tensor_map(const void* map) {
     asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(map) : "memory");
 }
