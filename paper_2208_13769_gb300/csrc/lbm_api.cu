@@ -972,7 +972,7 @@ lbm_status lbm_step(lbm_ctx* c, int64_t nsteps) {
     st = ctx_ensure_initialized(c);
     if (st != LBM_OK || nsteps == 0) return st;
     int64_t left = nsteps;
-    // plain launches until the variant is warm (attributes set outside capture)
+    // a plain launch first: the kernels are loaded outside a capture
     if (!c->variant_warm && left > 1) {
         st = launch(c, 0, false);
         if (st != LBM_OK) return st;

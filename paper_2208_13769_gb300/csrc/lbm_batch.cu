@@ -153,21 +153,28 @@ lbm_status batch_graph(lbm_batch* b, int q, cudaGraphExec_t* out) {
 // most rows go to chunks of about a wave's rows and the rest to shorter ones,
 // which even out the end of the launch; fewer than 12 rows a wave are split as
 // a single short body's, and short members of a batch of many, whose tiles even
-// out the end by themselves, into chunks of about 32 rows.  32 bodies of 64 to
-// 1024 nodes a side in FP32 (93 rows) 247 us a step with chunks of 32 rows and
-// 243 so, 12 of 128 to 2048 in FP16 (185) 367 and 347, 20 of 64 to 700 in FP16
-// (35) 110 and 92, 6 of 64 to 400 in FP32 (5) 36 and 21; 256 bodies of 32 to 128
-// nodes a side (22 rows) 122 us a step in FP32 lo16 in levels and 115 in chunks
-// of 32 rows, FP16 101 and 95; 128 of them (11 rows) in FP16 57 in such chunks
-// and 49 in short ones.
-ChunkLevels batch_levels(bool f64, int h, int tune_chunk, double one, int64_t all, int sms) {
+// out the end by themselves, into chunks of about 32 rows.  Where a wave has more
+// than 88 rows in 4-byte storage, or 240 in 16-bit storage, the chunks are as of
+// that many: the tiles in work at a time then lie closer together, as in a long
+// body (256 bodies of 64 to 1024 nodes a side, 790 rows a wave: FP32 lo16 1904 us
+// a step and 1740 so, 1732 to 1755 with 72 to 128; FP16 1502 and 1445, 1444 to
+// 1475 with 300 to 104).  FP64, bound by its operations, gains nothing by it.  32
+// bodies of 64 to 1024 nodes a side in FP32 (93 rows) 247 us a step with chunks
+// of 32 rows and 243 so, 12 of 128 to 2048 in FP16 (185) 367 and 344, 20 of 64 to
+// 700 in FP16 (35) 110 and 92, 6 of 64 to 400 in FP32 (5) 36 and 21; 256 bodies
+// of 32 to 128 nodes a side (22 rows) 122 us a step in FP32 lo16 in levels and
+// 115 in chunks of 32 rows, FP16 101 and 95; 128 of them (11 rows) in FP16 57 in
+// such chunks and 49 in short ones.
+ChunkLevels batch_levels(int fmt, int h, int tune_chunk, double one, int64_t all, int sms) {
+    const bool f64 = fmt == kFmtF64, half = fmt == kFmtF16 || fmt == kFmtBF16;
     int rows = tune_chunk;
     if (rows == 0 && one < 12) rows = short_rows(1, int(all), sms);
     if (rows == 0 && !f64 && h <= 128 && one < 43) rows = (h + (h + 31) / 32 - 1) / ((h + 31) / 32);
     if (rows > 0) return equal_chunks(h, rows);
     ChunkLevels L;
     memset(&L, 0, sizeof(L));
-    auto part = [&](double f) { return std::max(8, int(std::min(f * one, double(1 << 20)))); };
+    const double wave = std::min(one, f64 ? double(1 << 20) : (half ? 240.0 : 88.0));
+    auto part = [&](double f) { return std::max(8, int(f * wave)); };
     L.rows[0] = std::min(part(0.75), h);
     L.rows[1] = part(0.5);
     L.rows[2] = part(1.0 / 3);
@@ -340,7 +347,7 @@ lbm_status lbm_batch_create_tuned(lbm_ctx* const* members, int32_t n, void* cuda
                     const int e = int(ent.size()) - 1;
                     const int h = p.rect[3] - p.rect[2];
                     const ChunkLevels lev =
-                        bounded_chunks(batch_levels(f64, h, b->chunk_rows, one, int64_t(all_rows), sms), h,
+                        bounded_chunks(batch_levels(b->fmt, h, b->chunk_rows, one, int64_t(all_rows), sms), h,
                                        interior_max_rows(b->fmt, c->pitch));
                     const int64_t cnt = interior_items(mri.irect[q], e, ns, lev, nullptr, 0);
                     const size_t at = items.size();
@@ -596,8 +603,7 @@ lbm_status lbm_batch_autotune(lbm_ctx* const* members, int32_t n, int64_t steps,
             status = lbm_set_hole(scratch[size_t(i)], c->hole, c->hole_T);
     }
     // candidates: ring depth x rows per interior tile (0: the default) on the
-    // format's default strip grid, then the other two strip grids at the
-    // best of those
+    // default strip grid, then the other two strip grids at the best of those
     const int rings[3] = {4, 5, 6};
     const int chunks[5] = {0, 32, 64, 128, 256};
     const int al0 = kBatchAligned;
