@@ -163,8 +163,8 @@ LBM_API lbm_status lbm_set_hole(lbm_ctx* ctx, const int32_t hole[4], const doubl
  * edge tiles alone for a small body), plus, where the interior kernel runs
  * across a periodic seam (lbm_tuning.plan 2), a launch copying the nodes
  * next to the seam into their periodic images.  The observable fields (u,
- * v, r) are captured at the last step.  Asynchronous.  Errors: LBM_E_STATE (material or boundaries unset),
- * LBM_E_INVALID (nsteps < 0), LBM_E_CUDA. */
+ * v, r) are captured at the last step.  Asynchronous.  Errors: LBM_E_STATE
+ * (material or boundaries unset), LBM_E_INVALID (nsteps < 0), LBM_E_CUDA. */
 LBM_API lbm_status lbm_step(lbm_ctx* ctx, int64_t nsteps);
 
 /* Measurement aid (no counterpart in the paper).  Advances `nsteps` time
@@ -200,22 +200,25 @@ LBM_API lbm_status lbm_profile_interior(lbm_ctx* ctx, int64_t nlaunches, double 
  * the work is split, never the result: the interior settings give
  * bit-identical fields; the plan decides which kernel advances the nodes
  * more than two nodes from an edge, whose results agree to rounding).  The
- * interior kernel's row pipeline has a latency floor per launch (about 13 us
- * in FP32 with its shortest 8-row tiles) that small bodies do not fill, while edge tiles
- * take one memory round trip each: below the size thresholds of plan 0 the
- * edge tiles alone are faster (2 to 5 times up to 256 x 256). */
+ * interior kernel's row pipeline has a latency floor per launch that small
+ * bodies do not fill (about 7 us in FP32 and 45 in FP64), while
+ * edge tiles take one memory round trip each: below the size thresholds of plan
+ * 0 the edge tiles alone are faster (64 x 64 in 4.4 us in FP32 and
+ * 12 in FP64; the two meet at about 300 x 300 and 550 x 550). */
 typedef struct {
     int32_t ring_slots; /* rows of the interior kernel's pipeline in flight or in work, 4..8; 0:
-                           default (4) */
-    int32_t chunk_rows; /* rows per CTA, >= 8; 0: one wave of CTAs over the SMs, with shorter
-                           chunks after it on a large body; on a body of less than about 10
-                           rows each the 4 to 18 rows that take least time (default) */
+                           default (4; 5 for the extrapolated scheme with an FP32 pair carry
+                           where a CTA has 12 rows or more) */
+    int32_t chunk_rows; /* rows per CTA, >= 8; 0: by the rows that one wave of CTAs over the SMs
+                           would give each: up to 10, the 4 to 18 that take least time; then
+                           about a wave, from 20 to 48 rows on (by format) with shorter chunks
+                           after it, and chunks of 18 rows on the largest bodies (default) */
     int32_t aligned;    /* 1: the fewest strips of equal width on 32-byte sector boundaries (at
                            most 120 columns; 112 for 16-bit storage); 2: the same on 16-byte
                            boundaries (at most 124 columns; 120 for 16-bit storage);
-                           0: 124-column strips; -1: default (0 for 16-bit storage; otherwise
-                           1 in a batch, and for single bodies in 4-byte storage with 16
-                           rows or more per CTA of a wave) */
+                           0: 124-column strips; -1: default (2 in a batch; 1 for a single body
+                           in 4-byte storage with 16 rows or more per CTA, or with the ring of
+                           5; else 0) */
     int32_t plan;       /* 0: by size (default): a body of fewer than 2^17 nodes (3 x 2^17 in FP64)
                            runs as small tiles of the edge kernel only, a larger one as the
                            interior kernel plus the edge bands (a 3-node band each side of a
@@ -321,7 +324,8 @@ LBM_API lbm_status lbm_destroy(lbm_ctx* ctx);
  * to several independent bodies at once: each time step is one launch over
  * the interior tiles of every member and one over their edge tiles, so small
  * or uneven bodies share the GPU instead of each paying its own launches;
- * chunks of 64 steps replay as one CUDA graph.  The batch advances every
+ * chunks of 64 steps replay as one CUDA graph (not on a stream that the caller
+ * is capturing, where every step is recorded).  The batch advances every
  * member with the interior kernel where the body allows it (plan 2 of
  * lbm_tuning, unless the member asked for plan 1), through the same
  * arithmetic as a single body: results are bit-identical to lbm_step on a
@@ -349,7 +353,8 @@ LBM_API lbm_status lbm_batch_create(lbm_ctx* const* members, int32_t n, void* cu
  * counterpart in the paper; it changes the split of the work, never the
  * results): tuning->ring_slots, rows of the pipeline in flight or in work
  * (4..8; 0: 4), tuning->chunk_rows, rows per interior tile (>= 8; 0: about a
- * wave's rows for most of them, then shorter tiles), and tuning->aligned, the
+ * wave's rows for most of them, then shorter tiles; short tiles in a small
+ * batch, about 32 rows for the short members of a batch of many), and tuning->aligned, the
  * strip grid of each member (as for lbm_set_tuning; -1: 2); plan is ignored
  * (each member keeps its own).  NULL: the defaults.
  * Errors as lbm_batch_create, and LBM_E_INVALID for a tuning out of range. */
@@ -361,8 +366,7 @@ LBM_API lbm_status lbm_batch_create_tuned(lbm_ctx* const* members, int32_t n, vo
  * `members` (zero initial fields, lambda = mu = 0.3), times `steps`
  * graph-replayed steps of a scratch batch of them for each candidate
  * decomposition (ring 4, 5, 6 x rows per tile default, 32, 64, 128, 256 on
- * the format's default strip grid, then the other two strip grids at the
- * best of those) on a stream of its own, and returns the fastest in *best
+ * the default strip grid, then the other two strip grids at the best of those) on a stream of its own, and returns the fastest in *best
  * (its time per step in *best_ms, may be NULL).  The time of a step does not depend on the
  * field values, so the choice holds for the members.  The members are not
  * touched.  Holds as much device memory as the members, for the call.
